@@ -190,7 +190,9 @@ void release(ssm_plan_s* pl) {
   dfree(pl->Mq32);
   dfree(pl->Mhi);
   dfree(pl->Mlo);
-  dfree(pl->Gq32);
+  dfree(pl->Xs);
+  dfree(pl->xexp);
+  dfree(pl->vexp);
   for (int i = 0; i < 2; ++i) {
     dfree(pl->Z[i]);
     dfree(pl->Dl[i]);
@@ -208,7 +210,6 @@ void release(ssm_plan_s* pl) {
   dfree(pl->B_multi);
   dfree(pl->tprob);
   dfree(pl->ttable);
-  dfree(pl->C32);
   dfree(pl->S);
   dfree(pl->H);
   dfree(pl->Wf);
@@ -365,12 +366,19 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
       SSM_TRY(palloc(pl, &pl->V2l, (size_t)pl->R * pl->lrtc_qs, s));
     }
   } else {
-    SSM_TRY(palloc(pl, &pl->Gq32, (size_t)Q * n, s));
     SSM_TRY(palloc(pl, &pl->Mq32, (size_t)Q * pl->Qp, s));
     if (p.precision == SSM_BF16X3) {
       SSM_TRY(palloc(pl, &pl->Mhi, (size_t)Q * pl->Qp, s));
       SSM_TRY(palloc(pl, &pl->Mlo, (size_t)Q * pl->Qp, s));
     }
+  }
+  {
+    const int xr = p.form == SSM_FORM_LOWRANK ? pl->r : Q;
+    int xrp, xpp;
+    exact_shape(xr, P, &xrp, &xpp);
+    SSM_TRY(palloc(pl, &pl->Xs, (size_t)exact_elems(xr, P), s));
+    SSM_TRY(palloc(pl, &pl->xexp, (size_t)xrp, s));
+    SSM_TRY(palloc(pl, &pl->vexp, (size_t)pl->g.ld, s));
   }
   st = factors_fp64(pl, E, s);
   cudaFreeAsync(A, s);
@@ -395,7 +403,6 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
     AdmmState& a = pl->adm;
     for (float** v : {&a.x, &a.y, &a.z, &a.dx, &a.dy, &a.dz, &a.f, &a.w, &a.r, &a.t})
       SSM_TRY(palloc(pl, v, QN, s));
-    SSM_TRY(palloc(pl, &pl->C32, (size_t)n * pl->g.ld, s));
     SSM_TRY(palloc(pl, &pl->H, QN, s));
     SSM_TRY(palloc(pl, &pl->Acc, QN, s));
     std::vector<std::pair<float**, std::vector<float>>> tables;
@@ -421,7 +428,6 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
     const size_t pf = (size_t)lowrank_state_floats(pl, pl->lr_grid);
     for (int i = 0; i < 2; ++i) SSM_TRY(palloc(pl, &pl->U[i], pf, s));
   } else {
-    SSM_TRY(palloc(pl, &pl->C32, (size_t)n * pl->g.ld, s));
     SSM_TRY(palloc(pl, &pl->H, QN, s));
     if (p.precision == SSM_FP32) {
       SSM_TRY(palloc(pl, &pl->Wf, QN, s));
@@ -665,16 +671,22 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
     add(4, 2 * (int64_t)t.R);                 // coefA, coefW
     if (p.precision == SSM_TF32X3) add(4, 2 * (Q + t.lrtc_qs) * t.R);  // V1h/l, V2h/l
   } else {
-    add(4, Q * n);                            // Gq32
     add(4, Q * t.Qp);                         // Mq32
     if (p.precision == SSM_BF16X3) add(2, 2 * Q * t.Qp);  // Mhi, Mlo
+  }
+  {
+    const int xr = p.form == SSM_FORM_LOWRANK ? t.r : p.Q;
+    int xrp, xpp;
+    exact_shape(xr, p.P, &xrp, &xpp);
+    add(2, exact_elems(xr, p.P));             // Xs
+    add(4, xrp);                              // xexp
+    add(4, ld);                               // vexp
   }
   const int64_t QN = Q * ld;
   if (p.form != SSM_FORM_ADMM) add(4, 4 * QN);  // Z[2], Dl[2]
   int64_t maxparts = 1;
   if (p.form == SSM_FORM_ADMM) {
     add(4, 10 * QN);                          // x, y, z, d_x, d_y, d_z, f, w, r, t
-    add(4, n * ld);                           // C32
     add(4, 2 * QN);                           // H, Acc
     const int64_t dd[3] = {t.g.nx, t.g.ny, t.g.nz};
     for (int d = 0; d < 3; ++d)
@@ -693,7 +705,6 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
     }
     add(4, 2 * lowrank_state_floats(&t, t.lr_grid));  // U[2]
   } else {
-    add(4, n * ld);                           // C32
     add(4, QN);                               // H
     if (p.precision == SSM_FP32) {
       add(4, 2 * QN);                         // Wf, Acc
@@ -711,7 +722,7 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
   if (staging) add(4, (P + Q) * ld);          // Mstage, Fstage
   *persistent = b;
   int64_t tmp = 8 * (3 * n * n + 2) + 4 * n + 8 * P * Q;  // A, E, scratch, perm, K_r
-  if (p.form != SSM_FORM_LOWRANK) tmp += 8 * (n + Q * Q);   // inverse weights, FP64 inverse
+  if (p.form != SSM_FORM_LOWRANK) tmp += 8 * (2 * n + Q * (Q + P));   // weights, FP64 inverse and projection operand
   *peak = b + tmp;
   return SSM_OK;
 }
@@ -917,7 +928,7 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
     return SSM_EINVAL;
   }
   pl->has_state = false;   // set again when this solve completes
-  // step 4: projections of the data on the singular vectors (FP64 accumulation)
+  // step 4: projections of the data on the singular vectors (accurate to an FP64 accumulation)
   if (pl->ndict > 0) {
     // each voxel's projections on its own dictionary's factors (zero past its rank)
     SSM_TRY(table_project(pl->B_multi, pl->P, pl->R, pl->labels, M, ldm, pl->g.N, pl->S,
@@ -926,7 +937,7 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
       SSM_CUDA(cudaMemsetAsync(
           pl->U[0], 0, sizeof(float) * (size_t)lowrank_state_floats(pl, pl->lr_grid), s));
   } else if (p.form == SSM_FORM_LOWRANK) {
-    SSM_TRY(project_data(pl, M, ldm, pl->r, s));
+    SSM_TRY(project_data(pl, M, ldm, s));
     if (pl->R > pl->r)
       SSM_CUDA(cudaMemsetAsync(pl->S + (size_t)pl->r * ld, 0,
                                sizeof(float) * (size_t)(pl->R - pl->r) * ld, s));
@@ -934,10 +945,7 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
       SSM_CUDA(cudaMemsetAsync(
           pl->U[0], 0, sizeof(float) * (size_t)lowrank_state_floats(pl, pl->lr_grid), s));
   } else {
-    SSM_TRY(project_data(pl, M, ldm, pl->n, s));
-    // h = M g = sum_i Gq_i c_i
-    SSM_TRY(sgemm(pl->Q, (int)pl->g.N, pl->n, 1.f, pl->Gq32, pl->n, pl->C32, ld, 0.f, pl->H, ld,
-                  s));
+    SSM_TRY(project_data(pl, M, ldm, s));   // h = M g
     if (pl->Wf && !resume) SSM_CUDA(cudaMemsetAsync(pl->Wf, 0, sizeof(float) * QN, s));
     if (pl->Whi[0] && !resume) {
       const size_t WN = (size_t)pl->g.ld * pl->Qp;

@@ -166,13 +166,16 @@ struct ssm_plan_s {
   float* Mq32 = nullptr;       // Q x Q  (K^T K + beta I)^{-1}, row stride Qp
   __nv_bfloat16* Mhi = nullptr;  // Q x Qp (bf16 split of Mq: hi + lo)
   __nv_bfloat16* Mlo = nullptr;
-  float* Gq32 = nullptr;       // Q x n  : h = Gq c
+  // projections of the data (ssm_exact.cu): the FP64 operand cut into BF16 slices, its
+  // row exponents, and scratch for the data's column exponents
+  __nv_bfloat16* Xs = nullptr;
+  int* xexp = nullptr;
+  int* vexp = nullptr;               // ld
   int Qp = 0;                  // padded row stride of Q x Q operands
 
   // per-voxel state (map-major, leading dimension g.ld)
   float* Z[2] = {nullptr, nullptr};  // z ping-pong            (Q x ld)
   float* Dl[2] = {nullptr, nullptr}; // dual d ping-pong       (Q x ld)
-  float* C32 = nullptr;              // projections c          (n x ld)
   float* S = nullptr;                // S_i = sigma_i u_i^T m  (R x ld)
   float* U[2] = {nullptr, nullptr};  // partial u = V^T (beta z - d) per (tile, segment)
   int64_t lr_grid = 0;               // persistent grid of the low-rank kernel
@@ -251,10 +254,20 @@ ssm_status factors_fp64(ssm_plan_s* pl, const double* E, cudaStream_t s);
 ssm_status hessian_power(ssm_plan_s* pl, const double* A, int n, cudaStream_t s);
 ssm_status form_dense_inverse(ssm_plan_s* pl, cudaStream_t s);
 ssm_status beta_weights(ssm_plan_s* pl, cudaStream_t s);
-ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, int ncomp,
-                        cudaStream_t s);
+ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, cudaStream_t s);
 ssm_status split_bf16(const float* X, int rows, int cols, int64_t ldx,
                       __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t ldo, cudaStream_t s);
+
+// out = A m to FP64 grade on the tensor cores (ssm_exact.cu): the rows of A are cut into
+// slices once (exact_slice; the operand holds exact_elems BF16 values and the padded row
+// count of exponents)
+void exact_shape(int rows, int P, int* rows_pad, int* P_pad);
+int64_t exact_elems(int rows, int P);
+ssm_status exact_slice(const double* src, int64_t sr, int64_t sp, const double* scale, int rows,
+                       int P, __nv_bfloat16* slices, int* rexp, cudaStream_t s);
+ssm_status exact_product(const __nv_bfloat16* slices, const int* rexp, int rows, int P,
+                         const float* M, int64_t ldm, int64_t N, float* out, int64_t ldo,
+                         int* vexp, int* err, cudaStream_t s);
 
 // low-rank iteration (ssm_lowrank.cu)
 // low-rank iteration k -> k+1 with state (z, per-voxel u); `check` forms the residual

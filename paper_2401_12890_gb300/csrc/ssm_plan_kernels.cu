@@ -1,9 +1,9 @@
 // Plan-stage kernels (Algorithm 2, steps 3-4): FP64 Gram matrix, parallel cyclic
 // Jacobi eigendecomposition, the singular factors of Eq. 27, the weights of Eq. 28,
-// the full-rank inverse of Eq. 26, and the data projections g_n (step 4).
+// the full-rank inverse of Eq. 26, and the operand of the data projections (step 4,
+// ssm_exact.cu).
 //
-// All of this runs once per plan (factors) or once per solve (projections) and is
-// FP64 where the paper's conditioning needs it. GB300's FP64 rate is low, so the
+// All of this runs once per plan and is FP64 where the paper's conditioning needs it. GB300's FP64 rate is low, so the
 // kernels spread FP64 work over every SM rather than one CTA.
 #include <algorithm>
 #include <cmath>
@@ -247,15 +247,6 @@ __global__ void lowrank_basis(const double* __restrict__ Kt, int Q, int n, const
   }
 }
 
-// Gq[q][i] = Kt[q][i] / (sigma_i^2 + beta)   (h = M g = sum_i Gq_i c_i)
-__global__ void gq_kernel(const double* __restrict__ Kt, int Q, int n, const double* __restrict__ sig,
-                          double beta, float* __restrict__ Gq) {
-  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)Q * n) return;
-  int i = (int)(idx % n);
-  Gq[idx] = (float)(Kt[idx] / (sig[i] * sig[i] + beta));
-}
-
 __global__ void to_f32(const double* __restrict__ X, int64_t count, float* __restrict__ Y) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < count) Y[i] = (float)X[i];
@@ -291,49 +282,6 @@ __global__ void split_bf16_kernel(const float* __restrict__ X, int rows, int col
   __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
   hi[idx] = h;
   lo[idx] = l;
-}
-
-// ---------------------------------------------------------------------------
-// data projections (Algorithm 2, step 4):  out[i][n] = scale_i * sum_p Bp[p][i] m[p][n]
-// FP64 accumulation; a block covers 128 voxels x 8 components; Bp staged in smem.
-// ---------------------------------------------------------------------------
-constexpr int PJ_VOX = 128, PJ_COMP = 8, PJ_PCH = 128;
-
-__global__ void __launch_bounds__(PJ_VOX) project_kernel(const double* __restrict__ Bp, int P, int nB,
-                                                 int ncomp, const float* __restrict__ M,
-                                                 int64_t ldm, int64_t N,
-                                                 const double* __restrict__ scale,
-                                                 float* __restrict__ out, int64_t ldo) {
-  __shared__ double bs[PJ_PCH][PJ_COMP];
-  const int64_t nv = blockIdx.x * (int64_t)PJ_VOX + threadIdx.x;
-  const int c0 = blockIdx.y * PJ_COMP;
-  double acc[PJ_COMP];
-#pragma unroll
-  for (int j = 0; j < PJ_COMP; ++j) acc[j] = 0.0;
-  for (int p0 = 0; p0 < P; p0 += PJ_PCH) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < PJ_PCH * PJ_COMP; idx += PJ_VOX) {
-      int pp = idx / PJ_COMP, j = idx % PJ_COMP;
-      int p = p0 + pp, c = c0 + j;
-      bs[pp][j] = (p < P && c < ncomp) ? Bp[(int64_t)p * nB + c] : 0.0;
-    }
-    __syncthreads();
-    if (nv < N) {
-      int pend = min(PJ_PCH, P - p0);
-      for (int pp = 0; pp < pend; ++pp) {
-        double mv = (double)M[(int64_t)(p0 + pp) * ldm + nv];
-#pragma unroll
-        for (int j = 0; j < PJ_COMP; ++j) acc[j] = fma(bs[pp][j], mv, acc[j]);
-      }
-    }
-  }
-  if (nv < N) {
-#pragma unroll
-    for (int j = 0; j < PJ_COMP; ++j) {
-      int c = c0 + j;
-      if (c < ncomp) out[(int64_t)c * ldo + nv] = (float)(scale ? acc[j] * scale[c] : acc[j]);
-    }
-  }
 }
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -437,8 +385,8 @@ ssm_status factors_fp64(ssm_plan_s* pl, const double* E, cudaStream_t s) {
 }
 
 // The beta-dependent part of the plan (the factors above do not depend on beta):
-// low-rank V_r and the weights of Eq. 28, or the dense form's h-map Gq; the dense
-// inverse itself is form_dense_inverse.
+// low-rank V_r and the weights of Eq. 28, or the full-rank forms' map from the data to
+// h = M g; the dense inverse itself is form_dense_inverse.
 ssm_status beta_weights(ssm_plan_s* pl, cudaStream_t s) {
   const int Q = pl->Q, n = pl->n;
   const double floor = pl->sigma1 * 1e-15;
@@ -448,10 +396,19 @@ ssm_status beta_weights(ssm_plan_s* pl, cudaStream_t s) {
         pl->coefW, floor);
     SSM_LAUNCHED();
     if (pl->V1h) SSM_TRY(lrtc_split_basis(pl, s));
+    SSM_TRY(exact_slice(pl->Bp64, 1, n, pl->alpha64, pl->r, pl->P, pl->Xs, pl->xexp, s));
   } else {
-    gq_kernel<<<nblk((int64_t)Q * n, 256), 256, 0, s>>>(pl->Kt64, Q, n, pl->sig64, pl->p.beta,
-                                                        pl->Gq32);
+    // A = (K^T K + beta I)^{-1} K^T = sum_i k_i b_i^T / (sigma_i^2 + beta), b_i the left
+    // factors (rows of Bp^T), in FP64
+    double *w = nullptr, *A = nullptr;
+    SSM_CUDA(cudaMallocAsync(&w, sizeof(double) * n, s));
+    SSM_CUDA(cudaMallocAsync(&A, sizeof(double) * (int64_t)Q * pl->P, s));
+    inv_weights<<<nblk(n, 256), 256, 0, s>>>(pl->sig64, n, 1, pl->p.beta, w);
     SSM_LAUNCHED();
+    SSM_TRY(dgemm(Q, pl->P, n, pl->Kt64, n, false, pl->Bp64, n, true, A, pl->P, s, w));
+    SSM_TRY(exact_slice(A, pl->P, 1, nullptr, Q, pl->P, pl->Xs, pl->xexp, s));
+    SSM_CUDA(cudaFreeAsync(A, s));
+    SSM_CUDA(cudaFreeAsync(w, s));
   }
   return SSM_OK;
 }
@@ -483,18 +440,12 @@ ssm_status split_bf16(const float* X, int rows, int cols, int64_t ldx, __nv_bflo
   return SSM_OK;
 }
 
-// c (ncomp x ld, FP32) = scale .* (Bp^T m), FP64 accumulation. The low-rank form
-// writes S (scale = alpha), the dense form writes the raw coefficients.
-ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, int ncomp,
-                        cudaStream_t s) {
+// The projections of step 4: S_i = sigma_i u_i^T m (low-rank forms) or h = M g with
+// M g = (K^T K + beta I)^{-1} K^T m (full-rank forms and Algorithm 1)
+ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, cudaStream_t s) {
   const bool lowrank = pl->p.form == SSM_FORM_LOWRANK;
-  float* out = lowrank ? pl->S : pl->C32;
-  const double* scale = lowrank ? pl->alpha64 : nullptr;
-  dim3 grid(nblk(pl->g.N, PJ_VOX), (unsigned)((ncomp + PJ_COMP - 1) / PJ_COMP));
-  project_kernel<<<grid, PJ_VOX, 0, s>>>(pl->Bp64, pl->P, pl->n, ncomp, M, ldm, pl->g.N, scale,
-                                         out, pl->g.ld);
-  SSM_LAUNCHED();
-  return SSM_OK;
+  return exact_product(pl->Xs, pl->xexp, lowrank ? pl->r : pl->Q, pl->P, M, ldm, pl->g.N,
+                       lowrank ? pl->S : pl->H, pl->g.ld, pl->vexp, pl->dev_err, s);
 }
 
 }  // namespace ssm
