@@ -214,7 +214,6 @@ void release(ssm_plan_s* pl) {
   dfree(pl->H);
   dfree(pl->Wf);
   dfree(pl->Acc);
-  dfree(pl->Res);
   dfree(pl->Mstage);
   dfree(pl->Fstage);
   dfree(pl->red);
@@ -352,8 +351,8 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
   SSM_TRY(palloc(pl, &pl->Kt64, (size_t)Q * n, s));
   SSM_TRY(palloc(pl, &pl->sig64, (size_t)n, s));
   SSM_TRY(palloc(pl, &pl->alpha64, (size_t)n, s));
-  SSM_TRY(palloc(pl, &pl->K32, (size_t)P * Q, s));
-  SSM_TRY(palloc(pl, &pl->Kr32, (size_t)P * Q, s));
+  SSM_TRY(palloc(pl, &pl->K32, (size_t)Q * round_up(P, 4), s));
+  SSM_TRY(palloc(pl, &pl->Kr32, (size_t)Q * round_up(P, 4), s));
   if (p.form == SSM_FORM_LOWRANK) {
     SSM_TRY(palloc(pl, &pl->V32, (size_t)Q * pl->R, s));
     SSM_TRY(palloc(pl, &pl->coefA, (size_t)pl->R, s));
@@ -445,7 +444,7 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
       maxparts = std::max(tc_max_partials(pl), dense_max_partials(pl));
     }
   }
-  maxparts = std::max(maxparts, (int)((pl->g.N + 255) / 256));  // objective partials
+  maxparts = std::max(maxparts, objective_partials(pl));
   pl->red_cap = maxparts;
   SSM_TRY(palloc(pl, &pl->red, (size_t)maxparts * 4, s));
   SSM_TRY(palloc(pl, &pl->red_out, 8, s));
@@ -664,8 +663,7 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
   add(8, Q * n);                              // Kt64
   add(8, n);                                  // sig64
   add(8, n);                                  // alpha64
-  add(4, P * Q);                              // K32
-  add(4, P * Q);                              // Kr32
+  add(4, 2 * Q * round_up(P, 4));             // K32, Kr32
   if (p.form == SSM_FORM_LOWRANK) {
     add(4, Q * t.R);                          // V32
     add(4, 2 * (int64_t)t.R);                 // coefA, coefW
@@ -715,7 +713,7 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
       maxparts = std::max(tc_max_partials(&t), dense_max_partials(&t));
     }
   }
-  maxparts = std::max<int64_t>(maxparts, (t.g.N + 255) / 256);
+  maxparts = std::max<int64_t>(maxparts, objective_partials(&t));
   add(8, maxparts * 4);                       // red
   add(8, 8);                                  // red_out
   add(4, 1);                                  // dev_err
@@ -1254,16 +1252,9 @@ ssm_status ssm_objective(ssm_plan_t plan, const float* M_dev, int64_t ldm, const
   }
   SSM_CUDA(cudaSetDevice(plan->device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int64_t ld = plan->g.ld;
-  if (!plan->Res) SSM_TRY(palloc(plan, &plan->Res, (size_t)plan->P * ld, s));
-  SSM_CUDA(cudaMemcpy2DAsync(plan->Res, sizeof(float) * ld, M_dev, sizeof(float) * ldm,
-                             sizeof(float) * plan->g.N, plan->P, cudaMemcpyDeviceToDevice, s));
   const float* Kd = (use_full_k || plan->p.form != SSM_FORM_LOWRANK) ? plan->K32 : plan->Kr32;
-  // Res = M - K' F
-  SSM_TRY(sgemm(plan->P, (int)plan->g.N, plan->Q, -1.f, Kd, plan->Q, F_dev, ldf, 1.f, plan->Res,
-                ld, s));
   int nparts = 0;
-  SSM_TRY(objective_terms(plan, plan->Res, plan->P, F_dev, ldf, plan->red, &nparts, s));
+  SSM_TRY(objective_terms(plan, Kd, M_dev, ldm, F_dev, ldf, plan->red, &nparts, s));
   SSM_TRY(finish_partials(plan->red, nparts, 2, plan->red_out, s));
   SSM_CUDA(cudaMemcpyAsync(plan->red_host, plan->red_out, 2 * sizeof(double),
                            cudaMemcpyDeviceToHost, s));

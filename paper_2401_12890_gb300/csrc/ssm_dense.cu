@@ -9,6 +9,8 @@
 // the z-step (Eq. 31 with the nonnegativity projection) and the dual step, and
 // writes the next w (FP32 for this form, or the BF16 hi/lo pair for the tensor-core
 // form), so one iteration is: sgemm (M w) -> dense_update.
+#include <algorithm>
+
 #include "ssm_internal.cuh"
 
 namespace ssm {
@@ -214,59 +216,256 @@ __global__ void finish_kernel(const double* __restrict__ part, int nparts, int w
   }
 }
 
-// objective pieces: sum over the residual rows of r^2, and sum over every unordered
-// neighbour pair and every map of (F_n - F_m)^2 (the forward differences)
-__global__ void __launch_bounds__(UV) objective_kernel(const float* __restrict__ Res, int P,
-                                                       const float* __restrict__ F, int64_t ldf,
-                                                       int Q, Grid g,
+// B bytes from global to shared memory, of which the first `n` are read and the rest are 0
+template <int B>
+__device__ __forceinline__ void cp_async(float* dst, const float* src, int n) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n)
+                 : "memory");
+}
+
+struct ResidualArgs {
+  int P, N, Q;
+  const float* __restrict__ Kt;       // K^T: Q x P, row stride ldk
+  int64_t ldk;
+  const float* __restrict__ F;
+  int64_t ldf;
+  const float* __restrict__ M;
+  int64_t ldm;
+  const uint8_t* __restrict__ mask;   // voxels inside the object (nullptr: every voxel)
+  double* __restrict__ partial;       // 4 doubles per CTA
+};
+
+// s + c (unevaluated) += x, exactly (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum(float& s, float& c, float x) {
+  const float t = __fadd_rn(s, x);
+  const float b = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+  s = t;
+}
+
+template <int T>
+__device__ __forceinline__ void block_partial(double d1, double d2, double d3, double* out) {
+  for (int o = 16; o > 0; o >>= 1) {
+    d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+    d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    d3 += __shfl_xor_sync(0xffffffffu, d3, o);
+  }
+  __shared__ double red[T / 32][3];
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[w][0] = d1;
+    red[w][1] = d2;
+    red[w][2] = d3;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int k = 0; k < T / 32; ++k) t += red[k][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+}
+
+// sum over a chunk of maps and RT voxels of (F_n - F_m)^2, m the forward neighbours: a
+// float-float sum per thread (its error, 2^-48 relative, is far below that of the FP32
+// squares; an FP64 add per element would take 77 us of the 41 M elements of the 128 x 128
+// slice at this chip's FP64 rate)
+constexpr int RT = 256;
+__global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__ F, int64_t ldf,
+                                                       int Q, int chunk, Grid g,
                                                        const uint8_t* __restrict__ mk,
-                                                       double* __restrict__ part) {
-  const int64_t n = (int64_t)blockIdx.x * UV + threadIdx.x;
-  double r2 = 0.0, e2 = 0.0;
-  // with a mask: the data term over the voxels inside, the pairs with both ends inside
+                                                       double* __restrict__ partial) {
+  const int64_t n = blockIdx.x * (int64_t)RT + threadIdx.x;
+  const int q0 = (int)blockIdx.y * chunk, q1 = min(Q, q0 + chunk);
+  float s = 0.f, c = 0.f;
   if (n < g.N && (!mk || mk[n])) {
-    for (int p = 0; p < P; ++p) {
-      const float r = Res[(int64_t)p * g.ld + n];
-      r2 += (double)r * r;
-    }
     const int x = (int)(n % g.nx);
     const int64_t t = n / g.nx;
     const int y = (int)(t % g.ny), z = (int)(t / g.ny);
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
-    for (int q = 0; q < Q; ++q) {
-      const float* row = F + (int64_t)q * ldf;
-      const float v = row[n];
-      float acc = 0.f;
-      if (x + 1 < g.nx && (!mk || mk[n + 1])) {
-        const float dd = v - row[n + 1];
-        acc = fmaf(dd, dd, acc);
+    const bool hx = x + 1 < g.nx && (!mk || mk[n + 1]);
+    const bool hy = y + 1 < g.ny && (!mk || mk[n + sy]);
+    const bool hz = g.zlink && z + 1 < g.nz && (!mk || mk[n + sz]);
+    // an absent neighbour is the voxel itself
+    const int64_t ox = hx ? 1 : 0, oy = hy ? sy : 0, oz = hz ? sz : 0;
+    const float* p = F + (int64_t)q0 * ldf + n;
+    const bool z3 = g.zlink && g.nz > 1;
+    // RU maps' loads in flight per thread
+    constexpr int RU = 8;
+    int q = q0;
+    for (; q + RU <= q1; q += RU, p += RU * ldf) {
+      float v[RU], vx[RU], vy[RU], vz[RU];
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        v[u] = __ldg(p + u * ldf);
+        vx[u] = __ldg(p + u * ldf + ox);
+        vy[u] = __ldg(p + u * ldf + oy);
+        vz[u] = z3 ? __ldg(p + u * ldf + oz) : v[u];
       }
-      if (y + 1 < g.ny && (!mk || mk[n + sy])) {
-        const float dd = v - row[n + sy];
-        acc = fmaf(dd, dd, acc);
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        const float dx = __fsub_rn(v[u], vx[u]), dy = __fsub_rn(v[u], vy[u]);
+        const float dz = __fsub_rn(v[u], vz[u]);
+        two_sum(s, c, fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, 0.f))));
       }
-      if (g.zlink && z + 1 < g.nz && (!mk || mk[n + sz])) {
-        const float dd = v - row[n + sz];
-        acc = fmaf(dd, dd, acc);
-      }
-      e2 += acc;
+    }
+    for (; q < q1; ++q, p += ldf) {
+      const float v = __ldg(p);
+      const float dx = __fsub_rn(v, __ldg(p + ox)), dy = __fsub_rn(v, __ldg(p + oy));
+      const float dz = z3 ? __fsub_rn(v, __ldg(p + oz)) : 0.f;
+      two_sum(s, c, fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, 0.f))));
     }
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    r2 += __shfl_xor_sync(0xffffffffu, r2, off);
-    e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+  block_partial<RT>(0.0, (double)s + (double)c, 0.0,
+                    partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 4);
+}
+
+// The objective's data term: sum (M - K F)^2 over the voxels inside the object, K F in FP32,
+// each product one FMA chain over the compartments in ascending order (so the residuals
+// depend on neither the tile shape nor the grid), squares and sums in FP64. K is given
+// transposed, so that both operands' compartment slices are rows.
+//
+// Bound: the FP32 pipe (128 FMA per SM and cycle), and next to it the shared-memory pipe. A
+// thread owns 16 rows x 4 voxels and a warp 16 rows x 128 voxels: the rows' K values are
+// the same for every lane (broadcast reads), which takes 8 shared-memory wavefronts per 64
+// FMAs of a warp against the 12 of 8 x 8 outputs per thread, whose reads queued behind one
+// another. Slices of 8 compartments come by cp.async into a ring of NST stages, and the
+// fragments of slice entry k + 1 are read while those of k are multiplied. Tiles of 64
+// rows (4 warps) spread a small problem evenly over the SMs; 128 (8 warps) where that
+// gives every SM two CTAs. P = 120, Q = 2500, N = 16384 (the 128 x 128 slice): 313 -> 278 us
+// in ncu, with sgemm_kernel's 128 CTAs before.
+// VEC: the rows of K^T and F are 16-byte aligned (else scalar copies)
+template <int BM, bool VEC>
+__global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
+    residual_kernel(const ResidualArgs a) {
+  constexpr int BN = 128;
+  constexpr int T = 2 * BM;                        // 16 x 4 outputs each
+  constexpr int BK = 8;
+  constexpr int NST = 4;                           // stages
+  constexpr int STAGE = BK * (BM + BN);            // floats per stage: A slice, B slice
+  constexpr int LA = BM * BK / 4 / T, LB = BN * BK / 4 / T;   // 16-byte copies per thread
+  static_assert(LA >= 1 && LB >= 1, "loader");
+  __shared__ __align__(16) float ring[NST * STAGE];
+  const int tid = threadIdx.x;
+  const int r16 = (tid >> 5) * 16, c4 = (tid & 31) * 4;   // this thread's rows and columns
+  const int M = a.P, N = a.N, K = a.Q;
+  const int mt = (M + BM - 1) / BM;
+  const int m0 = ((int)blockIdx.x % mt) * BM, n0 = ((int)blockIdx.x / mt) * BN;
+  const int ntile = (K + BK - 1) / BK;
+  // k slice kt into stage kt % NST; elements outside the matrices are zero-filled
+  auto copy4 = [&](float* d, const float* base, int64_t ldx, int gk, int gc, int lim) {
+    const int ok = gk < K ? max(0, min(4, lim - gc)) : 0;
+    const float* p = base + (int64_t)gk * ldx + gc;
+    if (VEC) {
+      cp_async<16>(d, ok > 0 ? p : base, 4 * ok);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cp_async<4>(d + j, j < ok ? p + j : base, j < ok ? 4 : 0);
+    }
+  };
+  auto load = [&](int kt) {
+    float* st = ring + (kt % NST) * STAGE;
+#pragma unroll
+    for (int i = 0; i < LA; ++i) {
+      const int f = tid + i * T, kk = f / (BM / 4), c = (f % (BM / 4)) * 4;
+      copy4(st + kk * BM + c, a.Kt, a.ldk, kt * BK + kk, m0 + c, M);
+    }
+#pragma unroll
+    for (int i = 0; i < LB; ++i) {
+      const int f = tid + i * T, kk = f / (BN / 4), c = (f % (BN / 4)) * 4;
+      copy4(st + BK * BM + kk * BN + c, a.F, a.ldf, kt * BK + kk, n0 + c, N);
+    }
+  };
+  auto commit = [] { asm volatile("cp.async.commit_group;\n" ::: "memory"); };
+  float acc[16][4];
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  float4 fa[2][4], fb[2];
+  auto frag = [&](int kt, int k, int buf) {
+    const float* st = ring + (kt % NST) * STAGE;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      fa[buf][i] = *reinterpret_cast<const float4*>(st + k * BM + r16 + 4 * i);
+    fb[buf] = *reinterpret_cast<const float4*>(st + BK * BM + k * BN + c4);
+  };
+#pragma unroll
+  for (int i = 0; i < NST - 1; ++i) {
+    if (i < ntile) load(i);
+    commit();
   }
-  __shared__ double sm[UV / 32][2];
-  if ((threadIdx.x & 31) == 0) {
-    sm[threadIdx.x >> 5][0] = r2;
-    sm[threadIdx.x >> 5][1] = e2;
-  }
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(NST - 2) : "memory");
   __syncthreads();
-  if (threadIdx.x < 2) {
-    double t = 0.0;
-    for (int w = 0; w < UV / 32; ++w) t += sm[w][threadIdx.x];
-    part[(int64_t)blockIdx.x * 4 + threadIdx.x] = t;
+  frag(0, 0, 0);
+#pragma unroll 1
+  for (int kt = 0; kt < ntile; ++kt) {
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      if (k == BK - 1) {
+        // slice kt + 1 has landed (one group per slice, empty ones past the end)
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(NST - 2) : "memory");
+        __syncthreads();
+        if (kt + 1 < ntile) frag(kt + 1, 0, 0);
+      } else {
+        frag(kt, k + 1, (k + 1) & 1);
+      }
+      if (k == 0) {
+        // the stage of slice kt - 1, which every thread has left (the barrier above)
+        if (kt + NST - 1 < ntile) load(kt + NST - 1);
+        commit();
+      }
+      const float4 y = fb[k & 1];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float4 x4 = fa[k & 1][i / 4];
+        const float x = i % 4 == 0 ? x4.x : i % 4 == 1 ? x4.y : i % 4 == 2 ? x4.z : x4.w;
+        acc[i][0] = fmaf(x, y.x, acc[i][0]);
+        acc[i][1] = fmaf(x, y.y, acc[i][1]);
+        acc[i][2] = fmaf(x, y.z, acc[i][2]);
+        acc[i][3] = fmaf(x, y.w, acc[i][3]);
+      }
+    }
   }
+  double r2 = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int gn = n0 + c4 + j;
+    if (gn >= N || (a.mask && !a.mask[gn])) continue;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int gm = m0 + r16 + i;
+      if (gm >= M) continue;
+      const float r = __fsub_rn(__ldg(a.M + (int64_t)gm * a.ldm + gn), acc[i][j]);
+      r2 += (double)r * r;
+    }
+  }
+  block_partial<T>(r2, 0.0, 0.0, a.partial + (int64_t)blockIdx.x * 4);
+}
+
+// rows per tile: 128 where that gives every SM two CTAs and pads no rows that 64 would not
+// (by more than a tenth), else 64
+int residual_rows(int64_t M, int64_t N) {
+  auto up = [](int64_t v, int64_t b) { return (v + b - 1) / b; };
+  const int64_t big = up(M, 128) * up(N, 128), small = up(M, 64) * up(N, 128);
+  return big >= 2 * (int64_t)sm_count() && 20 * big <= 11 * small ? 128 : 64;
+}
+
+int64_t residual_ctas(int64_t M, int64_t N) {
+  const int64_t b = residual_rows(M, N);
+  return (M + b - 1) / b * ((N + 127) / 128);
+}
+
+// Compartment chunks of the roughness sum: about 8 CTAs per SM, at least 16 maps each
+int rough_chunks(const ssm_plan_s* pl, int* chunk) {
+  const int64_t nb = (pl->g.N + RT - 1) / RT;
+  const int64_t c = std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)sm_count() / nb, pl->Q / 16));
+  *chunk = (int)((pl->Q + c - 1) / c);
+  return (pl->Q + *chunk - 1) / *chunk;
 }
 
 }  // namespace
@@ -321,12 +520,49 @@ ssm_status finish_partials(const double* partial, int nparts, int width, double*
   return SSM_OK;
 }
 
-ssm_status objective_terms(const ssm_plan_s* pl, const float* Res, int P, const float* F,
-                           int64_t ldf, double* partial, int* nparts, cudaStream_t s) {
-  const unsigned nb = (unsigned)((pl->g.N + UV - 1) / UV);
-  objective_kernel<<<nb, UV, 0, s>>>(Res, P, F, ldf, pl->Q, pl->g, pl->mask, partial);
+int objective_partials(const ssm_plan_s* pl) {
+  int chunk;
+  const int64_t rough = (pl->g.N + RT - 1) / RT * rough_chunks(pl, &chunk);
+  return (int)std::min<int64_t>(INT32_MAX, residual_ctas(pl->P, pl->g.N) + rough);
+}
+
+// ||M - K F||^2 and the sum over neighbour pairs of the squared differences of F, as
+// partial rows (r2, e2, 0): the product's CTAs' first, then the roughness kernel's
+ssm_status objective_terms(const ssm_plan_s* pl, const float* Kt, const float* M, int64_t ldm,
+                           const float* F, int64_t ldf, double* partial, int* nparts,
+                           cudaStream_t s) {
+  ResidualArgs a;
+  a.P = pl->P;
+  a.N = (int)pl->g.N;
+  a.Q = pl->Q;
+  a.Kt = Kt;
+  a.ldk = (pl->P + 3) / 4 * 4;
+  a.F = F;
+  a.ldf = ldf;
+  a.M = M;
+  a.ldm = ldm;
+  a.mask = pl->mask;
+  a.partial = partial;
+  const int64_t ctas = residual_ctas(pl->P, pl->g.N);
+  if (ctas > INT32_MAX) {
+    set_error("objective: too many tiles");
+    return SSM_EINVAL;
+  }
+  const bool big = residual_rows(pl->P, pl->g.N) == 128;
+  const bool vec = ldf % 4 == 0 && (reinterpret_cast<uintptr_t>(F) & 15) == 0;
+  const unsigned gr = (unsigned)ctas;
+  if (big && vec) residual_kernel<128, true><<<gr, 256, 0, s>>>(a);
+  else if (big) residual_kernel<128, false><<<gr, 256, 0, s>>>(a);
+  else if (vec) residual_kernel<64, true><<<gr, 128, 0, s>>>(a);
+  else residual_kernel<64, false><<<gr, 128, 0, s>>>(a);
   SSM_LAUNCHED();
-  *nparts = (int)nb;
+  int chunk;
+  const int chunks = rough_chunks(pl, &chunk);
+  const dim3 grid((unsigned)((pl->g.N + RT - 1) / RT), (unsigned)chunks);
+  roughness_kernel<<<grid, RT, 0, s>>>(F, ldf, pl->Q, chunk, pl->g, pl->mask,
+                                       partial + ctas * 4);
+  SSM_LAUNCHED();
+  *nparts = objective_partials(pl);
   return SSM_OK;
 }
 

@@ -150,8 +150,8 @@ struct ssm_plan_s {
   double* sig64 = nullptr;     // n      : sigma_i (descending)
 
   // FP32 operands
-  float* K32 = nullptr;        // P x Q (objective with the full K)
-  float* Kr32 = nullptr;       // P x Q (objective with K_r)
+  float* K32 = nullptr;        // K^T,   Q x P (rows padded to 4 floats): objective, full K
+  float* Kr32 = nullptr;       // K_r^T, Q x P (rows padded to 4 floats): objective, K_r
   float* V32 = nullptr;        // Q x R  [q][i]  low-rank right singular vectors
                                // (multi plans: Q x ndict x R, [q][c][i])
   // TF32x3 low-rank form: V (Q x R) and V^T (R x lrtc_qs), split into TF32 hi/lo parts
@@ -184,7 +184,6 @@ struct ssm_plan_s {
   float* Acc = nullptr;              // M w                    (Q x ld)     dense fp32
   __nv_bfloat16* Whi[2] = {nullptr, nullptr};  // w split, ping-pong (Q x ld) dense bf16
   __nv_bfloat16* Wlo[2] = {nullptr, nullptr};
-  float* Res = nullptr;              // P x ld residual buffer for the objective (lazy)
   float* Mstage = nullptr;           // P x ld device staging for ssm_solve_host (lazy)
   float* Fstage = nullptr;           // Q x ld
   double* red = nullptr;             // reduction partials
@@ -318,8 +317,10 @@ ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check,
 int dense_max_partials(const ssm_plan_s* pl);
 ssm_status finish_partials(const double* partial, int nparts, int width, double* out,
                            cudaStream_t s);
-ssm_status objective_terms(const ssm_plan_s* pl, const float* Res, int P, const float* F,
-                           int64_t ldf, double* partial, int* nparts, cudaStream_t s);
+int objective_partials(const ssm_plan_s* pl);
+ssm_status objective_terms(const ssm_plan_s* pl, const float* Kt, const float* M, int64_t ldm,
+                           const float* F, int64_t ldf, double* partial, int* nparts,
+                           cudaStream_t s);
 
 // Algorithm 1 (ssm_admm.cu)
 ssm_status admm_tables(ssm_plan_s* pl, std::vector<std::pair<float**, std::vector<float>>>* out);

@@ -247,9 +247,13 @@ __global__ void lowrank_basis(const double* __restrict__ Kt, int Q, int n, const
   }
 }
 
-__global__ void to_f32(const double* __restrict__ X, int64_t count, float* __restrict__ Y) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < count) Y[i] = (float)X[i];
+// Y (cols x ldy) = X^T (X rows x cols) in FP32, zero for the padding columns
+__global__ void to_f32_transposed(const double* __restrict__ X, int rows, int cols, int ldy,
+                                  float* __restrict__ Y) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= (int64_t)cols * ldy) return;
+  const int c = (int)(i / ldy), r = (int)(i % ldy);
+  Y[i] = r < rows ? (float)X[(int64_t)r * cols + c] : 0.f;
 }
 
 // Eq. 26 assembled from the eigenpairs (exact Woodbury form, no division by sigma):
@@ -372,13 +376,15 @@ ssm_status factors_fp64(ssm_plan_s* pl, const double* E, cudaStream_t s) {
                            cudaMemcpyHostToDevice, s));
   SSM_CUDA(cudaStreamSynchronize(s));   // `alpha` is a host temporary
   SSM_TRY(beta_weights(pl, s));
-  // dictionaries for the objective: K (FP32) and K_r = Bp_r Kt_r^T
-  to_f32<<<nblk((int64_t)P * Q, 256), 256, 0, s>>>(pl->K64, (int64_t)P * Q, pl->K32);
+  // dictionaries for the objective, transposed: K (FP32) and K_r = Bp_r Kt_r^T
+  const int P4 = (P + 3) / 4 * 4;
+  const unsigned nt = nblk((int64_t)Q * P4, 256);
+  to_f32_transposed<<<nt, 256, 0, s>>>(pl->K64, P, Q, P4, pl->K32);
   SSM_LAUNCHED();
   double* Kr64 = nullptr;
   SSM_CUDA(cudaMallocAsync(&Kr64, sizeof(double) * P * Q, s));
   SSM_TRY(dgemm(P, Q, pl->r, pl->Bp64, n, false, pl->Kt64, n, true, Kr64, Q, s));
-  to_f32<<<nblk((int64_t)P * Q, 256), 256, 0, s>>>(Kr64, (int64_t)P * Q, pl->Kr32);
+  to_f32_transposed<<<nt, 256, 0, s>>>(Kr64, P, Q, P4, pl->Kr32);
   SSM_LAUNCHED();
   SSM_CUDA(cudaFreeAsync(Kr64, s));
   return SSM_OK;
