@@ -39,9 +39,9 @@ std::mutex& attr_mutex() {
   return m;
 }
 
-cudaError_t encode_2d(CUtensorMap* map, CUtensorMapDataType dtype, size_t elem, const void* base,
-                      uint64_t cols, uint64_t rows, uint64_t ld, unsigned box_cols,
-                      unsigned box_rows, CUtensorMapSwizzle swizzle) {
+cudaError_t encode_nd(CUtensorMap* map, CUtensorMapDataType dtype, unsigned rank, const void* base,
+                      const uint64_t* dims, const uint64_t* strides, const unsigned* box,
+                      CUtensorMapSwizzle swizzle) {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
     void* p = nullptr;
@@ -54,11 +54,15 @@ cudaError_t encode_2d(CUtensorMap* map, CUtensorMapDataType dtype, size_t elem, 
     }
     fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
   }
-  cuuint64_t dims[2] = {cols, rows};
-  cuuint64_t strides[1] = {ld * elem};
-  cuuint32_t box[2] = {box_cols, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(map, dtype, 2, const_cast<void*>(base), dims, strides, box, estr,
+  cuuint64_t d[5], st[4];
+  cuuint32_t bx[5], estr[5];
+  for (unsigned i = 0; i < rank; ++i) {
+    d[i] = dims[i];
+    bx[i] = box[i];
+    estr[i] = 1;
+    if (i + 1 < rank) st[i] = strides[i];
+  }
+  CUresult r = fn(map, dtype, rank, const_cast<void*>(base), d, st, bx, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
@@ -66,6 +70,14 @@ cudaError_t encode_2d(CUtensorMap* map, CUtensorMapDataType dtype, size_t elem, 
     return cudaErrorInvalidValue;
   }
   return cudaSuccess;
+}
+
+cudaError_t encode_2d(CUtensorMap* map, CUtensorMapDataType dtype, size_t elem, const void* base,
+                      uint64_t cols, uint64_t rows, uint64_t ld, unsigned box_cols,
+                      unsigned box_rows, CUtensorMapSwizzle swizzle) {
+  const uint64_t dims[2] = {cols, rows}, strides[1] = {ld * elem};
+  const unsigned box[2] = {box_cols, box_rows};
+  return encode_nd(map, dtype, 2, base, dims, strides, box, swizzle);
 }
 
 namespace {
@@ -87,6 +99,13 @@ int64_t lowrank_state_floats(const ssm_plan_s* pl, int64_t grid) {
   if (pl->ndict > 0) return table_state_floats(pl->g.N, pl->mseg, pl->R);
   return pl->p.precision == SSM_TF32X3 ? lrtc_partial_floats(pl, grid)
                                        : lowrank_partial_floats(pl, grid);
+}
+
+// floats of one state array (z or d): blocked for the TF32x3 form, else Q x ld
+int64_t state_floats(const ssm_plan_s* pl) {
+  if (pl->p.form == SSM_FORM_LOWRANK && pl->p.precision == SSM_TF32X3)
+    return lrtc_state_floats(pl);
+  return (int64_t)pl->Q * pl->g.ld;
 }
 
 int padded_rank(int r) {
@@ -173,6 +192,7 @@ ssm_status validate(const ssm_params* p) {
 void release(ssm_plan_s* pl) {
   if (!pl) return;
   tc_release(pl);
+  lrtc_release(pl);
   dfree(pl->K64);
   dfree(pl->Bp64);
   dfree(pl->Kt64);
@@ -391,11 +411,11 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
   SSM_CUDA(cudaMemsetAsync(pl->dev_err, 0, sizeof(int), s));
 
   // per-voxel state
-  const size_t QN = (size_t)Q * pl->g.ld;
+  const size_t QN = (size_t)Q * pl->g.ld, ZN = (size_t)state_floats(pl);
   if (p.form != SSM_FORM_ADMM)
     for (int i = 0; i < 2; ++i) {
-      SSM_TRY(palloc(pl, &pl->Z[i], QN, s));
-      SSM_TRY(palloc(pl, &pl->Dl[i], QN, s));
+      SSM_TRY(palloc(pl, &pl->Z[i], ZN, s));
+      SSM_TRY(palloc(pl, &pl->Dl[i], ZN, s));
     }
   int maxparts = 1;
   if (p.form == SSM_FORM_ADMM) {
@@ -417,7 +437,7 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
   } else if (p.form == SSM_FORM_LOWRANK) {
     SSM_TRY(palloc(pl, &pl->S, (size_t)pl->R * pl->g.ld, s));
     if (p.precision == SSM_TF32X3) {
-      SSM_TRY(lrtc_prepare());
+      SSM_TRY(lrtc_prepare(pl));
       pl->lr_grid = lrtc_grid(pl);
       maxparts = (int)pl->lr_grid;
     } else {
@@ -681,7 +701,7 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
     add(4, ld);                               // vexp
   }
   const int64_t QN = Q * ld;
-  if (p.form != SSM_FORM_ADMM) add(4, 4 * QN);  // Z[2], Dl[2]
+  if (p.form != SSM_FORM_ADMM) add(4, 4 * state_floats(&t));  // Z[2], Dl[2]
   int64_t maxparts = 1;
   if (p.form == SSM_FORM_ADMM) {
     add(4, 10 * QN);                          // x, y, z, d_x, d_y, d_z, f, w, r, t
@@ -962,9 +982,10 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
     // with a mask, voxels outside the object are never written: both ping-pong halves
     // (and both tensor-core operands) must hold zeros there
     const int nbuf = pl->mask ? 2 : 1;
+    const size_t zbytes = sizeof(float) * (size_t)state_floats(pl);
     for (int i = 0; i < nbuf; ++i) {
-      SSM_CUDA(cudaMemsetAsync(pl->Z[i], 0, sizeof(float) * QN, s));
-      SSM_CUDA(cudaMemsetAsync(pl->Dl[i], 0, sizeof(float) * QN, s));
+      SSM_CUDA(cudaMemsetAsync(pl->Z[i], 0, zbytes, s));
+      SSM_CUDA(cudaMemsetAsync(pl->Dl[i], 0, zbytes, s));
     }
     if (pl->mask && pl->Whi[1]) {
       const size_t WN = (size_t)pl->g.ld * pl->Qp;
@@ -1020,8 +1041,11 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
   pl->has_state = true;
   // F = z (the feasible iterate; y for Algorithm 1)
   const float* Fsrc = p.form == SSM_FORM_ADMM ? pl->adm.y : pl->Z[cur];
-  SSM_CUDA(cudaMemcpy2DAsync(F, sizeof(float) * ldf, Fsrc, sizeof(float) * ld,
-                             sizeof(float) * pl->g.N, pl->Q, cudaMemcpyDeviceToDevice, s));
+  if (pl->lrtc_state)
+    SSM_TRY(lrtc_output(pl, cur, F, ldf, s));
+  else
+    SSM_CUDA(cudaMemcpy2DAsync(F, sizeof(float) * ldf, Fsrc, sizeof(float) * ld,
+                               sizeof(float) * pl->g.N, pl->Q, cudaMemcpyDeviceToDevice, s));
   if (info) {
     SSM_CUDA(cudaStreamSynchronize(s));
     info->status = result;

@@ -160,6 +160,7 @@ struct ssm_plan_s {
   float* V2h = nullptr;
   float* V2l = nullptr;
   int lrtc_qs = 0;             // row stride of V^T: Q rounded up to 32
+  void* lrtc_state = nullptr;  // its tiles and tensor maps (ssm_lowrank_tc.cu)
   float* coefA = nullptr;      // R      1/(beta + sigma_i^2)
   float* coefW = nullptr;      // R      sigma_i^2/(beta^2 + beta sigma_i^2)
   double* alpha64 = nullptr;   // n      S_i = alpha_i c_i
@@ -173,7 +174,8 @@ struct ssm_plan_s {
   int* vexp = nullptr;               // ld
   int Qp = 0;                  // padded row stride of Q x Q operands
 
-  // per-voxel state (map-major, leading dimension g.ld)
+  // per-voxel state (map-major, leading dimension g.ld; z and d of the TF32x3 form are
+  // blocked, see ssm_lowrank_tc.cu)
   float* Z[2] = {nullptr, nullptr};  // z ping-pong            (Q x ld)
   float* Dl[2] = {nullptr, nullptr}; // dual d ping-pong       (Q x ld)
   float* S = nullptr;                // S_i = sigma_i u_i^T m  (R x ld)
@@ -281,7 +283,10 @@ int64_t lowrank_partial_floats(const ssm_plan_s* pl, int64_t grid);
 int lrtc_padded_rank(int r, bool three_d);
 int64_t lrtc_grid(const ssm_plan_s* pl);
 int64_t lrtc_partial_floats(const ssm_plan_s* pl, int64_t grid);
-ssm_status lrtc_prepare();
+int64_t lrtc_state_floats(const ssm_plan_s* pl);
+ssm_status lrtc_prepare(ssm_plan_s* pl);
+void lrtc_release(ssm_plan_s* pl);
+ssm_status lrtc_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, cudaStream_t s);
 ssm_status lrtc_split_basis(ssm_plan_s* pl, cudaStream_t s);
 ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                           int* nparts, cudaStream_t s);

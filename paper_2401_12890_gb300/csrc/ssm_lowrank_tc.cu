@@ -4,17 +4,17 @@
 // The iteration is the d-free recurrence of ssm_lowrank.cu (the algebra is derived there):
 // with a_i = S_i/(beta + sigma_i^2) - W_i u_i per voxel (u summed from the previous
 // iteration's partial products),
-//     t  = z + V a                                              (rank-r product 1)
+//     t  = z + V a                                            (rank-r product 1)
 //     z' = max(0, e1 z + c2 sum_nbr z + c3 (V a))               (Eq. 31)
 //     d' = beta (t - z')                                        (step 11)
 //     w  = beta (2 z' - t)            (= beta z' - d')
 //     u' = V^T w                                                (rank-r product 2)
-// For a tile of 128 voxels and a chunk of QC = 32 compartments both products are matrix
-// products with the voxels as the M dimension:
+// For a tile of up to 128 voxels and a chunk of QC = 32 compartments both products are
+// matrix products with the voxels as the M dimension:
 //     VA [128 x 32] = A [128 x RP] . V_c^T [RP x 32]      (K = rank, padded to RP = 32/64)
 //     U  [128 x RP] = W [128 x 32] . V_c   [32 x RP]      (K = the chunk's compartments)
 // Both run as tcgen05.mma kind::tf32 with FP32 accumulation in tensor memory (TMEM). The
-// A operands live in TMEM too: the epilogue warps own one voxel (= one TMEM lane) each
+// A operands live in TMEM too: the epilogue warps own one voxel (= one TMEM lane) per thread
 // and write a (once per tile segment) and w (per chunk) with tcgen05.st; the B operands
 // (the chunk's rows of V and of V^T) are TMA boxes in the 128-byte-swizzled K-major layout.
 //
@@ -28,30 +28,58 @@
 // chunk and its 32-compartment partial sums are added into registers the same way (a
 // chain over all Q compartments would bias u').
 //
+// State layout: z and d are kept blocked, [chunk][voxel][32 compartments], 128 bytes per
+// voxel and chunk (the compartments past Q are zero and stay zero). A tile is a patch of
+// bx x by x bz <= 128 voxels of the grid; one five-dimensional TMA box loads it with its
+// halo as 128-byte-swizzled rows, zero-filled beyond the grid, and another stores it. What
+// this buys over map-major rows of 128 voxels (the layout of F, used here before):
+//   - a 16 x 8 patch of a 2D grid loads 180 rows per chunk instead of 3 x 128 and their
+//     alignment slack, an 8 x 4 x 4 patch 360 instead of 5 x 128: about half the traffic
+//     between L2 and the SMs, and room for more stages;
+//   - a thread reads 4 compartments of a voxel (and of each neighbour) with one 128-bit
+//     shared-memory load, straight into the register pairs of the packed FP32x2
+//     arithmetic, and neighbours beyond the grid (or outside the object, whose z is 0)
+//     read as zeros: no neighbour flags in the loop;
+//   - z' leaves by TMA: no global address arithmetic and no store instructions.
+// Measured per iteration in a solve, map-major tiles and one MMA warp before, now:
+//   128x128, Q = 2500, r = 20          110.6 -> 86.0 us
+//   256x256, Q = 2500, r = 20          446.9 -> 297 us
+//   96x96x64, Q = 1600, r = 30          3300 -> 2041 us
+//   192x192, Q = 900, r = 8            85.4 -> 67.0 us
+//   40 slices of 37x29, Q = 225, r = 20  44.9 -> 37.6 us
+//   32x32, Q = 225, r = 20             10.3 -> 9.7 us
+//
 // Schedule (one CTA per SM): the work units are (segment, tile) pairs, segment-major,
 // dealt round-robin to the CTAs; a segment is a contiguous run of a tile's chunks (one
 // segment per tile when there are at least as many tiles as CTAs, several otherwise).
-// CTAs running together therefore hold the same chunks of consecutive tiles, and the
-// neighbour rows each of them stages were just read by another: L2 hits. With between
-// half as many tiles as CTAs and as many, each tile is one main unit and one tail unit
-// instead, the tails going to the CTAs that would otherwise idle (see layout()). Each segment
-// writes its partial u' to its own slot; the next iteration sums a tile's slots in
-// segment order (fixed, hence deterministic). Warp roles:
-//   warp 0      TMA: per chunk, z with its x halo, the -+nx (-+nx*ny) neighbour rows and
-//               the chunk's V / V^T boxes (hi and lo) into a ring of NS stages
-//   warp 1      MMA: product 1 of chunk g, then product 2 of chunk g - (NVA - 1) (so the
-//               tensor core works ahead of the epilogue); commits release stages and buffers
-//   warps 2-9   epilogue (2-17 on 3D grids and in residual-test iterations), two (four)
-//               per TMEM lane quarter, each a half (quarter) of a chunk's compartments:
-//               tcgen05.ld of V a, the z-step and dual step, z' (and d') stores, w split
-//               into TMEM, and the running sum of product 2 in registers
+// CTAs running together therefore hold the same chunks of neighbouring tiles, and the
+// halos are L2 hits. With between half as many tiles as CTAs and as many, each tile is one
+// main unit and one tail unit instead, the tails going to the CTAs that would otherwise
+// idle (see layout()). Each segment writes its partial u' to its own slot; the next
+// iteration sums a tile's slots in segment order (fixed, hence deterministic). Warp roles:
+//   warp 0      TMA: per chunk, the patch of z with its halo (and of d on residual-test
+//               iterations) and the chunk's V / V^T boxes (hi and lo)
+//   warp 1      product 1, up to NSV - 1 chunks ahead of product 2
+//   warp 2      product 2 as soon as a chunk's w is complete. Two warps, because an MMA takes
+//               62 cycles to issue whatever its N (measured, N <= 128): issued by one
+//               thread in turn with its waits, 21 MMAs per chunk (N = 32 each) bounded the
+//               whole kernel at 2900 cycles per chunk. The hi and lo rows of V lie side by
+//               side as one operand of N = 64 (2 RP), which takes 14
+//   warps 4-11  epilogue: two groups of four (one per TMEM lane quarter), which take the
+//               chunks alternately, so that one group's waits and TMEM round trips overlap
+//               the other's arithmetic: tcgen05.ld of V a, the z-step and dual step, z' (and
+//               d') to shared memory, w split into TMEM, and the running sum of its chunks'
+//               product 2 in registers. One thread per group issues the TMA stores.
 // Waiting warps sleep in mbarrier.try_wait (with a suspend-time hint) instead of polling.
-// TMEM: V a (main, correction) and w (hi, lo) are double-buffered by chunk parity, a is
-// per segment, U (main, correction) is double-buffered for RP = 32 and single for 64.
+// TMEM: NVA slots of 64 columns, each holding a chunk's V a (main, correction) and then,
+// column by column once read, its w (hi, lo), until product 2 of the chunk has completed. a
+// (hi, lo) is per segment; U (main, correction) is double-buffered for RP = 32 and single
+// for 64.
 // HBM traffic per state element and iteration: read z, write z' (8 B); per voxel and rank:
 // S, the partial u in and out. Every mbarrier wait is bounded and reports SSM_ETIMEOUT
-// through the plan's device error word; the TMA warp waits (bounded) for its last copies
-// and the MMA warp for its last products before the CTA frees its TMEM and exits.
+// through the plan's device error word; the TMA warp waits (bounded) for its last copies,
+// the storing threads for their stores and the MMA warp for its last products before the
+// CTA frees its TMEM and exits.
 #include <algorithm>
 #include <cstdlib>
 
@@ -61,105 +89,82 @@
 namespace ssm {
 namespace {
 
-constexpr int TV = 128;              // voxels per tile: MMA M, TMEM lanes
+constexpr int TV = 128;              // lanes per tile: MMA M, TMEM lanes
 constexpr int QC = 32;               // compartments per chunk
-// epilogue warps: 8 on 1D/2D grids, 16 on 3D grids (whose elements read four neighbour
-// rows: more warps hide their longer latency chains) and in residual-test iterations
-// (which also load d^k per element); EPQ per TMEM lane quarter, each taking GC
-// compartments of a chunk
-template <int NR, bool CHECK> struct Epi {
-  static constexpr int NEPI = (NR == 4 || CHECK) ? 16 : 8;
-  static constexpr int EPQ = NEPI / 4;
-  static constexpr int GC = 32 / EPQ;
-  static constexpr int NT = 32 * (2 + NEPI);
-  static_assert(NEPI % 4 == 0 && GC % 8 == 0, "epilogue split");
-};
-constexpr int ZW = TV + 8;           // staged z row: voxels n0-4 .. n0+TV+3
-constexpr int NW = TV + 4;           // staged neighbour row: 4-aligned base .. +TV+3
+constexpr int NG = 2;                // epilogue groups of four warps
+constexpr int NT = 128 + 128 * NG;
+constexpr int NVA = 4;               // V a / w slots in TMEM: even, so that a slot's chunks all
+                                     // belong to one group (its phases complete in the order
+                                     // that group waits for them)
+constexpr int kPrefetch = 4;         // chunks of a tile's own z rows prefetched into L2 ahead
+constexpr int kMaxNSZ = 8;           // z stages (as many as fit, at most)
+constexpr int OUT_BYTES = TV * 128;  // one chunk of a tile's z' (or d')
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int kSmemLimit = 227 * 1024;
-constexpr int kPrefetch = 8;         // chunks of a tile's own z rows prefetched into L2 ahead
+constexpr int kReserve = 1024 + 1024 + 512 + 1024;   // alignment, the residual variant's static
+                                                     // array, barriers, weights and zero row
 
-// Rings, buffers and tensor-memory columns of one kernel configuration.
-//   V ring (NSV stages): the chunk's V boxes (B of product 1) and V^T boxes (B of product
-//     2), hi and lo; a stage is held from its load until product 2 of its chunk completes
-//   z ring (NSZ stages): z with its x halo and the NR neighbour rows; held until the
-//     epilogue warps have read it
-//   TMEM: V a in NVA buffers (main and correction, 64 columns each), w in 2 (hi and lo),
-//     a (hi and lo, per segment), U in UB buffers (main and correction, 2 RP columns)
-// Product 1 runs NVA - 1 chunks ahead of the epilogue and the epilogue reads product 2's
-// sums two chunks late, so neither MMA latency is on the epilogue's path.
-template <int RP, int NR>
+template <int RP, int NAX>
 struct Lay {
-  static constexpr int NVA = RP == 32 ? 3 : 2;
+  // V stages (product 1 runs up to NSV - 1 chunks ahead of product 2)
+  static constexpr int NSV = RP == 32 && NAX < 3 ? NVA : NVA - 1;
   static constexpr int UB = RP == 32 ? 2 : 1;
   static constexpr int V1 = RP / 32 * QC * 128;   // V rows of the chunk: RP/32 swizzle atoms
   static constexpr int V2 = RP * 128;            // V^T rows (RP) x the chunk (128 bytes)
-  static constexpr int v1h = 0, v1l = V1, v2h = 2 * V1, v2l = 2 * V1 + V2;
+  // per 32 ranks: the chunk's rows of V_hi, then those of V_lo (one B operand of N = 64);
+  // then the rows of V_hi^T and of V_lo^T (one of N = 2 RP)
+  static constexpr int v1(int at, int part) { return (2 * at + part) * QC * 128; }
+  static constexpr int v2h = 2 * V1, v2l = 2 * V1 + V2;
   static constexpr int VST = 2 * V1 + 2 * V2;    // V stage (a multiple of 1024)
-  static constexpr int zc = 0;
-  static constexpr int zn = QC * ZW * 4;
-  static constexpr int ZST = (zn + NR * QC * NW * 4 + 1023) / 1024 * 1024;
-  static constexpr int RESERVE = 1024 + 512;     // alignment slack, barriers, TMEM slot
-  static constexpr int STATIC_MAX = 1024;       // the residual variant's reduction array
-  static constexpr int budget = kSmemLimit - RESERVE - STATIC_MAX;
-  static constexpr int nsz_with(int nsv) { return (budget - nsv * VST) / ZST; }
-  static constexpr int NSV = nsz_with(NVA + 1) >= 2 ? NVA + 1 : NVA;
-  static constexpr int NSZ = nsz_with(NSV) > 4 ? 4 : nsz_with(NSV);
-  static constexpr bool valid = NSZ >= 2 && NSV >= 2;
-  static constexpr int zbase = NSV * VST;        // the z ring after the V ring
-  static constexpr int bytes = (valid ? zbase + NSZ * ZST : 0) + RESERVE;
-  static constexpr unsigned VBYTES = (unsigned)VST;
-  static constexpr unsigned ZBYTES = (unsigned)(QC * ZW * 4 + NR * QC * NW * 4);
-  static constexpr uint32_t T_VA = 0;                     // buffer b: main 64 b, corr +32
-  static constexpr uint32_t T_W = 64 * NVA;               // buffer p: hi 64 p, lo +32
-  static constexpr uint32_t T_A = T_W + 128;              // hi, lo at + RP
+  static constexpr uint32_t T_VA = 0;                     // slot b: 64 b (main / hi, +32)
+  static constexpr uint32_t T_A = 64 * NVA;               // hi, lo at + RP
   static constexpr uint32_t T_U = T_A + 2 * RP;           // buffer b: main 2 RP b, corr + RP
   // kind::tf32 instruction descriptors: D = F32 (bits 4-5 = 1), A = B = TF32 (bits 7-9,
   // 10-12 = 2), both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28
-  static constexpr uint32_t IDESC1 = (1u << 4) | (2u << 7) | (2u << 10) |
-                                     ((uint32_t)(QC >> 3) << 17) | ((uint32_t)(TV >> 4) << 24);
-  static constexpr uint32_t IDESC2 = (1u << 4) | (2u << 7) | (2u << 10) |
-                                     ((uint32_t)(RP >> 3) << 17) | ((uint32_t)(TV >> 4) << 24);
-  static_assert(VST % 1024 == 0 && ZST % 1024 == 0 && zn % 128 == 0 && v1l % 1024 == 0 &&
-                    v2h % 1024 == 0 && v2l % 1024 == 0,
-                "layout");
+  static constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(TV >> 4) << 24);
+  }
+  static_assert(VST % 1024 == 0 && v2h % 1024 == 0 && v2l % 1024 == 0, "layout");
   static_assert(T_U + 2 * RP * UB <= TMEM_COLS, "tensor memory");
+};
+
+// The tiles of a grid: patches of bx x by x bz voxels (lane = lx + bx (ly + by lz)), loaded
+// with a halo of one voxel on every axis with smoothness (h = 1) as X x Y x Z rows
+struct Patch {
+  int bx, by, bz, hx, hy, hz;
+  int X, Y, Z, rows;
+  int tx, ty, tz;            // tiles per axis
+  int64_t ntiles;
+  int naxes;                 // axes with smoothness (at least 1: see patch_of)
+  int zst;                   // bytes of the z rows, rounded up to 1024
 };
 
 struct LrtcMaps {
   CUtensorMap v1h, v1l;   // V (Q x RP), box {32, QC}, 128-byte swizzle
   CUtensorMap v2h, v2l;   // V^T (RP x Qs), box {QC, RP}, 128-byte swizzle
-  CUtensorMap zc, zn;     // z^k (Q x N), boxes {ZW, QC} and {NW, QC}
-  CUtensorMap dd;         // d^k (Q x N), box {TV, QC}: prefetched into L2 before a residual
-                          // test reads it
+  CUtensorMap zi, zp;     // z^k, boxes {32, X, Y, Z, 1} and {32, bx, by, bz, 1} (prefetch)
+  CUtensorMap zo, di, dd; // z^{k+1}, d^k, d^{k+1}: box {32, bx, by, bz, 1}
 };
 
 struct LrtcArgs {
-  float* __restrict__ Zout;
-  float* __restrict__ Dout;         // d^{k+1} (iterations before a residual test)
-  const float* __restrict__ Din;    // d^k (residual-test iterations)
   const float* __restrict__ S;      // RP x ld
-  const float* __restrict__ Pin;    // partial u of the previous iteration [tile][seg][RP][TV]
+  const float* __restrict__ Pin;    // partial u of the previous iteration [tile][slot][RP][TV]
   float* __restrict__ Pout;         // partial u of this iteration
-  int64_t ntiles;                   // voxel tiles
   int nch;                          // compartment chunks per tile
   int spc;                          // segments per tile (each a contiguous run of chunks)
   int split;                        // > 0: main/tail layout, the chunk where tails start
   int kr;                           // K steps of 8 ranks holding the rank r (<= RP / 8)
+  int nsz, nob;                     // z stages; z' (and d') buffers per group, 1 or 2
   const float* __restrict__ coefA;  // RP
   const float* __restrict__ coefW;  // RP
   double* __restrict__ partial;     // 4 doubles per block (check iterations)
   const uint8_t* __restrict__ mask; // voxels inside the object (nullptr: every voxel)
   int* __restrict__ err;            // device error word
   Grid g;
-  int Q;
+  Patch p;
   float beta, inv_beta, xi, lam_s, inv_xb;
 };
-
-__host__ __device__ __forceinline__ int64_t floor4(int64_t v) {
-  return v >= 0 ? (v & ~(int64_t)3) : -(((-v) + 3) & ~(int64_t)3);
-}
 
 // x rounded to TF32 (10 stored mantissa bits), to nearest with ties away from zero: add
 // half a unit of the last kept place to the magnitude bits and clear the 13 bits below
@@ -213,111 +218,127 @@ __device__ __forceinline__ void tst_wait() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// C consecutive 32-bit columns at each of two TMEM addresses (one lane per thread): both
-// loads are in flight together and one wait covers them (the outputs are defined by the
-// statement that waits, so no use of them can be scheduled before the wait)
+// C consecutive 32-bit columns of this warp's TMEM lanes; the values are defined after the
+// next tld_wait on the same registers
 template <int C>
-__device__ __forceinline__ void tld2(uint32_t t0, uint32_t t1, float* v0, float* v1) {
+__device__ __forceinline__ void tld(uint32_t t, uint32_t* r) {
   static_assert(C == 8 || C == 16, "columns per load");
-  uint32_t r[2 * C];
-  if constexpr (C == 8) {
+  if constexpr (C == 8)
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
-        "tcgen05.wait::ld.sync.aligned;\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7])
+        : "r"(t)
+        : "memory");
+  else
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+        "%11, %12, %13, %14, %15}, [%16];\n"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
           "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(t0), "r"(t1)
+        : "r"(t)
         : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-        "%11, %12, %13, %14, %15}, [%32];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, "
-        "%25, %26, %27, %28, %29, %30, %31}, [%33];\n\t"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(t0), "r"(t1)
-        : "memory");
-  }
-#pragma unroll
-  for (int i = 0; i < C; ++i) {
-    v0[i] = __uint_as_float(r[i]);
-    v1[i] = __uint_as_float(r[C + i]);
-  }
 }
-
-// C columns (a multiple of 8) at each of two TMEM addresses, 16 (or 8) per wait
 template <int C>
-__device__ __forceinline__ void tld2_cols(uint32_t t0, uint32_t t1, float* v0, float* v1) {
-  static_assert(C % 8 == 0, "columns");
-  constexpr int S = C % 16 == 0 ? 16 : 8;
+__device__ __forceinline__ void tld_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int k = 0; k < C; k += S) tld2<S>(t0 + k, t1 + k, v0 + k, v1 + k);
+  for (int i = 0; i < C; ++i) asm volatile("" : "+r"(r[i]));   // no use moves above the wait
 }
 
-template <int RP, int NR, bool CHECK, bool WD>
-__global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __grid_constant__ LrtcMaps maps,
-                                                              const LrtcArgs a) {
-  using L = Lay<RP, NR>;
-  using E = Epi<NR, CHECK>;
-  constexpr int NEPI = E::NEPI, EPQ = E::EPQ, GC = E::GC, NT = E::NT;
-  constexpr int NSV = L::NSV, NSZ = L::NSZ, NVA = L::NVA, UB = L::UB;
-  constexpr int D1 = NVA - 1;         // chunks product 1 runs ahead of product 2
-  constexpr int RQ = RP / EPQ;        // ranks per epilogue warp of a lane quarter
-  static_assert(L::valid, "two ring stages");
-  static_assert(RQ % 8 == 0, "rank split");
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(x), "f"(y), "f"(z),
+               "f"(w)
+               : "memory");
+}
+__device__ __forceinline__ void group_barrier(int id) {
+  asm volatile("bar.sync %0, 128;\n" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() {
+  asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+// the thread's bulk stores have read their shared memory
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() {
+  asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+}
+
+// NAX: axes with smoothness (neighbour pairs per element)
+template <int RP, int NAX, bool CHECK, bool WD>
+__global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ LrtcMaps maps,
+                                                     const LrtcArgs a) {
+  using L = Lay<RP, NAX>;
+  constexpr int UB = L::UB, NSV = L::NSV;
+  constexpr int RQ = RP / NG;         // ranks of a per epilogue group
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // aligned by an offset from the shared array itself (not through an integer), so that
   // the compiler keeps the shared address space of every pointer derived from it
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int nsz = a.nsz, nob = a.nob;
+  const int zst = a.p.zst + (CHECK ? OUT_BYTES : 0);      // z rows, then d^k
   unsigned char* vring = smem;
-  unsigned char* zring = smem + L::zbase;
-  uint64_t* vfull = reinterpret_cast<uint64_t*>(zring + NSZ * L::ZST);
+  unsigned char* obuf = smem + NSV * L::VST;              // [group][buffer]: z', then d'
+  // a residual test that also stores d writes it over the staged d^k
+  constexpr bool OWN_D = WD && !CHECK;
+  constexpr int OB = OUT_BYTES * (OWN_D ? 2 : 1);
+  unsigned char* zring = obuf + NG * nob * OB;
+  unsigned char* tail = zring + nsz * zst;
+  float* zero_row = reinterpret_cast<float*>(tail);       // 128 bytes of zeros (128-aligned)
+  float* cAW = zero_row + 32;                             // coefA, coefW (RP each)
+  uint64_t* vfull = reinterpret_cast<uint64_t*>(cAW + 2 * RP);
   uint64_t* vempty = vfull + NSV;
   uint64_t* zfull = vempty + NSV;
-  uint64_t* zempty = zfull + NSZ;
-  uint64_t* va_full = zempty + NSZ;
-  uint64_t* va_free = va_full + NVA;
-  uint64_t* w_full = va_free + NVA;
-  uint64_t* u_full = w_full + 2;
-  uint64_t* u_free = u_full + 2;
+  uint64_t* zempty = zfull + 2 * kMaxNSZ;
+  uint64_t* va_full = zempty + kMaxNSZ;
+  uint64_t* w_full = va_full + NVA;
+  uint64_t* p2_done = w_full + NVA;       // product 2 of a slot's chunk has completed
+  uint64_t* u_free = p2_done + NVA;
   uint64_t* a_ready = u_free + 2;
   uint64_t* a_free = a_ready + 1;
   uint64_t* fin = a_free + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 2);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t nunits = a.ntiles * a.spc;
   const int nch = a.nch, spc = a.spc;
+  const int64_t ntiles = a.p.ntiles, nunits = ntiles * spc;
 
   if (tid == 0) {
     for (int s = 0; s < NSV; ++s) {
       mbar_init(&vfull[s], 1);
       mbar_init(&vempty[s], 1);
     }
-    for (int s = 0; s < NSZ; ++s) {
-      mbar_init(&zfull[s], 1);
-      mbar_init(&zempty[s], NEPI);
+    for (int s = 0; s < nsz; ++s) {
+      mbar_init(&zfull[2 * s], 1);
+      mbar_init(&zfull[2 * s + 1], 1);
+      mbar_init(&zempty[s], 1);
     }
     for (int i = 0; i < NVA; ++i) {
       mbar_init(&va_full[i], 1);
-      mbar_init(&va_free[i], NEPI);
+      mbar_init(&w_full[i], 4);
+      mbar_init(&p2_done[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&w_full[i], NEPI);
-      mbar_init(&u_full[i], 1);
-      mbar_init(&u_free[i], NEPI);
+      mbar_init(&u_free[i], 4);
     }
-    mbar_init(a_ready, NEPI);
+    mbar_init(a_ready, 4 * NG);
     mbar_init(a_free, 1);
-    mbar_init(fin, 1);
+    mbar_init(&fin[0], 1);
+    mbar_init(&fin[1], 1);
     mbar_fence_init();
+  }
+  if (tid < 32) zero_row[tid] = 0.f;
+  if (tid < RP) {
+    cAW[tid] = a.coefA[tid];
+    cAW[RP + tid] = a.coefW[tid];
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -333,28 +354,16 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
   bool failed = false;
   float s1 = 0.f, s2 = 0.f, s3 = 0.f;
 
-  const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
-  const int64_t plane = (int64_t)nx * ny;
-  // neighbour rows beyond x: -nx, +nx, -nx*ny, +nx*ny (the y pair first when there is one)
-  const int64_t off[4] = {ny > 1 ? -(int64_t)nx : -plane, ny > 1 ? (int64_t)nx : plane, -plane,
-                          plane};
-  // unit u = (segment s, tile t), segment-major: the CTAs running together hold the
-  // same chunks of consecutive tiles, so the neighbour rows they stage are L2 hits
-  auto unit_of = [&](int64_t u, int64_t& tile, int& c0, int& c1, int& sg) {
-    sg = (int)(u / a.ntiles);
-    tile = u - (int64_t)sg * a.ntiles;
-    c0 = (int)((int64_t)sg * nch / spc);
-    c1 = (int)((int64_t)(sg + 1) * nch / spc);
-  };
   // the k-th unit of this CTA. Main/tail layout (a.split > 0, fewer tiles than CTAs but
   // more than half as many): CTA j < ntiles owns chunks [0, split) of tile j; the other
   // CTAs take the tails [split, nch) of tiles j - ntiles, j - ntiles + (G - ntiles), ...
   // (concurrent tails are of consecutive tiles too). Otherwise units are dealt
-  // round-robin in segment-major order.
+  // round-robin in segment-major order, so that the CTAs running together hold the same
+  // chunks of consecutive tiles.
   auto unit_at = [&](int k, int64_t& tile, int& c0, int& c1, int& sg) -> bool {
     if (a.split > 0) {
       const int64_t j = blockIdx.x, G = gridDim.x;
-      if (j < a.ntiles) {
+      if (j < ntiles) {
         if (k > 0) return false;
         tile = j;
         sg = 0;
@@ -362,8 +371,8 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
         c1 = a.split;
         return true;
       }
-      tile = j - a.ntiles + (int64_t)k * (G - a.ntiles);
-      if (tile >= a.ntiles) return false;
+      tile = j - ntiles + (int64_t)k * (G - ntiles);
+      if (tile >= ntiles) return false;
       sg = 1;
       c0 = a.split;
       c1 = nch;
@@ -371,103 +380,86 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
     }
     const int64_t u = blockIdx.x + (int64_t)k * gridDim.x;
     if (u >= nunits) return false;
-    unit_of(u, tile, c0, c1, sg);
+    sg = (int)(u / ntiles);
+    tile = u - (int64_t)sg * ntiles;
+    c0 = (int)((int64_t)sg * nch / spc);
+    c1 = (int)((int64_t)(sg + 1) * nch / spc);
     return true;
+  };
+  // first voxel of a tile
+  auto origin = [&](int64_t tile, int& x0, int& y0, int& z0) {
+    const unsigned t = (unsigned)tile, tx = (unsigned)a.p.tx, ty = (unsigned)a.p.ty;
+    x0 = (int)(t % tx) * a.p.bx;
+    y0 = (int)(t / tx % ty) * a.p.by;
+    z0 = (int)(t / tx / ty) * a.p.bz;
   };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch_map(&maps.zc);
-      tma_prefetch_map(&maps.zn);
+      tma_prefetch_map(&maps.zi);
+      tma_prefetch_map(&maps.zp);
       tma_prefetch_map(&maps.v1h);
       tma_prefetch_map(&maps.v2h);
-      if (CHECK) tma_prefetch_map(&maps.dd);
+      const unsigned zbytes = (unsigned)a.p.rows * 128u +
+                              (CHECK ? (unsigned)(a.p.bx * a.p.by * a.p.bz) * 128u : 0u);
       int g = 0;
       int64_t tile;
       int c0, c1, sg;
       for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k) {
-        const int64_t n0 = tile * TV;
-        // the tile's own z rows come from HBM: they are prefetched into L2 kPrefetch chunks
-        // ahead of their staged loads, so that enough bytes are in flight per SM (the
-        // staged loads and the neighbour rows, which other CTAs prefetched, hit L2)
+        int x0, y0, z0;
+        origin(tile, x0, y0, z0);
+        // the tile's own rows come from HBM: they are prefetched into L2 kPrefetch chunks
+        // ahead of the stages, so that enough bytes are in flight per SM (the halo rows are
+        // prefetched by the CTAs that own them)
         for (int c = c0 + 1; c < c0 + kPrefetch && c < c1; ++c)
-          tma_prefetch_2d(&maps.zc, (int)(n0 - 4), c * QC);
-        // a residual test also reads d^k, element by element in the epilogue: its rows
-        // are prefetched into L2 the same way (the first kPrefetch chunks at once)
-        if (CHECK)
-          for (int c = c0; c < c0 + kPrefetch && c < c1; ++c)
-            tma_prefetch_2d(&maps.dd, (int)n0, c * QC);
+          tma_prefetch_5d(&maps.zp, 0, x0, y0, z0, c);
         for (int c = c0; c < c1; ++c, ++g) {
-          const int q0 = c * QC;
-          if (c + kPrefetch < c1) tma_prefetch_2d(&maps.zc, (int)(n0 - 4), q0 + kPrefetch * QC);
-          if (CHECK && c + kPrefetch < c1)
-            tma_prefetch_2d(&maps.dd, (int)n0, q0 + kPrefetch * QC);
-          // the chunk's V boxes (product 1 needs them first)
-          const int sv = g % NSV, kv = g / NSV;
-          if (kv > 0 && !mbar_wait_sleep(&vempty[sv], (kv - 1) & 1)) {
+          if (c + kPrefetch < c1) tma_prefetch_5d(&maps.zp, 0, x0, y0, z0, c + kPrefetch);
+          const int sz = g % nsz, kz = g / nsz;
+          if (kz > 0 && !mbar_wait_sleep(&zempty[sz], (kz - 1) & 1)) {
             failed = true;
+            break;
+          }
+          // a stage's loads complete on two barriers in turn: with an odd number of stages
+          // the groups alternate on a stage, and a group waiting for its load must not take
+          // the one before last (of the same parity on a single barrier) for it
+          unsigned char* zs = zring + sz * zst;
+          uint64_t* bar = &zfull[2 * sz + (kz & 1)];
+          mbar_arrive_expect_tx(bar, zbytes);
+          tma_load_5d(zs, &maps.zi, 0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, c, bar);
+          if (CHECK) tma_load_5d(zs + a.p.zst, &maps.di, 0, x0, y0, z0, c, bar);
+          const int sv = g % NSV, kv = g / NSV, q0 = c * QC;
+          uint64_t* ve = NSV == NVA ? &p2_done[sv] : &vempty[sv];
+          if (kv > 0 && !mbar_wait_sleep(ve, (kv - 1) & 1)) {
+            failed = true;
+            ++g;          // the z copies of this chunk were issued
             break;
           }
           unsigned char* vs = vring + sv * L::VST;
-          mbar_arrive_expect_tx(&vfull[sv], L::VBYTES);
+          mbar_arrive_expect_tx(&vfull[sv], (unsigned)L::VST);
 #pragma unroll
           for (int at = 0; at < RP / 32; ++at) {
-            tma_load_2d(vs + L::v1h + at * QC * 128, &maps.v1h, at * 32, q0, &vfull[sv]);
-            tma_load_2d(vs + L::v1l + at * QC * 128, &maps.v1l, at * 32, q0, &vfull[sv]);
+            tma_load_2d(vs + L::v1(at, 0), &maps.v1h, at * 32, q0, &vfull[sv]);
+            tma_load_2d(vs + L::v1(at, 1), &maps.v1l, at * 32, q0, &vfull[sv]);
           }
           tma_load_2d(vs + L::v2h, &maps.v2h, q0, 0, &vfull[sv]);
           tma_load_2d(vs + L::v2l, &maps.v2l, q0, 0, &vfull[sv]);
-          // z with its x halo and the neighbour rows
-          const int sz = g % NSZ, kz = g / NSZ;
-          if (kz > 0 && !mbar_wait_sleep(&zempty[sz], (kz - 1) & 1)) {
-            failed = true;
-            ++g;          // the V copies of this chunk were issued
-            break;
-          }
-          unsigned char* zs = zring + sz * L::ZST;
-          mbar_arrive_expect_tx(&zfull[sz], L::ZBYTES);
-          tma_load_2d(zs + L::zc, &maps.zc, (int)(n0 - 4), q0, &zfull[sz]);
-#pragma unroll
-          for (int j = 0; j < NR; ++j)
-            tma_load_2d(zs + L::zn + j * QC * NW * 4, &maps.zn, (int)floor4(n0 + off[j]), q0,
-                        &zfull[sz]);
         }
       }
       // no copy may still be in flight when the CTA exits: wait (bounded) for the last
       // phase issued into every stage
       for (int s = 0; s < NSV && s < g; ++s)
         mbar_wait_sleep(&vfull[s], ((s + ((g - 1 - s) / NSV) * NSV) / NSV) & 1);
-      for (int s = 0; s < NSZ && s < g; ++s)
-        mbar_wait_sleep(&zfull[s], ((s + ((g - 1 - s) / NSZ) * NSZ) / NSZ) & 1);
+      for (int s = 0; s < nsz && s < g; ++s) {
+        const int kz = (g - 1 - s) / nsz;            // the stage's last round
+        mbar_wait_sleep(&zfull[2 * s + (kz & 1)], (kz >> 1) & 1);
+      }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
+    // ------------------------------------------------------------------ product 1
     if (lane == 0) {
       const uint32_t a_hi = tmem + L::T_A, a_lo = tmem + L::T_A + RP;
-      // product 2 of chunk gg: U (main, correction) = w (hi, lo) . V_c (hi, lo)
-      auto product2 = [&](int gg) {
-        const int p = gg & 1;
-        if (!failed && !mbar_wait_sleep(&w_full[p], (gg >> 1) & 1)) failed = true;
-        // the U buffer is free once the epilogue has read chunk gg - UB's
-        const int gp = gg - UB;
-        if (!failed && gp >= 0 && !mbar_wait_sleep(&u_free[gp & 1], (gp >> 1) & 1))
-          failed = true;
-        if (failed) return;
-        fence_after();
-        const uint32_t vs = smem_u32(vring + (gg % NSV) * L::VST);
-        const uint32_t dm = tmem + L::T_U + 2 * RP * (gg % UB), dc = dm + RP;
-        const uint32_t w_hi = tmem + L::T_W + 64 * p, w_lo = w_hi + 32;
-#pragma unroll
-        for (int k = 0; k < QC / 8; ++k) {
-          const uint64_t bh = sdesc(vs + L::v2h + k * 32), bl = sdesc(vs + L::v2l + k * 32);
-          mma_tf32(dm, w_hi + 8 * k, bh, L::IDESC2, k > 0 ? 1u : 0u);
-          mma_tf32(dc, w_hi + 8 * k, bl, L::IDESC2, k > 0 ? 1u : 0u);
-          mma_tf32(dc, w_lo + 8 * k, bh, L::IDESC2, 1u);
-        }
-        commit(&u_full[p]);
-        commit(&vempty[gg % NSV]);    // the V stage is free once these complete
-      };
       int g = 0, si = 0;
       int64_t tile;
       int c0, c1, sg;
@@ -478,11 +470,12 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
           break;
         }
         fence_after();
-        for (int i = 0; i < nchk && !failed; ++i) {
-          // product 1 of chunk gg: V a (main, correction) = a (hi, lo) . V_c^T (hi, lo)
+        for (int i = 0; i < nchk; ++i) {
+          // V a (main, correction) of chunk gg: a_hi . [V_hi | V_lo]^T into both, then
+          // a_lo . V_hi^T into the correction; its slot's previous w has been read
           const int gg = g + i, b = gg % NVA;
           if (!mbar_wait_sleep(&vfull[gg % NSV], (gg / NSV) & 1)) failed = true;
-          if (!failed && gg >= NVA && !mbar_wait_sleep(&va_free[b], ((gg / NVA) - 1) & 1))
+          if (!failed && gg >= NVA && !mbar_wait_sleep(&p2_done[b], (gg / NVA - 1) & 1))
             failed = true;
           if (failed) break;
           fence_after();
@@ -490,294 +483,380 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
           const uint32_t dm = tmem + L::T_VA + 64 * b, dc = dm + 32;
           // the padding ranks beyond r carry zero a: their K steps are skipped
 #pragma unroll 4
-          for (int k = 0; k < a.kr; ++k) {
-            const int at = k / 4, o = (k % 4) * 32;
-            const uint64_t bh = sdesc(vs + L::v1h + at * QC * 128 + o);
-            const uint64_t bl = sdesc(vs + L::v1l + at * QC * 128 + o);
-            mma_tf32(dm, a_hi + 8 * k, bh, L::IDESC1, k > 0 ? 1u : 0u);
-            mma_tf32(dc, a_hi + 8 * k, bl, L::IDESC1, k > 0 ? 1u : 0u);
-            mma_tf32(dc, a_lo + 8 * k, bh, L::IDESC1, 1u);
+          for (int k8 = 0; k8 < a.kr; ++k8) {
+            const uint64_t bh = sdesc(vs + L::v1(k8 / 4, 0) + (k8 % 4) * 32);
+            mma_tf32(dm, a_hi + 8 * k8, bh, L::idesc(2 * QC), k8 > 0 ? 1u : 0u);
+            mma_tf32(dc, a_lo + 8 * k8, bh, L::idesc(QC), 1u);
           }
           commit(&va_full[b]);
           if (i == nchk - 1) commit(a_free);     // a may be rewritten once these complete
-          if (i >= D1) product2(gg - D1);
         }
-        // the segment's last products 2
-        for (int j = (nchk > D1 ? nchk - D1 : 0); j < nchk && !failed; ++j) product2(g + j);
         g += nchk;
         ++si;
       }
       // every product issued has completed before the TMEM is freed
-      commit(fin);
-      mbar_wait_sleep(fin, 0);
+      commit(&fin[0]);
+      mbar_wait_sleep(&fin[0], 0);
     }
-  } else {
+  } else if (warp == 2) {
+    // ------------------------------------------------------------------ product 2
+    if (lane == 0) {
+      int g = 0;
+      int64_t tile;
+      int c0, c1, sg;
+      for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k) {
+        for (int c = c0; c < c1; ++c, ++g) {
+          // U (main, correction) of chunk g: w_hi . [V_hi | V_lo] into both, then w_lo . V_hi
+          // into the correction
+          const int b = g % NVA, gp = g - UB;
+          if (!mbar_wait_sleep(&vfull[g % NSV], (g / NSV) & 1)) failed = true;
+          if (!failed && !mbar_wait_sleep(&w_full[b], (g / NVA) & 1)) failed = true;
+          // the U buffer is free once the epilogue has read chunk g - UB's
+          if (!failed && gp >= 0 && !mbar_wait_sleep(&u_free[gp & 1], (gp >> 1) & 1))
+            failed = true;
+          if (failed) break;
+          fence_after();
+          const uint32_t vs = smem_u32(vring + (g % NSV) * L::VST);
+          const uint32_t dm = tmem + L::T_U + 2 * RP * (g % UB), dc = dm + RP;
+          const uint32_t w_hi = tmem + L::T_VA + 64 * b, w_lo = w_hi + 32;
+#pragma unroll
+          for (int k8 = 0; k8 < QC / 8; ++k8) {
+            const uint64_t bh = sdesc(vs + L::v2h + k8 * 32);
+            mma_tf32(dm, w_hi + 8 * k8, bh, L::idesc(2 * RP), k8 > 0 ? 1u : 0u);
+            mma_tf32(dc, w_lo + 8 * k8, bh, L::idesc(RP), 1u);
+          }
+          commit(&p2_done[b]);
+          if (NSV != NVA) commit(&vempty[g % NSV]);   // the V stage is free too
+        }
+      }
+      commit(&fin[1]);
+      mbar_wait_sleep(&fin[1], 0);
+    }
+  } else if (warp >= 4) {
     // ------------------------------------------------------------------ epilogue warps
     const int quarter = warp & 3;
-    const int grp = (warp - 2) >> 2;                 // compartments grp*GC .. of a chunk
-    const int v = quarter * 32 + lane;               // voxel within the tile = TMEM lane
+    const int grp = (warp - 4) >> 2;                 // takes the chunks gg with gg % NG == grp
+    const int v = quarter * 32 + lane;               // lane of the tile = TMEM lane
+    const bool storer = quarter == 0 && lane == 0;   // issues the group's TMA stores
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-    const int64_t ld = a.g.ld, N = a.g.N;
-    const int Q = a.Q;
+    const int64_t ld = a.g.ld;
+    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
+    const int64_t plane = (int64_t)nx * ny;
     const bool zl = nz > 1 && a.g.zlink;
     const float c2 = a.lam_s * a.inv_xb;             // weight of the neighbour sum
     const float c3 = a.beta * a.inv_xb;              // weight of V a
-    const float beta = a.beta, inv_beta = a.inv_beta;
+    const float beta = a.beta;
     const float2 c2_2 = make_float2(c2, c2), c3_2 = make_float2(c3, c3);
     const float2 beta2 = make_float2(beta, beta), two2 = make_float2(2.f, 2.f);
-    int g = 0, si = 0;
-    int64_t tile;
-    int c0, c1, sg;
-    for (int k = 0; unit_at(k, tile, c0, c1, sg); ++k) {
-      const int nchk = c1 - c0;
-      const int64_t n0 = tile * TV;
-      const int64_t n = n0 + v;
-      const bool valid = n < N;
-      // voxel coordinates in 32-bit arithmetic (N < 2^31)
-      int x = 0, y = 0, zc = 0;
-      if (valid) {
-        const unsigned nn = (unsigned)n, t = nn / (unsigned)nx;
-        x = (int)(nn - t * (unsigned)nx);
-        y = (int)(t % (unsigned)ny);
-        zc = (int)(t / (unsigned)ny);
+    // this lane's voxel within a patch, and its row among the staged rows (swizzled: the
+    // 16-byte piece j of row r sits at piece j ^ (r & 7))
+    const int lx = v % a.p.bx, ly = v / a.p.bx % a.p.by, lz = v / (a.p.bx * a.p.by);
+    const bool used = lz < a.p.bz;
+    auto srow = [](int r) { return (uint32_t)(r * 128 + ((r & 7) << 4)); };
+    const int r0 = ((lz + a.p.hz) * a.p.Y + ly + a.p.hy) * a.p.X + lx + a.p.hx;
+    uint32_t ro[1 + 2 * NAX];                        // own row, then minus / plus per axis
+    ro[0] = srow(r0);
+    {
+      // strides of the axes with smoothness, in the order x, y, z
+      int st[3] = {0, 0, 0}, k = 0;
+      if (a.p.hx) st[k++] = 1;
+      if (a.p.hy) st[k++] = a.p.X;
+      if (a.p.hz) st[k++] = a.p.X * a.p.Y;
+#pragma unroll
+      for (int i = 0; i < NAX; ++i) {
+        ro[1 + 2 * i] = srow(r0 - st[i]);
+        ro[2 + 2 * i] = srow(r0 + st[i]);
       }
+    }
+    const uint32_t vrow = srow(v);                   // own row of an unhaloed buffer
+    const uint32_t zero = smem_u32(zero_row), ring = smem_u32(zring);
+    const uint32_t ob0 = smem_u32(obuf) + grp * nob * OB;
+
+    int64_t tile = 0, n = 0;
+    int c0 = 0, c1 = 0, sg = 0;
+    bool in = false;
+    float e1 = 0.f;
+    float us[RQ], sv[RQ];
+    // unit k: its voxel, and the loads of its a-vector (S and the u slots of the previous
+    // iteration, in slot order)
+    auto begin = [&](int k) -> bool {
+      if (!unit_at(k, tile, c0, c1, sg)) return false;
+      int x0, y0, z0;
+      origin(tile, x0, y0, z0);
+      const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+      const bool valid = used && x < nx && y < ny && z < nz;
+      n = valid ? x + (int64_t)nx * (y + (int64_t)ny * z) : 0;
       // a voxel outside the object is left alone (its z stays 0) and is nobody's neighbour
       const uint8_t* mk = a.mask;
-      const bool in = valid && (!mk || mk[n]);
-      const bool hxm = in && x > 0 && (!mk || mk[n - 1]);
-      const bool hxp = in && x < nx - 1 && (!mk || mk[n + 1]);
-      const bool hym = in && y > 0 && (!mk || mk[n - nx]);
-      const bool hyp = in && y < ny - 1 && (!mk || mk[n + nx]);
-      const bool hzm = zl && in && zc > 0 && (!mk || mk[n - plane]);
-      const bool hzp = zl && in && zc < nz - 1 && (!mk || mk[n + plane]);
-      const float deg = (float)(hxm + hxp + hym + hyp + hzm + hzp);
-      const float e1 = (a.xi + a.beta - a.lam_s * deg) * a.inv_xb;   // weight of z
-      // neighbour presence as 0/1 weights: the staged rows are always readable (finite
-      // z values or the copy's zero fill), so every neighbour term is a fused add
-      const float fxm = hxm ? 1.f : 0.f, fxp = hxp ? 1.f : 0.f;
-      const float2 fxm2 = make_float2(fxm, fxm), fxp2 = make_float2(fxp, fxp);
-      const float2 e1_2 = make_float2(e1, e1);
-      int nidx[4];
-      float fk[4];
-      {
-        const bool flags[4] = {ny > 1 ? hym : hzm, ny > 1 ? hyp : hzp, hzm, hzp};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          nidx[j] = j < NR ? (int)(n + off[j] - floor4(n0 + off[j])) : 0;
-          fk[j] = (j < NR && flags[j]) ? 1.f : 0.f;
-        }
+      in = valid && (!mk || mk[n]);
+      int deg = 0;
+      if (in) {
+        deg = (x > 0 && (!mk || mk[n - 1])) + (x < nx - 1 && (!mk || mk[n + 1])) +
+              (y > 0 && (!mk || mk[n - nx])) + (y < ny - 1 && (!mk || mk[n + nx]));
+        if (zl)
+          deg += (z > 0 && (!mk || mk[n - plane])) + (z < nz - 1 && (!mk || mk[n + plane]));
       }
-      float2 fk2[4];
+      e1 = (a.xi + a.beta - a.lam_s * (float)deg) * a.inv_xb;   // weight of z
+      const float* pt = a.Pin + tile * spc * (int64_t)(RP * TV) + grp * RQ * TV + v;
+      const float* sp = a.S + (int64_t)(grp * RQ) * ld + n;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) fk2[j] = make_float2(fk[j], fk[j]);
-      // a for this warp's ranks: a_i = S_i/(beta + sigma_i^2) - W_i u_i, u_i summed over
-      // the tile's segment slots of the previous iteration in segment order
+      for (int i = 0; i < RQ; ++i) {
+        sv[i] = in ? __ldg(sp + i * ld) : 0.f;
+        us[i] = pt[i * TV];
+      }
+      // (SB slots' loads in flight together; a slot past the last reads the last with weight 0)
+      constexpr int SB = RQ <= 16 ? 3 : 1;
+#pragma unroll 1
+      for (int s = 1; s < spc; s += SB) {
+        float u1[SB][RQ];
+#pragma unroll
+        for (int t = 0; t < SB; ++t)
+#pragma unroll
+          for (int i = 0; i < RQ; ++i) u1[t][i] = pt[(min(s + t, spc - 1) * RP + i) * TV];
+#pragma unroll
+        for (int t = 0; t < SB; ++t)
+#pragma unroll
+          for (int i = 0; i < RQ; ++i) us[i] += s + t < spc ? u1[t][i] : 0.f;
+      }
+      return true;
+    };
+    int g = 0, si = 0, own = 0;                      // own: chunks this group has processed
+    bool more = begin(0);
+    for (int k = 0; more; ++k) {
+      const int nchk = c1 - c0;
+      // a_i = S_i/(beta + sigma_i^2) - W_i u_i for this group's ranks
       if (si > 0 && !failed && !mbar_wait_sleep(a_free, (si - 1) & 1)) failed = true;
       fence_after();
-      {
-        float ah[RQ], al[RQ];
-        const float* pt = a.Pin + (tile * spc) * (int64_t)(RP * TV) + grp * RQ * TV + v;
-        const float* sp = a.S + (int64_t)(grp * RQ) * ld + n;
-        // every load of the a-vector is issued before any is used
-        float us[RQ], sv[RQ];
 #pragma unroll
-        for (int i = 0; i < RQ; ++i) {
-          sv[i] = in ? __ldg(sp + i * ld) : 0.f;
-          us[i] = in ? pt[i * TV] : 0.f;
-        }
-        for (int k = 1; k < spc; ++k) {
+      for (int i = 0; i < RQ; i += 8) {
+        float ah[8], al[8];
 #pragma unroll
-          for (int i = 0; i < RQ; ++i) us[i] += in ? pt[(k * RP + i) * TV] : 0.f;
+        for (int j = 0; j < 8; ++j) {
+          const int r = grp * RQ + i + j;
+          const float av = in ? sv[i + j] * cAW[r] - cAW[RP + r] * us[i + j] : 0.f;
+          ah[j] = tf32_rna(av);
+          al[j] = tf32_rna(av - ah[j]);
         }
-#pragma unroll
-        for (int i = 0; i < RQ; ++i) {
-          const int r = grp * RQ + i;
-          const float av = in ? sv[i] * __ldg(a.coefA + r) - __ldg(a.coefW + r) * us[i] : 0.f;
-          ah[i] = tf32_rna(av);
-          al[i] = tf32_rna(av - ah[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < RQ; i += 8) {
-          tst8(tmem + lane_base + L::T_A + grp * RQ + i, ah + i);
-          tst8(tmem + lane_base + L::T_A + RP + grp * RQ + i, al + i);
-        }
-        tst_wait();
+        tst8(tmem + lane_base + L::T_A + grp * RQ + i, ah);
+        tst8(tmem + lane_base + L::T_A + RP + grp * RQ + i, al);
       }
+      tst_wait();
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(a_ready);
-      float uacc[RQ];
+      // lanes outside the object read zeros for every row, so that their z', w and d' are 0
+      uint32_t rr[1 + 2 * NAX];
 #pragma unroll
-      for (int i = 0; i < RQ; ++i) uacc[i] = 0.f;
+      for (int i = 0; i < 1 + 2 * NAX; ++i) rr[i] = in ? ro[i] : 0u;
+      const uint32_t dro = in ? vrow : 0u;
+      const float2 e1_2 = make_float2(e1, e1);
+      float uacc[RP];
+#pragma unroll
+      for (int i = 0; i < RP; ++i) uacc[i] = 0.f;
       // product 2's sums of chunk gg (main + correction, rounded to nearest in registers)
       auto consume_u = [&](int gg) {
-        const int p = gg & 1;
-        if (!failed && !mbar_wait_sleep(&u_full[p], (gg >> 1) & 1)) failed = true;
+        if (!failed && !mbar_wait_sleep(&p2_done[gg % NVA], (gg / NVA) & 1)) failed = true;
         fence_after();
-        const uint32_t ub = tmem + lane_base + L::T_U + 2 * RP * (gg % UB) + grp * RQ;
-        {
-          float um[RQ], uc[RQ];
-          tld2_cols<RQ>(ub, ub + RP, um, uc);
+        const uint32_t ub = tmem + lane_base + L::T_U + 2 * RP * (gg % UB);
 #pragma unroll
-          for (int j = 0; j < RQ; j += 2) {
-            const float2 t2 = __fadd2_rn(make_float2(um[j], um[j + 1]), make_float2(uc[j], uc[j + 1]));
-            const float2 s2 = __fadd2_rn(make_float2(uacc[j], uacc[j + 1]), t2);
-            uacc[j] = s2.x;
-            uacc[j + 1] = s2.y;
+        for (int j0 = 0; j0 < RP; j0 += 16) {
+          uint32_t um[32];
+          tld<16>(ub + j0, um);
+          tld<16>(ub + RP + j0, um + 16);
+          tld_wait<32>(um);
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            const float2 t2 = __fadd2_rn(
+                make_float2(__uint_as_float(um[j]), __uint_as_float(um[j + 1])),
+                make_float2(__uint_as_float(um[16 + j]), __uint_as_float(um[17 + j])));
+            const float2 s2 = __fadd2_rn(make_float2(uacc[j0 + j], uacc[j0 + j + 1]), t2);
+            uacc[j0 + j] = s2.x;
+            uacc[j0 + j + 1] = s2.y;
           }
         }
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&u_free[p]);
+        if (lane == 0) mbar_arrive(&u_free[gg & 1]);
       };
-      for (int i = 0; i < nchk; ++i) {
-        const int gg = g + i, sz = gg % NSZ, b = gg % NVA, p = gg & 1;
-        const int qg = (c0 + i) * QC + grp * GC;   // this warp's first compartment
-        // a residual test needs d^k, read from global memory element by element: the
-        // chunk's loads are issued before the waits, so that their latency overlaps the
-        // chunk's processing (loading them where they are used cost 2.7x per iteration)
-        float dkc[CHECK ? GC : 1];
-        if constexpr (CHECK) {
-          const int jn0 = min(GC, Q - qg);
-          const float* dq = a.Din + (int64_t)qg * ld + n;
-#pragma unroll
-          for (int j = 0; j < GC; ++j) dkc[j] = (in && j < jn0) ? __ldg(dq + j * ld) : 0.f;
-        }
-        if (!failed && !mbar_wait_sleep(&zfull[sz], (gg / NSZ) & 1)) failed = true;
+      int x0, y0, z0;
+      origin(tile, x0, y0, z0);
+      int pend = -1;                                 // own chunk whose u is not yet summed
+#pragma unroll 1
+      for (int i = (g ^ grp) & 1; i < nchk; i += NG) {
+        const int gg = g + i, sz = gg % nsz, b = gg % NVA;
+        const int kz = gg / nsz;
+        if (!failed && !mbar_wait_sleep(&zfull[2 * sz + (kz & 1)], (kz >> 1) & 1)) failed = true;
         if (!failed && !mbar_wait_sleep(&va_full[b], (gg / NVA) & 1)) failed = true;
         fence_after();
-        float va[GC];
-        {
-          float vc[GC];
-          const uint32_t tb = tmem + lane_base + L::T_VA + 64 * b + grp * GC;
-          tld2_cols<GC>(tb, tb + 32, va, vc);
-#pragma unroll
-          for (int k = 0; k < GC; k += 2) {
-            const float2 s2 = __fadd2_rn(make_float2(va[k], va[k + 1]), make_float2(vc[k], vc[k + 1]));
-            va[k] = s2.x;
-            va[k + 1] = s2.y;
-          }
+        const uint32_t tb = tmem + lane_base + L::T_VA + 64 * b;
+        uint32_t vr[16];
+        tld<8>(tb, vr);
+        tld<8>(tb + 32, vr + 8);
+        if (nob == 1) {
+          // the group's single buffer: the previous store has read it
+          if (storer) bulk_wait_read();
+          __syncwarp();
+          group_barrier(1 + grp);
         }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&va_free[b]);
-        const bool work = in && !failed;
-        const int jn = min(GC, Q - qg);              // the same for every lane
-        const float* zcr = reinterpret_cast<const float*>(zring + sz * L::ZST + L::zc) +
-                           grp * GC * ZW + 4 + v;
-        const float* znr = reinterpret_cast<const float*>(zring + sz * L::ZST + L::zn) +
-                           grp * GC * NW;
-        float w[GC];
-        float* zp = a.Zout + (int64_t)qg * ld + n;
-        if (work) {
-          // in halves of 8 compartments: the staged rows first (all shared-memory loads of
-          // the half in flight at once, before any store to global memory), then the
-          // arithmetic, then the stores
+        const uint32_t zb = in ? ring + sz * zst : zero;
+        const uint32_t db = in ? ring + sz * zst + a.p.zst : zero;
+        const uint32_t ob = ob0 + (nob == 2 ? (own & 1) * OB : 0) + vrow;
 #pragma unroll
-          for (int h = 0; h < GC; h += 8) {
-            // compartments in pairs, in packed FP32x2 arithmetic: each half of an FP32x2
-            // operation rounds as the scalar one, so the values are those of scalar code
-            float2 zz2[4], nb2[4];
+        for (int sb = 0; sb < 4; ++sb) {
+          // 8 compartments: V a (the next 8's TMEM loads issued ahead), the staged rows, the
+          // z-step and dual step in packed FP32x2 arithmetic (each half rounds as the scalar
+          // operation)
+          tld_wait<16>(vr);
+          float2 va2[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int r = h + 2 * j;
-              zz2[j] = make_float2(zcr[r * ZW], zcr[(r + 1) * ZW]);
-              nb2[j] = __fmul2_rn(fxm2, make_float2(zcr[r * ZW - 1], zcr[(r + 1) * ZW - 1]));
-              nb2[j] = __ffma2_rn(fxp2, make_float2(zcr[r * ZW + 1], zcr[(r + 1) * ZW + 1]), nb2[j]);
+          for (int j = 0; j < 4; ++j)
+            va2[j] = __fadd2_rn(
+                make_float2(__uint_as_float(vr[2 * j]), __uint_as_float(vr[2 * j + 1])),
+                make_float2(__uint_as_float(vr[8 + 2 * j]), __uint_as_float(vr[9 + 2 * j])));
+          if (sb < 3) {
+            tld<8>(tb + 8 * (sb + 1), vr);
+            tld<8>(tb + 32 + 8 * (sb + 1), vr + 8);
+          }
+          float4 zz[2], nb[2 * NAX][2];
 #pragma unroll
-              for (int k = 0; k < NR; ++k)
-                nb2[j] = __ffma2_rn(fk2[k],
-                                    make_float2(znr[(k * QC + r) * NW + nidx[k]],
-                                                znr[(k * QC + r + 1) * NW + nidx[k]]),
-                                    nb2[j]);
-            }
-            float zz[8], zn[8], tt[8];
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
+            zz[h] = lds4(zb + (rr[0] ^ jx));
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int r = h + 2 * j;
-              const float2 va2 = make_float2(va[r], va[r + 1]);
-              const float2 y = __ffma2_rn(e1_2, zz2[j], __ffma2_rn(c2_2, nb2[j], __fmul2_rn(c3_2, va2)));
-              const float2 z2 = make_float2(fmaxf(0.f, y.x), fmaxf(0.f, y.y));
-              const float2 t2 = __fadd2_rn(zz2[j], va2);
-              const float2 w2 =
-                  __fmul2_rn(beta2, __ffma2_rn(two2, z2, make_float2(-t2.x, -t2.y)));
-              zz[2 * j] = zz2[j].x;
-              zz[2 * j + 1] = zz2[j].y;
-              zn[2 * j] = z2.x;
-              zn[2 * j + 1] = z2.y;
-              tt[2 * j] = t2.x;
-              tt[2 * j + 1] = t2.y;
-              // compartments past Q read the copies' zero fill (z) and zero rows of V
-              // (V a): their w is exactly 0 without a test
-              w[r] = w2.x;
-              w[r + 1] = w2.y;
+            for (int q = 0; q < 2 * NAX; ++q) nb[q][h] = lds4(zb + (rr[1 + q] ^ jx));
+          }
+          float zn[8], w[8];
+          float4 dk[2];
+          if constexpr (CHECK) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) dk[h] = lds4(db + (dro ^ ((uint32_t)(2 * sb + h) << 4)));
+          }
+          float dn[8];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int h = j >> 1;
+            auto pr = [&](const float4& f) {
+              return (j & 1) ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
+            };
+            const float2 z2 = pr(zz[h]);
+            float2 s = __fadd2_rn(pr(nb[0][h]), pr(nb[1][h]));
+#pragma unroll
+            for (int q = 2; q < 2 * NAX; ++q) s = __fadd2_rn(s, pr(nb[q][h]));
+            const float2 y = __ffma2_rn(e1_2, z2, __ffma2_rn(c2_2, s, __fmul2_rn(c3_2, va2[j])));
+            const float2 n2 = make_float2(fmaxf(0.f, y.x), fmaxf(0.f, y.y));
+            const float2 t2 = __fadd2_rn(z2, va2[j]);
+            const float2 w2 = __fmul2_rn(beta2, __ffma2_rn(two2, n2, make_float2(-t2.x, -t2.y)));
+            zn[2 * j] = n2.x;
+            zn[2 * j + 1] = n2.y;
+            w[2 * j] = w2.x;
+            w[2 * j + 1] = w2.y;
+            if constexpr (WD) {
+              dn[2 * j] = beta * (t2.x - n2.x);
+              dn[2 * j + 1] = beta * (t2.y - n2.y);
             }
             if constexpr (CHECK) {
-              // f^{k+1} = t - d^k / beta needs d^k
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                if (h + j < jn) {
-                  const float f = tt[j] - dkc[h + j] * inv_beta;
-                  const float e = zn[j] - f, ch = zn[j] - zz[j];
-                  s1 = fmaf(e, e, s1);
-                  s2 = fmaf(ch, ch, s2);
-                  s3 = fmaf(zn[j], zn[j], s3);
-                }
-            }
-            if (jn == GC) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j) __stcs(zp + (h + j) * ld, zn[j]);
-              if constexpr (WD) {
-                float* dp = a.Dout + (zp - a.Zout);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) dp[(h + j) * ld] = beta * (tt[j] - zn[j]);
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 8; ++j)
-                if (h + j < jn) {
-                  zp[(h + j) * ld] = zn[j];
-                  if constexpr (WD) a.Dout[(zp - a.Zout) + (h + j) * ld] = beta * (tt[j] - zn[j]);
-                }
+              // f^{k+1} = t - d^k / beta
+              const float2 d2 = pr(dk[h]);
+              const float f0 = t2.x - d2.x * a.inv_beta, f1 = t2.y - d2.y * a.inv_beta;
+              const float ea = n2.x - f0, eb = n2.y - f1;
+              const float ca = n2.x - z2.x, cb = n2.y - z2.y;
+              s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
+              s2 = fmaf(cb, cb, fmaf(ca, ca, s2));
+              s3 = fmaf(n2.y, n2.y, fmaf(n2.x, n2.x, s3));
             }
           }
-        } else {
 #pragma unroll
-          for (int j = 0; j < GC; ++j) w[j] = 0.f;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&zempty[sz]);   // the staged rows are no longer read
-        // product 2 of chunk gg - 2 has completed (it read the w buffer about to be
-        // rewritten); its sums join the running u'
-        if (i >= 2) consume_u(gg - 2);
-#pragma unroll
-        for (int j = 0; j < GC; j += 8) {
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
+            sts4(ob ^ jx, zn[4 * h], zn[4 * h + 1], zn[4 * h + 2], zn[4 * h + 3]);
+            if constexpr (OWN_D)
+              sts4((ob + OUT_BYTES) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2], dn[4 * h + 3]);
+            else if constexpr (WD)
+              sts4((ring + sz * zst + a.p.zst + vrow) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2],
+                   dn[4 * h + 3]);
+          }
           float wh[8], wl[8];
 #pragma unroll
-          for (int k = 0; k < 8; k += 2) {
-            wh[k] = tf32_rna(w[j + k]);
-            wh[k + 1] = tf32_rna(w[j + k + 1]);
-            const float2 l2 = __fadd2_rn(make_float2(w[j + k], w[j + k + 1]),
-                                         make_float2(-wh[k], -wh[k + 1]));
-            wl[k] = tf32_rna(l2.x);
-            wl[k + 1] = tf32_rna(l2.y);
+          for (int j = 0; j < 8; j += 2) {
+            wh[j] = tf32_rna(w[j]);
+            wh[j + 1] = tf32_rna(w[j + 1]);
+            const float2 l2 =
+                __fadd2_rn(make_float2(w[j], w[j + 1]), make_float2(-wh[j], -wh[j + 1]));
+            wl[j] = tf32_rna(l2.x);
+            wl[j + 1] = tf32_rna(l2.y);
           }
-          tst8(tmem + lane_base + L::T_W + 64 * p + grp * GC + j, wh);
-          tst8(tmem + lane_base + L::T_W + 64 * p + 32 + grp * GC + j, wl);
+          tst8(tb + 8 * sb, wh);
+          tst8(tb + 32 + 8 * sb, wl);
+          // the sums of this group's previous chunk join the running u'
+          if (sb == 1 && pend >= 0) consume_u(pend);
         }
+        pend = gg;
         tst_wait();
         fence_before();
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(&w_full[p]);
+        if (lane == 0) mbar_arrive(&w_full[b]);
+        // the other buffer: its store (of the previous chunk) has read it, so the group may
+        // write it after the barrier
+        if (nob == 2 && storer) bulk_wait_read();
+        __syncwarp();
+        group_barrier(1 + grp);
+        if (storer) {
+          const unsigned char* ob_ = obuf + grp * nob * OB + (nob == 2 ? (own & 1) * OB : 0);
+          tma_store_5d(&maps.zo, ob_, 0, x0, y0, z0, c0 + i);
+          if constexpr (OWN_D)
+            tma_store_5d(&maps.dd, ob_ + OUT_BYTES, 0, x0, y0, z0, c0 + i);
+          else if constexpr (WD)
+            tma_store_5d(&maps.dd, zring + sz * zst + a.p.zst, 0, x0, y0, z0, c0 + i);
+          bulk_commit();
+          // the staged rows are no longer read (d' over the staged d^k is, by its store)
+          if constexpr (WD && CHECK) bulk_wait_read();
+          mbar_arrive(&zempty[sz]);
+        }
+        __syncwarp();
+        ++own;
       }
-      for (int j = (nchk > 2 ? nchk - 2 : 0); j < nchk; ++j) consume_u(g + j);
-      // this segment's partial u' (zero for voxels past the grid or outside the object)
-      float* po = a.Pout + ((tile * spc + sg) * (int64_t)RP) * TV;
+      // the next unit's loads go out before this one's last sums are waited for
+      float* po = a.Pout + (tile * spc + sg) * (int64_t)(RP * TV) + v;
+      const bool in0 = in;
+      const int gl = g + nchk - 1;                   // the unit's last chunk
+      more = begin(k + 1);
+      if (pend >= 0) consume_u(pend);
+      // the unit's partial u': the second group hands its sums over in the TMEM slot of its
+      // last chunk (read by product 2, and not written by product 1 before both groups have
+      // arrived for the next unit), the first adds and stores them (zero for lanes outside
+      // the grid or the object). A unit of one chunk has one group's sums only
+      if (nchk > 1) {
+        const uint32_t xt =
+            tmem + lane_base + L::T_VA + 64 * (((gl & 1) == 1 ? gl : gl - 1) % NVA);
+        if (grp == 1) {
 #pragma unroll
-      for (int i = 0; i < RQ; ++i) po[(grp * RQ + i) * TV + v] = in ? uacc[i] : 0.f;
+          for (int i = 0; i < RP; i += 8) tst8(xt + i, uacc + i);
+          tst_wait();
+          fence_before();
+          asm volatile("bar.arrive 3, 256;\n" ::: "memory");
+        } else {
+          asm volatile("bar.sync 3, 256;\n" ::: "memory");
+          fence_after();
+#pragma unroll
+          for (int j0 = 0; j0 < RP; j0 += 16) {
+            uint32_t x[16];
+            tld<16>(xt + j0, x);
+            tld_wait<16>(x);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) uacc[j0 + j] += __uint_as_float(x[j]);
+          }
+          fence_before();
+        }
+      }
+      if (nchk > 1 ? grp == 0 : (gl & 1) == grp) {
+#pragma unroll
+        for (int i = 0; i < RP; ++i) po[i * TV] = in0 ? uacc[i] : 0.f;
+      }
       g += nchk;
       ++si;
     }
+    if (storer) bulk_wait_all();
   }
   if (failed) atomicExch(a.err, (int)SSM_ETIMEOUT);
   if constexpr (CHECK) {
@@ -810,6 +889,39 @@ __global__ void __launch_bounds__(Epi<NR, CHECK>::NT, 1) lrtc_kernel(const __gri
   }
 }
 
+// F (Q x ldf, map-major) from the blocked z: a block transposes 128 voxels of a chunk
+// through shared memory (both sides coalesced; bound by memory)
+__global__ void __launch_bounds__(256) unblock_kernel(const float* __restrict__ Z, int64_t N,
+                                                      int Q, float* __restrict__ F,
+                                                      int64_t ldf) {
+  __shared__ float sm[QC][129];
+  const int64_t n0 = blockIdx.x * (int64_t)128;
+  const int c = blockIdx.y;
+  const float4* src = reinterpret_cast<const float4*>(Z) + ((int64_t)c * N + n0) * (QC / 4);
+  const int nv = (int)min((int64_t)128, N - n0);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int t = threadIdx.x + i * 256, n = t >> 3, j = t & 7;
+    if (n < nv) {
+      const float4 f = __ldg(src + t);
+      sm[4 * j][n] = f.x;
+      sm[4 * j + 1][n] = f.y;
+      sm[4 * j + 2][n] = f.z;
+      sm[4 * j + 3][n] = f.w;
+    }
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int r = w; r < QC; r += 8) {
+    const int q = c * QC + r;
+    if (q >= Q) break;
+    float* dst = F + (int64_t)q * ldf + n0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (lane + 32 * i < nv) dst[lane + 32 * i] = sm[r][lane + 32 * i];
+  }
+}
+
 // V (Q x RP) and V^T (RP x Qs), each split into TF32 hi/lo parts (round to nearest)
 __global__ void split_basis_kernel(const float* __restrict__ V32, int Q, int RP, int Qs,
                                    float* __restrict__ v1h, float* __restrict__ v1l,
@@ -828,53 +940,93 @@ __global__ void split_basis_kernel(const float* __restrict__ V32, int Q, int RP,
   }
 }
 
-template <int RP, int NR, bool CHECK, bool WD>
+// The patch of a grid's tiles: among all bx x by x bz <= 128 whose rows with halo fit the
+// staging area, the one with the least tiles x (a tile's fixed work + its staged rows). The
+// weight of the fixed work (300 rows) and the penalty for rows that do not start on
+// multiples of 8 (a quarter warp's 128-bit loads then meet in the same banks) only break
+// near-ties: 16 x 8 (2D) and 8 x 4 x 4 (3D) where the grid divides. An axis without
+// smoothness (one voxel, or the stacking axis of a batch) needs no halo; a single voxel
+// takes one on x (zero-filled rows), so that there is always a neighbour pair to read.
+constexpr int kMaxRows = 400;
+Patch patch_of(const Grid& g) {
+  Patch best{};
+  double cost = 1e300;
+  const int hy = g.ny > 1, hz = g.nz > 1 && g.zlink;
+  const int hx = g.nx > 1 || (!hy && !hz);
+  const int rmax = hx + hy + hz == 3 ? kMaxRows : 260;
+  for (int bz = 1; bz <= std::min(g.nz, TV); ++bz)
+    for (int by = 1; by <= std::min(g.ny, TV / bz); ++by)
+      for (int bx = 1; bx <= std::min(g.nx, TV / (bz * by)); ++bx) {
+        const int X = bx + 2 * hx, Y = by + 2 * hy, Z = bz + 2 * hz, rows = X * Y * Z;
+        if (rows > rmax) continue;
+        const int64_t tx = (g.nx + bx - 1) / bx, ty = (g.ny + by - 1) / by, tz = (g.nz + bz - 1) / bz;
+        const double c = (double)tx * ty * tz * (300 + rows + (bx % 8 ? 60 : 0));
+        if (c < cost) {
+          cost = c;
+          best = Patch{bx, by, bz, hx, hy, hz, X, Y, Z, rows, (int)tx, (int)ty, (int)tz,
+                       tx * ty * tz, hx + hy + hz, (rows * 128 + 1023) / 1024 * 1024};
+        }
+      }
+  return best;
+}
+
+// what a plan of this form keeps: the tiles, and the tensor maps of both ping-pong halves
+struct LrtcState {
+  Patch p;
+  LrtcMaps maps[2];
+};
+
+template <int RP, int NAX, bool CHECK, bool WD>
 ssm_status set_attr() {
-  return cudaFuncSetAttribute(lrtc_kernel<RP, NR, CHECK, WD>,
+  return cudaFuncSetAttribute(lrtc_kernel<RP, NAX, CHECK, WD>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              Lay<RP, NR>::bytes) == cudaSuccess
+                              kSmemLimit - (CHECK ? 1024 : 0)) == cudaSuccess
              ? SSM_OK
              : SSM_ECUDA;
 }
 
-template <int RP, int NR>
+template <int RP, int NAX>
 ssm_status prepare_rn() {
-  if constexpr (Lay<RP, NR>::valid) {
-    SSM_TRY((set_attr<RP, NR, false, false>()));
-    SSM_TRY((set_attr<RP, NR, false, true>()));
-    SSM_TRY((set_attr<RP, NR, true, false>()));
-    SSM_TRY((set_attr<RP, NR, true, true>()));
-  }
+  SSM_TRY((set_attr<RP, NAX, false, false>()));
+  SSM_TRY((set_attr<RP, NAX, false, true>()));
+  SSM_TRY((set_attr<RP, NAX, true, false>()));
+  SSM_TRY((set_attr<RP, NAX, true, true>()));
   return SSM_OK;
 }
 
-template <int RP, int NR>
+template <int RP, int NAX, bool CHECK, bool WD>
+ssm_status launch_one(const LrtcMaps& maps, LrtcArgs args, int64_t grid, cudaStream_t s) {
+  const int zst = args.p.zst + (CHECK ? OUT_BYTES : 0);
+  const int ob = OUT_BYTES * (WD && !CHECK ? 2 : 1);
+  constexpr int vbytes = Lay<RP, NAX>::NSV * Lay<RP, NAX>::VST;
+  const int room = kSmemLimit - kReserve - vbytes;
+  // two z' buffers per group spare a barrier per chunk, where three z stages still fit
+  args.nob = (room - NG * 2 * ob) / zst >= 3 ? 2 : 1;
+  args.nsz = std::min(kMaxNSZ, (room - NG * args.nob * ob) / zst);
+  if (args.nsz < 2) {
+    set_error("tensor-core low-rank form: two ring stages do not fit");
+    return SSM_EUNSUPPORTED;
+  }
+  const size_t shm = (size_t)(kReserve - 1024) + vbytes + NG * args.nob * ob +
+                     (size_t)args.nsz * zst;
+  lrtc_kernel<RP, NAX, CHECK, WD><<<(unsigned)grid, NT, shm, s>>>(maps, args);
+  SSM_LAUNCHED();
+  return SSM_OK;
+}
+
+template <int RP, int NAX>
 ssm_status launch_rn(const LrtcMaps& maps, const LrtcArgs& args, bool check, bool write_d,
                      int64_t grid, cudaStream_t s) {
-  if constexpr (!Lay<RP, NR>::valid) {
-    set_error("tensor-core low-rank form: this rank does not fit on 3D grids (r <= 32)");
-    return SSM_EUNSUPPORTED;
-  } else {
-    const size_t shm = Lay<RP, NR>::bytes;
-    const unsigned gr = (unsigned)grid;
-    if (check && write_d)
-      lrtc_kernel<RP, NR, true, true><<<gr, Epi<NR, true>::NT, shm, s>>>(maps, args);
-    else if (check)
-      lrtc_kernel<RP, NR, true, false><<<gr, Epi<NR, true>::NT, shm, s>>>(maps, args);
-    else if (write_d)
-      lrtc_kernel<RP, NR, false, true><<<gr, Epi<NR, false>::NT, shm, s>>>(maps, args);
-    else
-      lrtc_kernel<RP, NR, false, false><<<gr, Epi<NR, false>::NT, shm, s>>>(maps, args);
-    SSM_LAUNCHED();
-    return SSM_OK;
-  }
+  if (check && write_d) return launch_one<RP, NAX, true, true>(maps, args, grid, s);
+  if (check) return launch_one<RP, NAX, true, false>(maps, args, grid, s);
+  if (write_d) return launch_one<RP, NAX, false, true>(maps, args, grid, s);
+  return launch_one<RP, NAX, false, false>(maps, args, grid, s);
 }
 
-int grid_nr(const ssm_plan_s* pl) {
-  return (pl->g.ny > 1 ? 2 : 0) + (pl->g.nz > 1 && pl->g.zlink ? 2 : 0);
+int64_t ntiles_of(const ssm_plan_s* pl) {
+  if (pl->lrtc_state) return static_cast<const LrtcState*>(pl->lrtc_state)->p.ntiles;
+  return patch_of(pl->g).ntiles;
 }
-
-int64_t ntiles_of(const ssm_plan_s* pl) { return (pl->g.N + TV - 1) / TV; }
 int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 
 // Launch layout: the CTAs' budget G0 (one per SM per launch wave).
@@ -935,6 +1087,9 @@ int lrtc_padded_rank(int r, bool three_d) {
   return 0;
 }
 
+// floats of one blocked state array
+int64_t lrtc_state_floats(const ssm_plan_s* pl) { return chunks_of(pl) * QC * pl->g.N; }
+
 int64_t lrtc_grid(const ssm_plan_s* pl) {
   int64_t grid;
   int spc, split;
@@ -950,14 +1105,54 @@ int64_t lrtc_partial_floats(const ssm_plan_s* pl, int64_t grid) {
   return ntiles_of(pl) * spc * (int64_t)pl->R * TV;
 }
 
-// once per process and device: the kernels' shared-memory limits
-ssm_status lrtc_prepare() {
-  std::lock_guard<std::mutex> lock(attr_mutex());
-  SSM_TRY((prepare_rn<32, 0>()));
-  SSM_TRY((prepare_rn<32, 2>()));
-  SSM_TRY((prepare_rn<32, 4>()));
-  SSM_TRY((prepare_rn<64, 0>()));
-  SSM_TRY((prepare_rn<64, 2>()));
+// the kernels' shared-memory limits, and the plan's tiles and tensor maps (the state
+// buffers are allocated)
+ssm_status lrtc_prepare(ssm_plan_s* pl) {
+  {
+    std::lock_guard<std::mutex> lock(attr_mutex());
+    SSM_TRY((prepare_rn<32, 1>()));
+    SSM_TRY((prepare_rn<32, 2>()));
+    SSM_TRY((prepare_rn<32, 3>()));
+    SSM_TRY((prepare_rn<64, 1>()));
+    SSM_TRY((prepare_rn<64, 2>()));
+  }
+  auto* st = new LrtcState();
+  pl->lrtc_state = st;
+  st->p = patch_of(pl->g);
+  const Patch& p = st->p;
+  const uint64_t Q = (uint64_t)pl->Q, RP = (uint64_t)pl->R, Qs = (uint64_t)pl->lrtc_qs;
+  const auto SW = CU_TENSOR_MAP_SWIZZLE_128B;
+  const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  const uint64_t nx = (uint64_t)pl->g.nx, ny = (uint64_t)pl->g.ny, nz = (uint64_t)pl->g.nz;
+  const uint64_t dims[5] = {QC, nx, ny, nz, (uint64_t)chunks_of(pl)};
+  const uint64_t strides[4] = {128, 128 * nx, 128 * nx * ny, 128 * nx * ny * nz};
+  const unsigned halo[5] = {QC, (unsigned)p.X, (unsigned)p.Y, (unsigned)p.Z, 1};
+  const unsigned patch[5] = {QC, (unsigned)p.bx, (unsigned)p.by, (unsigned)p.bz, 1};
+  for (int cur = 0; cur < 2; ++cur) {
+    LrtcMaps& m = st->maps[cur];
+    SSM_CUDA(encode_2d(&m.v1h, F32, 4, pl->V1h, RP, Q, RP, 32, QC, SW));
+    SSM_CUDA(encode_2d(&m.v1l, F32, 4, pl->V1l, RP, Q, RP, 32, QC, SW));
+    SSM_CUDA(encode_2d(&m.v2h, F32, 4, pl->V2h, Q, RP, Qs, QC, (unsigned)RP, SW));
+    SSM_CUDA(encode_2d(&m.v2l, F32, 4, pl->V2l, Q, RP, Qs, QC, (unsigned)RP, SW));
+    SSM_CUDA(encode_nd(&m.zi, F32, 5, pl->Z[cur], dims, strides, halo, SW));
+    SSM_CUDA(encode_nd(&m.zp, F32, 5, pl->Z[cur], dims, strides, patch, SW));
+    SSM_CUDA(encode_nd(&m.zo, F32, 5, pl->Z[cur ^ 1], dims, strides, patch, SW));
+    SSM_CUDA(encode_nd(&m.di, F32, 5, pl->Dl[cur], dims, strides, patch, SW));
+    SSM_CUDA(encode_nd(&m.dd, F32, 5, pl->Dl[cur ^ 1], dims, strides, patch, SW));
+  }
+  return SSM_OK;
+}
+
+void lrtc_release(ssm_plan_s* pl) {
+  delete static_cast<LrtcState*>(pl->lrtc_state);
+  pl->lrtc_state = nullptr;
+}
+
+// F = z of ping-pong half `cur`
+ssm_status lrtc_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, cudaStream_t s) {
+  const dim3 grid((unsigned)((pl->g.N + 127) / 128), (unsigned)chunks_of(pl));
+  unblock_kernel<<<grid, 256, 0, s>>>(pl->Z[cur], pl->g.N, pl->Q, F, ldf);
+  SSM_LAUNCHED();
   return SSM_OK;
 }
 
@@ -973,18 +1168,7 @@ ssm_status lrtc_split_basis(ssm_plan_s* pl, cudaStream_t s) {
 
 ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                           int* nparts, cudaStream_t s) {
-  const uint64_t N = (uint64_t)pl->g.N, Q = (uint64_t)pl->Q, ld = (uint64_t)pl->g.ld;
-  const uint64_t RP = (uint64_t)pl->R, Qs = (uint64_t)pl->lrtc_qs;
-  LrtcMaps m;
-  const auto SW = CU_TENSOR_MAP_SWIZZLE_128B;
-  const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  SSM_CUDA(encode_2d(&m.v1h, F32, 4, pl->V1h, RP, Q, RP, 32, QC, SW));
-  SSM_CUDA(encode_2d(&m.v1l, F32, 4, pl->V1l, RP, Q, RP, 32, QC, SW));
-  SSM_CUDA(encode_2d(&m.v2h, F32, 4, pl->V2h, Q, RP, Qs, QC, (unsigned)RP, SW));
-  SSM_CUDA(encode_2d(&m.v2l, F32, 4, pl->V2l, Q, RP, Qs, QC, (unsigned)RP, SW));
-  SSM_CUDA(encode_2d(&m.zc, F32, 4, pl->Z[cur], N, Q, ld, ZW, QC));
-  SSM_CUDA(encode_2d(&m.zn, F32, 4, pl->Z[cur], N, Q, ld, NW, QC));
-  SSM_CUDA(encode_2d(&m.dd, F32, 4, pl->Dl[cur], N, Q, ld, TV, QC));
+  const LrtcState& st = *static_cast<const LrtcState*>(pl->lrtc_state);
   int64_t grid;
   int spc, split;
   layout(pl, &grid, &spc, &split);
@@ -993,40 +1177,38 @@ ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, dou
     return SSM_ECUDA;
   }
   LrtcArgs a;
-  a.Zout = pl->Z[cur ^ 1];
-  a.Dout = pl->Dl[cur ^ 1];
-  a.Din = pl->Dl[cur];
   a.S = pl->S;
   a.Pin = pl->U[cur];
   a.Pout = pl->U[cur ^ 1];
-  a.ntiles = ntiles_of(pl);
   a.nch = (int)chunks_of(pl);
   a.spc = spc;
   a.split = split;
-  a.kr = std::max(1, std::min((int)RP / 8, (pl->r + 7) / 8));
+  a.kr = std::max(1, std::min(pl->R / 8, (pl->r + 7) / 8));
+  a.nsz = a.nob = 0;                 // set per variant (launch_one)
   a.coefA = pl->coefA;
   a.coefW = pl->coefW;
   a.partial = partial;
   a.mask = pl->mask;
   a.err = pl->dev_err;
   a.g = pl->g;
-  a.Q = pl->Q;
+  a.p = st.p;
   a.beta = (float)pl->p.beta;
   a.inv_beta = (float)(1.0 / pl->p.beta);
   a.xi = (float)pl->xi;
   a.lam_s = (float)pl->lam_s;
   a.inv_xb = (float)(1.0 / (pl->xi + pl->p.beta));
   *nparts = (int)grid;
-  const int nr = grid_nr(pl);
+  const LrtcMaps& m = st.maps[cur];
   if (pl->R == 32) {
-    if (nr == 0) return launch_rn<32, 0>(m, a, check, write_d, grid, s);
-    if (nr == 2) return launch_rn<32, 2>(m, a, check, write_d, grid, s);
-    return launch_rn<32, 4>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 1) return launch_rn<32, 1>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 2) return launch_rn<32, 2>(m, a, check, write_d, grid, s);
+    return launch_rn<32, 3>(m, a, check, write_d, grid, s);
   }
   if (pl->R == 64) {
-    if (nr == 0) return launch_rn<64, 0>(m, a, check, write_d, grid, s);
-    if (nr == 2) return launch_rn<64, 2>(m, a, check, write_d, grid, s);
-    return launch_rn<64, 4>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 1) return launch_rn<64, 1>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 2) return launch_rn<64, 2>(m, a, check, write_d, grid, s);
+    set_error("tensor-core low-rank form: this rank is not offered on 3D grids (r <= 32)");
+    return SSM_EUNSUPPORTED;
   }
   set_error("tensor-core low-rank form: unsupported padded rank");
   return SSM_EUNSUPPORTED;
