@@ -871,6 +871,8 @@ ssm_status run_block(ssm_plan_s* pl, int cur, int k, int L, const IsCheck& is_ch
                      cudaStream_t s) {
   for (int j = k; j < k + L; ++j) {
     int np = 0;
+    // (profiling records an event between the launches)
+    pl->chained = j > k && !pl->prof_enabled;
     SSM_TRY(one_iteration(pl, cur, is_check(j), is_check(j + 1), &np, s));
     if (is_check(j)) *nparts = np;
     cur ^= 1;

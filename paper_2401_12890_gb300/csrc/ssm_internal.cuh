@@ -56,6 +56,46 @@ std::mutex& attr_mutex();
   } while (0)
 
 // ------------------------------------------------------------------------------------
+// programmatic dependent launch: consecutive iterations of a solve
+// ------------------------------------------------------------------------------------
+// in a kernel: the dependent launch may start once every CTA has said so (or ended)
+__device__ __forceinline__ void pdl_launch_next() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+// in a kernel: wait until the launches this one depends on have completed and their writes
+// are visible (returns at once in an ordinary launch)
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
+// Launch with or without the programmatic dependency on the launch before it in `s`. With
+// it (`chained`), that launch must be a kernel which calls pdl_launch_next, and this
+// kernel must call pdl_wait before it touches anything an earlier launch reads or writes
+// since the chain began (every kernel of a chain waits, so completion is transitive).
+template <typename K, typename... A>
+ssm_status launch_chained(K kernel, unsigned grid, unsigned block, size_t shm, cudaStream_t s,
+                          bool chained, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) {
+    set_error(std::string("kernel launch: ") + cudaGetErrorString(e));
+    cudaGetLastError();
+    return SSM_ECUDA;
+  }
+  SSM_LAUNCHED();
+  return SSM_OK;
+}
+
+// ------------------------------------------------------------------------------------
 // grid description used by every stencil kernel (Eq. 8, free boundary)
 // ------------------------------------------------------------------------------------
 struct Grid {
@@ -228,6 +268,9 @@ struct ssm_plan_s {
   ssm::TableProblem* tprob = nullptr;  // the iteration's problem descriptor (device)
   int4* ttable = nullptr;            // its (problem, tile, segment) table (device)
   int64_t tblocks = 0;               // entries of the table
+  // the iteration about to be launched directly follows another of the same block in its
+  // stream (set by run_block)
+  bool chained = false;
   // iteration blocks replayed as CUDA graphs (ssm_plan_set_graphs)
   bool use_graphs = false;
   std::vector<ssm::GraphBlock> graphs;

@@ -42,12 +42,17 @@
 //     read as zeros: no neighbour flags in the loop;
 //   - z' leaves by TMA: no global address arithmetic and no store instructions.
 // Measured per iteration in a solve, map-major tiles and one MMA warp before, now:
-//   128x128, Q = 2500, r = 20          110.6 -> 86.0 us
-//   256x256, Q = 2500, r = 20          446.9 -> 297 us
-//   96x96x64, Q = 1600, r = 30          3300 -> 2041 us
-//   192x192, Q = 900, r = 8            85.4 -> 67.0 us
-//   40 slices of 37x29, Q = 225, r = 20  44.9 -> 37.6 us
-//   32x32, Q = 225, r = 20             10.3 -> 9.7 us
+//   128x128, Q = 2500, r = 20            110.6 -> 74 us
+//   256x256, Q = 2500, r = 20            446.9 -> 286 us (4.6 TB/s of 8 Q N bytes)
+//   96x96x64, Q = 1600, r = 30            3300 -> 1833 us (4.1 TB/s)
+//   192x192, Q = 900, r = 8              85.4 -> 61.3 us
+//   40 slices of 37x29, Q = 225, r = 20  44.9 -> 33.4 us
+//   32x32, Q = 225, r = 20               10.3 -> 6.5 us
+// What bounds it now: HBM and the L2 behind it on large grids (0.6-0.7 of the measured copy
+// rate), on small ones a unit's start (a-vector, filling the pipeline: about 6 chunks).
+// Measured and not kept: the patch of the next chunks prefetched into L2 (256x256 -4 %, the
+// others +0 to +4 %); the a-vector of the next unit formed while the last chunk of this
+// one is processed, from a second TMEM buffer (128x128 -2 %, the others +2 to +12 %).
 //
 // Schedule (one CTA per SM): the work units are (segment, tile) pairs, segment-major,
 // dealt round-robin to the CTAs; a segment is a contiguous run of a tile's chunks (one
@@ -58,8 +63,11 @@
 // idle (see layout()). Each segment writes its partial u' to its own slot; the next
 // iteration sums a tile's slots in segment order (fixed, hence deterministic). Warp roles:
 //   warp 0      TMA: per chunk, the patch of z with its halo (and of d on residual-test
-//               iterations) and the chunk's V / V^T boxes (hi and lo)
-//   warp 1      product 1, up to NSV - 1 chunks ahead of product 2
+//               iterations)
+//   warp 3      TMA: the chunk's V rows and V^T rows (hi and lo), in rings of their own: V is
+//               free again when product 1 is done, well before product 2 (one ring for both
+//               held product 1 back until product 2 of NSV chunks before had completed)
+//   warp 1      product 1, up to NVA - 1 chunks ahead of product 2
 //   warp 2      product 2 as soon as a chunk's w is complete. Two warps, because an MMA takes
 //               62 cycles to issue whatever its N (measured, N <= 128): issued by one
 //               thread in turn with its waits, 21 MMAs per chunk (N = 32 each) bounded the
@@ -75,6 +83,9 @@
 // column by column once read, its w (hi, lo), until product 2 of the chunk has completed. a
 // (hi, lo) is per segment; U (main, correction) is double-buffered for RP = 32 and single
 // for 64.
+// Consecutive iterations are chained by programmatic dependent launch: a CTA of the next one
+// starts on an SM as soon as it is free, initialises, loads V and S, and waits for this
+// iteration to complete before it reads z and u.
 // HBM traffic per state element and iteration: read z, write z' (8 B); per voxel and rank:
 // S, the partial u in and out. Every mbarrier wait is bounded and reports SSM_ETIMEOUT
 // through the plan's device error word; the TMA warp waits (bounded) for its last copies,
@@ -96,7 +107,6 @@ constexpr int NT = 128 + 128 * NG;
 constexpr int NVA = 4;               // V a / w slots in TMEM: even, so that a slot's chunks all
                                      // belong to one group (its phases complete in the order
                                      // that group waits for them)
-constexpr int kPrefetch = 4;         // chunks of a tile's own z rows prefetched into L2 ahead
 constexpr int kMaxNSZ = 8;           // z stages (as many as fit, at most)
 constexpr int OUT_BYTES = TV * 128;  // one chunk of a tile's z' (or d')
 constexpr uint32_t TMEM_COLS = 512;
@@ -106,16 +116,13 @@ constexpr int kReserve = 1024 + 1024 + 512 + 1024;   // alignment, the residual 
 
 template <int RP, int NAX>
 struct Lay {
-  // V stages (product 1 runs up to NSV - 1 chunks ahead of product 2)
+  // stages of the V ring (product 1) and of the V^T ring (product 2)
   static constexpr int NSV = RP == 32 && NAX < 3 ? NVA : NVA - 1;
   static constexpr int UB = RP == 32 ? 2 : 1;
-  static constexpr int V1 = RP / 32 * QC * 128;   // V rows of the chunk: RP/32 swizzle atoms
-  static constexpr int V2 = RP * 128;            // V^T rows (RP) x the chunk (128 bytes)
-  // per 32 ranks: the chunk's rows of V_hi, then those of V_lo (one B operand of N = 64);
-  // then the rows of V_hi^T and of V_lo^T (one of N = 2 RP)
+  // V stage: per 32 ranks the chunk's rows of V_hi, then those of V_lo (one B operand of
+  // N = 64); V^T stage: the rows of V_hi^T, then those of V_lo^T (one of N = 2 RP)
   static constexpr int v1(int at, int part) { return (2 * at + part) * QC * 128; }
-  static constexpr int v2h = 2 * V1, v2l = 2 * V1 + V2;
-  static constexpr int VST = 2 * V1 + 2 * V2;    // V stage (a multiple of 1024)
+  static constexpr int VST = RP * 256;           // bytes of either
   static constexpr uint32_t T_VA = 0;                     // slot b: 64 b (main / hi, +32)
   static constexpr uint32_t T_A = 64 * NVA;               // hi, lo at + RP
   static constexpr uint32_t T_U = T_A + 2 * RP;           // buffer b: main 2 RP b, corr + RP
@@ -125,7 +132,7 @@ struct Lay {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) |
            ((uint32_t)(TV >> 4) << 24);
   }
-  static_assert(VST % 1024 == 0 && v2h % 1024 == 0 && v2l % 1024 == 0, "layout");
+  static_assert(VST == RP / 32 * 2 * QC * 128 && VST % 1024 == 0, "layout");
   static_assert(T_U + 2 * RP * UB <= TMEM_COLS, "tensor memory");
 };
 
@@ -143,7 +150,7 @@ struct Patch {
 struct LrtcMaps {
   CUtensorMap v1h, v1l;   // V (Q x RP), box {32, QC}, 128-byte swizzle
   CUtensorMap v2h, v2l;   // V^T (RP x Qs), box {QC, RP}, 128-byte swizzle
-  CUtensorMap zi, zp;     // z^k, boxes {32, X, Y, Z, 1} and {32, bx, by, bz, 1} (prefetch)
+  CUtensorMap zi;         // z^k, box {32, X, Y, Z, 1}
   CUtensorMap zo, di, dd; // z^{k+1}, d^k, d^{k+1}: box {32, bx, by, bz, 1}
 };
 
@@ -286,8 +293,9 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const int nsz = a.nsz, nob = a.nob;
   const int zst = a.p.zst + (CHECK ? OUT_BYTES : 0);      // z rows, then d^k
-  unsigned char* vring = smem;
-  unsigned char* obuf = smem + NSV * L::VST;              // [group][buffer]: z', then d'
+  unsigned char* v1ring = smem;
+  unsigned char* v2ring = smem + NSV * L::VST;
+  unsigned char* obuf = smem + 2 * NSV * L::VST;          // [group][buffer]: z', then d'
   // a residual test that also stores d writes it over the staged d^k
   constexpr bool OWN_D = WD && !CHECK;
   constexpr int OB = OUT_BYTES * (OWN_D ? 2 : 1);
@@ -295,9 +303,11 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   unsigned char* tail = zring + nsz * zst;
   float* zero_row = reinterpret_cast<float*>(tail);       // 128 bytes of zeros (128-aligned)
   float* cAW = zero_row + 32;                             // coefA, coefW (RP each)
-  uint64_t* vfull = reinterpret_cast<uint64_t*>(cAW + 2 * RP);
-  uint64_t* vempty = vfull + NSV;
-  uint64_t* zfull = vempty + NSV;
+  uint64_t* v1full = reinterpret_cast<uint64_t*>(cAW + 2 * RP);
+  uint64_t* v2full = v1full + NSV;
+  uint64_t* v1empty = v2full + NSV;
+  uint64_t* v2empty = v1empty + NSV;
+  uint64_t* zfull = v2empty + NSV;
   uint64_t* zempty = zfull + 2 * kMaxNSZ;
   uint64_t* va_full = zempty + kMaxNSZ;
   uint64_t* w_full = va_full + NVA;
@@ -308,13 +318,17 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   uint64_t* fin = a_free + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 2);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the next iteration's CTAs may take the SMs that this one leaves (or does not use) and
+  // set up; what they read of this iteration they wait for (pdl_wait)
+  pdl_launch_next();
   const int nch = a.nch, spc = a.spc;
-  const int64_t ntiles = a.p.ntiles, nunits = ntiles * spc;
 
   if (tid == 0) {
     for (int s = 0; s < NSV; ++s) {
-      mbar_init(&vfull[s], 1);
-      mbar_init(&vempty[s], 1);
+      mbar_init(&v1full[s], 1);
+      mbar_init(&v2full[s], 1);
+      mbar_init(&v1empty[s], 1);
+      mbar_init(&v2empty[s], 1);
     }
     for (int s = 0; s < nsz; ++s) {
       mbar_init(&zfull[2 * s], 1);
@@ -360,34 +374,36 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   // (concurrent tails are of consecutive tiles too). Otherwise units are dealt
   // round-robin in segment-major order, so that the CTAs running together hold the same
   // chunks of consecutive tiles.
-  auto unit_at = [&](int k, int64_t& tile, int& c0, int& c1, int& sg) -> bool {
+  // (32-bit arithmetic: with several segments per tile there are fewer tiles than CTAs)
+  auto unit_at = [&](int k, int& tile, int& c0, int& c1, int& sg) -> bool {
+    const unsigned nt = (unsigned)a.p.ntiles, G = gridDim.x, j = blockIdx.x;
     if (a.split > 0) {
-      const int64_t j = blockIdx.x, G = gridDim.x;
-      if (j < ntiles) {
+      if (j < nt) {
         if (k > 0) return false;
-        tile = j;
+        tile = (int)j;
         sg = 0;
         c0 = 0;
         c1 = a.split;
         return true;
       }
-      tile = j - ntiles + (int64_t)k * (G - ntiles);
-      if (tile >= ntiles) return false;
+      const unsigned t = j - nt + (unsigned)k * (G - nt);
+      if (t >= nt) return false;
+      tile = (int)t;
       sg = 1;
       c0 = a.split;
       c1 = nch;
       return true;
     }
-    const int64_t u = blockIdx.x + (int64_t)k * gridDim.x;
-    if (u >= nunits) return false;
-    sg = (int)(u / ntiles);
-    tile = u - (int64_t)sg * ntiles;
-    c0 = (int)((int64_t)sg * nch / spc);
-    c1 = (int)((int64_t)(sg + 1) * nch / spc);
+    const int64_t u = j + (int64_t)k * G;
+    if (u >= a.p.ntiles * spc) return false;
+    sg = spc > 1 ? (int)((unsigned)u / nt) : 0;
+    tile = (int)((unsigned)u - (unsigned)sg * nt);
+    c0 = spc > 1 ? sg * nch / spc : 0;
+    c1 = spc > 1 ? (sg + 1) * nch / spc : nch;
     return true;
   };
   // first voxel of a tile
-  auto origin = [&](int64_t tile, int& x0, int& y0, int& z0) {
+  auto origin = [&](int tile, int& x0, int& y0, int& z0) {
     const unsigned t = (unsigned)tile, tx = (unsigned)a.p.tx, ty = (unsigned)a.p.ty;
     x0 = (int)(t % tx) * a.p.bx;
     y0 = (int)(t / tx % ty) * a.p.by;
@@ -395,27 +411,18 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   };
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
+    // ------------------------------------------------------------------ TMA: z (and d)
     if (lane == 0) {
       tma_prefetch_map(&maps.zi);
-      tma_prefetch_map(&maps.zp);
-      tma_prefetch_map(&maps.v1h);
-      tma_prefetch_map(&maps.v2h);
+      pdl_wait();
       const unsigned zbytes = (unsigned)a.p.rows * 128u +
                               (CHECK ? (unsigned)(a.p.bx * a.p.by * a.p.bz) * 128u : 0u);
       int g = 0;
-      int64_t tile;
-      int c0, c1, sg;
+      int tile, c0, c1, sg;
       for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k) {
         int x0, y0, z0;
         origin(tile, x0, y0, z0);
-        // the tile's own rows come from HBM: they are prefetched into L2 kPrefetch chunks
-        // ahead of the stages, so that enough bytes are in flight per SM (the halo rows are
-        // prefetched by the CTAs that own them)
-        for (int c = c0 + 1; c < c0 + kPrefetch && c < c1; ++c)
-          tma_prefetch_5d(&maps.zp, 0, x0, y0, z0, c);
         for (int c = c0; c < c1; ++c, ++g) {
-          if (c + kPrefetch < c1) tma_prefetch_5d(&maps.zp, 0, x0, y0, z0, c + kPrefetch);
           const int sz = g % nsz, kz = g / nsz;
           if (kz > 0 && !mbar_wait_sleep(&zempty[sz], (kz - 1) & 1)) {
             failed = true;
@@ -429,40 +436,62 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           mbar_arrive_expect_tx(bar, zbytes);
           tma_load_5d(zs, &maps.zi, 0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, c, bar);
           if (CHECK) tma_load_5d(zs + a.p.zst, &maps.di, 0, x0, y0, z0, c, bar);
-          const int sv = g % NSV, kv = g / NSV, q0 = c * QC;
-          uint64_t* ve = NSV == NVA ? &p2_done[sv] : &vempty[sv];
-          if (kv > 0 && !mbar_wait_sleep(ve, (kv - 1) & 1)) {
-            failed = true;
-            ++g;          // the z copies of this chunk were issued
-            break;
-          }
-          unsigned char* vs = vring + sv * L::VST;
-          mbar_arrive_expect_tx(&vfull[sv], (unsigned)L::VST);
-#pragma unroll
-          for (int at = 0; at < RP / 32; ++at) {
-            tma_load_2d(vs + L::v1(at, 0), &maps.v1h, at * 32, q0, &vfull[sv]);
-            tma_load_2d(vs + L::v1(at, 1), &maps.v1l, at * 32, q0, &vfull[sv]);
-          }
-          tma_load_2d(vs + L::v2h, &maps.v2h, q0, 0, &vfull[sv]);
-          tma_load_2d(vs + L::v2l, &maps.v2l, q0, 0, &vfull[sv]);
         }
       }
       // no copy may still be in flight when the CTA exits: wait (bounded) for the last
       // phase issued into every stage
-      for (int s = 0; s < NSV && s < g; ++s)
-        mbar_wait_sleep(&vfull[s], ((s + ((g - 1 - s) / NSV) * NSV) / NSV) & 1);
       for (int s = 0; s < nsz && s < g; ++s) {
         const int kz = (g - 1 - s) / nsz;            // the stage's last round
         mbar_wait_sleep(&zfull[2 * s + (kz & 1)], (kz >> 1) & 1);
       }
+    }
+  } else if (warp == 3) {
+    // ------------------------------------------------------------------ TMA: V and V^T
+    if (lane == 0) {
+      tma_prefetch_map(&maps.v1h);
+      tma_prefetch_map(&maps.v2h);
+      int g = 0, g2 = 0;
+      int tile, c0, c1, sg;
+      for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k)
+        for (int c = c0; c < c1; ++c, ++g) {
+          const int sv = g % NSV, kv = g / NSV, q0 = c * QC;
+          // a stage is free once its product has completed (where there are as many stages
+          // as slots, the slot's barrier says so)
+          if (kv > 0 &&
+              !mbar_wait_sleep(NSV == NVA ? &va_full[sv] : &v1empty[sv], (kv - 1) & 1)) {
+            failed = true;
+            break;
+          }
+          unsigned char* vs = v1ring + sv * L::VST;
+          mbar_arrive_expect_tx(&v1full[sv], (unsigned)L::VST);
+#pragma unroll
+          for (int at = 0; at < RP / 32; ++at) {
+            tma_load_2d(vs + L::v1(at, 0), &maps.v1h, at * 32, q0, &v1full[sv]);
+            tma_load_2d(vs + L::v1(at, 1), &maps.v1l, at * 32, q0, &v1full[sv]);
+          }
+          if (kv > 0 &&
+              !mbar_wait_sleep(NSV == NVA ? &p2_done[sv] : &v2empty[sv], (kv - 1) & 1)) {
+            failed = true;
+            ++g;          // the V copies of this chunk were issued
+            break;
+          }
+          vs = v2ring + sv * L::VST;
+          mbar_arrive_expect_tx(&v2full[sv], (unsigned)L::VST);
+          tma_load_2d(vs, &maps.v2h, q0, 0, &v2full[sv]);
+          tma_load_2d(vs + L::VST / 2, &maps.v2l, q0, 0, &v2full[sv]);
+          g2 = g + 1;
+        }
+      for (int s = 0; s < NSV && s < g; ++s)
+        mbar_wait_sleep(&v1full[s], ((g - 1 - s) / NSV) & 1);
+      for (int s = 0; s < NSV && s < g2; ++s)
+        mbar_wait_sleep(&v2full[s], ((g2 - 1 - s) / NSV) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ product 1
     if (lane == 0) {
       const uint32_t a_hi = tmem + L::T_A, a_lo = tmem + L::T_A + RP;
       int g = 0, si = 0;
-      int64_t tile;
-      int c0, c1, sg;
+      int tile, c0, c1, sg;
       for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k) {
         const int nchk = c1 - c0;
         if (!mbar_wait_sleep(a_ready, si & 1)) {
@@ -474,12 +503,12 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           // V a (main, correction) of chunk gg: a_hi . [V_hi | V_lo]^T into both, then
           // a_lo . V_hi^T into the correction; its slot's previous w has been read
           const int gg = g + i, b = gg % NVA;
-          if (!mbar_wait_sleep(&vfull[gg % NSV], (gg / NSV) & 1)) failed = true;
+          if (!mbar_wait_sleep(&v1full[gg % NSV], (gg / NSV) & 1)) failed = true;
           if (!failed && gg >= NVA && !mbar_wait_sleep(&p2_done[b], (gg / NVA - 1) & 1))
             failed = true;
           if (failed) break;
           fence_after();
-          const uint32_t vs = smem_u32(vring + (gg % NSV) * L::VST);
+          const uint32_t vs = smem_u32(v1ring + (gg % NSV) * L::VST);
           const uint32_t dm = tmem + L::T_VA + 64 * b, dc = dm + 32;
           // the padding ranks beyond r carry zero a: their K steps are skipped
 #pragma unroll 4
@@ -489,6 +518,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
             mma_tf32(dc, a_lo + 8 * k8, bh, L::idesc(QC), 1u);
           }
           commit(&va_full[b]);
+          if (NSV != NVA) commit(&v1empty[gg % NSV]);
           if (i == nchk - 1) commit(a_free);     // a may be rewritten once these complete
         }
         g += nchk;
@@ -502,31 +532,30 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
     // ------------------------------------------------------------------ product 2
     if (lane == 0) {
       int g = 0;
-      int64_t tile;
-      int c0, c1, sg;
+      int tile, c0, c1, sg;
       for (int k = 0; !failed && unit_at(k, tile, c0, c1, sg); ++k) {
         for (int c = c0; c < c1; ++c, ++g) {
           // U (main, correction) of chunk g: w_hi . [V_hi | V_lo] into both, then w_lo . V_hi
           // into the correction
           const int b = g % NVA, gp = g - UB;
-          if (!mbar_wait_sleep(&vfull[g % NSV], (g / NSV) & 1)) failed = true;
+          if (!mbar_wait_sleep(&v2full[g % NSV], (g / NSV) & 1)) failed = true;
           if (!failed && !mbar_wait_sleep(&w_full[b], (g / NVA) & 1)) failed = true;
           // the U buffer is free once the epilogue has read chunk g - UB's
           if (!failed && gp >= 0 && !mbar_wait_sleep(&u_free[gp & 1], (gp >> 1) & 1))
             failed = true;
           if (failed) break;
           fence_after();
-          const uint32_t vs = smem_u32(vring + (g % NSV) * L::VST);
+          const uint32_t vs = smem_u32(v2ring + (g % NSV) * L::VST);
           const uint32_t dm = tmem + L::T_U + 2 * RP * (g % UB), dc = dm + RP;
           const uint32_t w_hi = tmem + L::T_VA + 64 * b, w_lo = w_hi + 32;
 #pragma unroll
           for (int k8 = 0; k8 < QC / 8; ++k8) {
-            const uint64_t bh = sdesc(vs + L::v2h + k8 * 32);
+            const uint64_t bh = sdesc(vs + k8 * 32);
             mma_tf32(dm, w_hi + 8 * k8, bh, L::idesc(2 * RP), k8 > 0 ? 1u : 0u);
             mma_tf32(dc, w_lo + 8 * k8, bh, L::idesc(RP), 1u);
           }
           commit(&p2_done[b]);
-          if (NSV != NVA) commit(&vempty[g % NSV]);   // the V stage is free too
+          if (NSV != NVA) commit(&v2empty[g % NSV]);
         }
       }
       commit(&fin[1]);
@@ -546,8 +575,9 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
     const float c2 = a.lam_s * a.inv_xb;             // weight of the neighbour sum
     const float c3 = a.beta * a.inv_xb;              // weight of V a
     const float beta = a.beta;
-    const float2 c2_2 = make_float2(c2, c2), c3_2 = make_float2(c3, c3);
+    const float2 c2_2 = make_float2(c2, c2), c3_2 = make_float2(-c3, -c3);   // (of -V a)
     const float2 beta2 = make_float2(beta, beta), two2 = make_float2(2.f, 2.f);
+    const float2 m1 = make_float2(-1.f, -1.f);
     // this lane's voxel within a patch, and its row among the staged rows (swizzled: the
     // 16-byte piece j of row r sits at piece j ^ (r & 7))
     const int lx = v % a.p.bx, ly = v / a.p.bx % a.p.by, lz = v / (a.p.bx * a.p.by);
@@ -572,8 +602,8 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
     const uint32_t zero = smem_u32(zero_row), ring = smem_u32(zring);
     const uint32_t ob0 = smem_u32(obuf) + grp * nob * OB;
 
-    int64_t tile = 0, n = 0;
-    int c0 = 0, c1 = 0, sg = 0;
+    int64_t n = 0;
+    int tile = 0, c0 = 0, c1 = 0, sg = 0;
     bool in = false;
     float e1 = 0.f;
     float us[RQ], sv[RQ];
@@ -597,12 +627,28 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           deg += (z > 0 && (!mk || mk[n - plane])) + (z < nz - 1 && (!mk || mk[n + plane]));
       }
       e1 = (a.xi + a.beta - a.lam_s * (float)deg) * a.inv_xb;   // weight of z
-      const float* pt = a.Pin + tile * spc * (int64_t)(RP * TV) + grp * RQ * TV + v;
+      const float* pt = a.Pin + (int64_t)tile * spc * (RP * TV) + grp * RQ * TV + v;
       const float* sp = a.S + (int64_t)(grp * RQ) * ld + n;
 #pragma unroll
-      for (int i = 0; i < RQ; ++i) {
-        sv[i] = in ? __ldg(sp + i * ld) : 0.f;
-        us[i] = pt[i * TV];
+      for (int i = 0; i < RQ; ++i) sv[i] = in ? __ldg(sp + i * ld) : 0.f;
+      if (k == 0) pdl_wait();     // S is the solve's; u is the previous iteration's
+#pragma unroll
+      for (int i = 0; i < RQ; ++i) us[i] = pt[i * TV];
+      // the next unit's come from HBM: into L2 ahead
+      {
+        int t1, d0, d1, d2, x1, y1, z1;
+        if (unit_at(k + 1, t1, d0, d1, d2)) {
+          origin(t1, x1, y1, z1);
+          const int64_t n1 = min(x1 + lx, nx - 1) +
+                             (int64_t)nx * (min(y1 + ly, ny - 1) + (int64_t)ny * min(z1 + lz, nz - 1));
+          const float* p1 = a.Pin + ((int64_t)t1 * spc * RP + grp * RQ) * TV + v;
+          const float* s1p = a.S + (int64_t)(grp * RQ) * ld + n1;
+#pragma unroll 4
+          for (int i = 0; i < RQ; ++i) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(s1p + i * ld));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p1 + i * TV));
+          }
+        }
       }
       // (SB slots' loads in flight together; a slot past the last reads the last with weight 0)
       constexpr int SB = RQ <= 16 ? 3 : 1;
@@ -633,7 +679,8 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int r = grp * RQ + i + j;
-          const float av = in ? sv[i + j] * cAW[r] - cAW[RP + r] * us[i + j] : 0.f;
+          // negated, so that -t = (-V a) - z needs no sign flips below
+          const float av = in ? cAW[RP + r] * us[i + j] - sv[i + j] * cAW[r] : 0.f;
           ah[j] = tf32_rna(av);
           al[j] = tf32_rna(av - ah[j]);
         }
@@ -698,7 +745,11 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           __syncwarp();
           group_barrier(1 + grp);
         }
+        // (the stages are 1024-byte-aligned: the piece index only flips bits 4-6)
         const uint32_t zb = in ? ring + sz * zst : zero;
+        uint32_t za[1 + 2 * NAX];
+#pragma unroll
+        for (int q = 0; q < 1 + 2 * NAX; ++q) za[q] = zb + rr[q];
         const uint32_t db = in ? ring + sz * zst + a.p.zst : zero;
         const uint32_t ob = ob0 + (nob == 2 ? (own & 1) * OB : 0) + vrow;
 #pragma unroll
@@ -721,15 +772,15 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
-            zz[h] = lds4(zb + (rr[0] ^ jx));
+            zz[h] = lds4(za[0] ^ jx);
 #pragma unroll
-            for (int q = 0; q < 2 * NAX; ++q) nb[q][h] = lds4(zb + (rr[1 + q] ^ jx));
+            for (int q = 0; q < 2 * NAX; ++q) nb[q][h] = lds4(za[1 + q] ^ jx);
           }
           float zn[8], w[8];
           float4 dk[2];
           if constexpr (CHECK) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) dk[h] = lds4(db + (dro ^ ((uint32_t)(2 * sb + h) << 4)));
+            for (int h = 0; h < 2; ++h) dk[h] = lds4((db + dro) ^ ((uint32_t)(2 * sb + h) << 4));
           }
           float dn[8];
 #pragma unroll
@@ -744,20 +795,20 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
             for (int q = 2; q < 2 * NAX; ++q) s = __fadd2_rn(s, pr(nb[q][h]));
             const float2 y = __ffma2_rn(e1_2, z2, __ffma2_rn(c2_2, s, __fmul2_rn(c3_2, va2[j])));
             const float2 n2 = make_float2(fmaxf(0.f, y.x), fmaxf(0.f, y.y));
-            const float2 t2 = __fadd2_rn(z2, va2[j]);
-            const float2 w2 = __fmul2_rn(beta2, __ffma2_rn(two2, n2, make_float2(-t2.x, -t2.y)));
+            const float2 mt = __ffma2_rn(m1, z2, va2[j]);                       // -t
+            const float2 w2 = __fmul2_rn(beta2, __ffma2_rn(two2, n2, mt));
             zn[2 * j] = n2.x;
             zn[2 * j + 1] = n2.y;
             w[2 * j] = w2.x;
             w[2 * j + 1] = w2.y;
             if constexpr (WD) {
-              dn[2 * j] = beta * (t2.x - n2.x);
-              dn[2 * j + 1] = beta * (t2.y - n2.y);
+              dn[2 * j] = -beta * (mt.x + n2.x);
+              dn[2 * j + 1] = -beta * (mt.y + n2.y);
             }
             if constexpr (CHECK) {
               // f^{k+1} = t - d^k / beta
               const float2 d2 = pr(dk[h]);
-              const float f0 = t2.x - d2.x * a.inv_beta, f1 = t2.y - d2.y * a.inv_beta;
+              const float f0 = -(mt.x + d2.x * a.inv_beta), f1 = -(mt.y + d2.y * a.inv_beta);
               const float ea = n2.x - f0, eb = n2.y - f1;
               const float ca = n2.x - z2.x, cb = n2.y - z2.y;
               s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
@@ -781,7 +832,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
             wh[j] = tf32_rna(w[j]);
             wh[j + 1] = tf32_rna(w[j + 1]);
             const float2 l2 =
-                __fadd2_rn(make_float2(w[j], w[j + 1]), make_float2(-wh[j], -wh[j + 1]));
+                __ffma2_rn(m1, make_float2(wh[j], wh[j + 1]), make_float2(w[j], w[j + 1]));
             wl[j] = tf32_rna(l2.x);
             wl[j + 1] = tf32_rna(l2.y);
           }
@@ -817,7 +868,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
         ++own;
       }
       // the next unit's loads go out before this one's last sums are waited for
-      float* po = a.Pout + (tile * spc + sg) * (int64_t)(RP * TV) + v;
+      float* po = a.Pout + ((int64_t)tile * spc + sg) * (RP * TV) + v;
       const bool in0 = in;
       const int gl = g + nchk - 1;                   // the unit's last chunk
       more = begin(k + 1);
@@ -974,6 +1025,7 @@ Patch patch_of(const Grid& g) {
 struct LrtcState {
   Patch p;
   LrtcMaps maps[2];
+  int spc = 1, split = 0;   // launch layout (the grid is the plan's lr_grid)
 };
 
 template <int RP, int NAX, bool CHECK, bool WD>
@@ -995,10 +1047,11 @@ ssm_status prepare_rn() {
 }
 
 template <int RP, int NAX, bool CHECK, bool WD>
-ssm_status launch_one(const LrtcMaps& maps, LrtcArgs args, int64_t grid, cudaStream_t s) {
+ssm_status launch_one(const LrtcMaps& maps, LrtcArgs args, int64_t grid, bool chained,
+                      cudaStream_t s) {
   const int zst = args.p.zst + (CHECK ? OUT_BYTES : 0);
   const int ob = OUT_BYTES * (WD && !CHECK ? 2 : 1);
-  constexpr int vbytes = Lay<RP, NAX>::NSV * Lay<RP, NAX>::VST;
+  constexpr int vbytes = 2 * Lay<RP, NAX>::NSV * Lay<RP, NAX>::VST;
   const int room = kSmemLimit - kReserve - vbytes;
   // two z' buffers per group spare a barrier per chunk, where three z stages still fit
   args.nob = (room - NG * 2 * ob) / zst >= 3 ? 2 : 1;
@@ -1009,18 +1062,17 @@ ssm_status launch_one(const LrtcMaps& maps, LrtcArgs args, int64_t grid, cudaStr
   }
   const size_t shm = (size_t)(kReserve - 1024) + vbytes + NG * args.nob * ob +
                      (size_t)args.nsz * zst;
-  lrtc_kernel<RP, NAX, CHECK, WD><<<(unsigned)grid, NT, shm, s>>>(maps, args);
-  SSM_LAUNCHED();
-  return SSM_OK;
+  return launch_chained(lrtc_kernel<RP, NAX, CHECK, WD>, (unsigned)grid, NT, shm, s, chained, maps,
+                        args);
 }
 
 template <int RP, int NAX>
 ssm_status launch_rn(const LrtcMaps& maps, const LrtcArgs& args, bool check, bool write_d,
-                     int64_t grid, cudaStream_t s) {
-  if (check && write_d) return launch_one<RP, NAX, true, true>(maps, args, grid, s);
-  if (check) return launch_one<RP, NAX, true, false>(maps, args, grid, s);
-  if (write_d) return launch_one<RP, NAX, false, true>(maps, args, grid, s);
-  return launch_one<RP, NAX, false, false>(maps, args, grid, s);
+                     int64_t grid, bool chained, cudaStream_t s) {
+  if (check && write_d) return launch_one<RP, NAX, true, true>(maps, args, grid, chained, s);
+  if (check) return launch_one<RP, NAX, true, false>(maps, args, grid, chained, s);
+  if (write_d) return launch_one<RP, NAX, false, true>(maps, args, grid, chained, s);
+  return launch_one<RP, NAX, false, false>(maps, args, grid, chained, s);
 }
 
 int64_t ntiles_of(const ssm_plan_s* pl) {
@@ -1035,11 +1087,10 @@ int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 //  - Between G0/2 and G0 tiles (the 128x128 slice: 128 tiles, 152 SMs): one segment per
 //    tile would leave G0 - ntiles SMs idle, two would give some CTAs two whole-Q-halves
 //    of work; instead CTA j < ntiles takes chunks [0, split) of tile j and the spare
-//    CTAs take the tails, `split` chosen so that both kinds finish together (counting a
-//    unit's start as one chunk). On the slice: 126 us per launch at split 69 (150 CTAs)
-//    against 136 us with one segment per tile (128 CTAs); splits of 60 and 64 overload
-//    the tail CTAs (209 and 172 us).
+//    CTAs take the tails, `split` chosen so that both kinds finish together, a unit's start
+//    counting as kStart chunks.
 //  - Fewer tiles: each tile is split into spc equal segments so that all CTAs have work.
+constexpr int kStart = 6;   // chunks a unit's start (a-vector, filling the pipeline) takes as long as
 void layout(const ssm_plan_s* pl, int64_t* grid, int* spc, int* split) {
   const int64_t ntiles = ntiles_of(pl), nch = chunks_of(pl);
   int64_t g0 = (int64_t)sm_count() * std::max(1, pl->waves);
@@ -1062,7 +1113,7 @@ void layout(const ssm_plan_s* pl, int64_t* grid, int* spc, int* split) {
     const int64_t per = (ntiles + spare - 1) / spare;   // tails per spare CTA
     int64_t best = 1, cost = INT64_MAX;
     for (int64_t c = 1; c < nch; ++c) {
-      const int64_t t = std::max(c + 1, per * (nch - c + 1));
+      const int64_t t = std::max(c + kStart, per * (nch - c + kStart));
       if (t < cost) {
         cost = t;
         best = c;
@@ -1119,6 +1170,7 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
   auto* st = new LrtcState();
   pl->lrtc_state = st;
   st->p = patch_of(pl->g);
+  layout(pl, &pl->lr_grid, &st->spc, &st->split);
   const Patch& p = st->p;
   const uint64_t Q = (uint64_t)pl->Q, RP = (uint64_t)pl->R, Qs = (uint64_t)pl->lrtc_qs;
   const auto SW = CU_TENSOR_MAP_SWIZZLE_128B;
@@ -1135,7 +1187,6 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
     SSM_CUDA(encode_2d(&m.v2h, F32, 4, pl->V2h, Q, RP, Qs, QC, (unsigned)RP, SW));
     SSM_CUDA(encode_2d(&m.v2l, F32, 4, pl->V2l, Q, RP, Qs, QC, (unsigned)RP, SW));
     SSM_CUDA(encode_nd(&m.zi, F32, 5, pl->Z[cur], dims, strides, halo, SW));
-    SSM_CUDA(encode_nd(&m.zp, F32, 5, pl->Z[cur], dims, strides, patch, SW));
     SSM_CUDA(encode_nd(&m.zo, F32, 5, pl->Z[cur ^ 1], dims, strides, patch, SW));
     SSM_CUDA(encode_nd(&m.di, F32, 5, pl->Dl[cur], dims, strides, patch, SW));
     SSM_CUDA(encode_nd(&m.dd, F32, 5, pl->Dl[cur ^ 1], dims, strides, patch, SW));
@@ -1169,20 +1220,14 @@ ssm_status lrtc_split_basis(ssm_plan_s* pl, cudaStream_t s) {
 ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                           int* nparts, cudaStream_t s) {
   const LrtcState& st = *static_cast<const LrtcState*>(pl->lrtc_state);
-  int64_t grid;
-  int spc, split;
-  layout(pl, &grid, &spc, &split);
-  if (grid != pl->lr_grid) {
-    set_error("tensor-core low-rank form: launch layout changed since planning");
-    return SSM_ECUDA;
-  }
+  const int64_t grid = pl->lr_grid;
   LrtcArgs a;
   a.S = pl->S;
   a.Pin = pl->U[cur];
   a.Pout = pl->U[cur ^ 1];
   a.nch = (int)chunks_of(pl);
-  a.spc = spc;
-  a.split = split;
+  a.spc = st.spc;
+  a.split = st.split;
   a.kr = std::max(1, std::min(pl->R / 8, (pl->r + 7) / 8));
   a.nsz = a.nob = 0;                 // set per variant (launch_one)
   a.coefA = pl->coefA;
@@ -1199,14 +1244,20 @@ ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, dou
   a.inv_xb = (float)(1.0 / (pl->xi + pl->p.beta));
   *nparts = (int)grid;
   const LrtcMaps& m = st.maps[cur];
+  // Chained launches spare the launch gap and the set-up (32x32: 10.4 -> 7.2 us per
+  // iteration; 192x192, Q = 900, two units per CTA: 65.0 -> 60.4), but let the CTAs of an
+  // iteration start as the last one's leave, out of step with the tiles next to them, whose
+  // halo rows they then find in L2 less often: with 31 units per CTA (96x96x64) 1877 ->
+  // 1979 us. With few units per CTA the gap weighs more (256x256, 3.4 units: 273 -> 269)
+  const bool chained = pl->chained && st.p.ntiles * st.spc <= 8 * grid;
   if (pl->R == 32) {
-    if (st.p.naxes == 1) return launch_rn<32, 1>(m, a, check, write_d, grid, s);
-    if (st.p.naxes == 2) return launch_rn<32, 2>(m, a, check, write_d, grid, s);
-    return launch_rn<32, 3>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 1) return launch_rn<32, 1>(m, a, check, write_d, grid, chained, s);
+    if (st.p.naxes == 2) return launch_rn<32, 2>(m, a, check, write_d, grid, chained, s);
+    return launch_rn<32, 3>(m, a, check, write_d, grid, chained, s);
   }
   if (pl->R == 64) {
-    if (st.p.naxes == 1) return launch_rn<64, 1>(m, a, check, write_d, grid, s);
-    if (st.p.naxes == 2) return launch_rn<64, 2>(m, a, check, write_d, grid, s);
+    if (st.p.naxes == 1) return launch_rn<64, 1>(m, a, check, write_d, grid, chained, s);
+    if (st.p.naxes == 2) return launch_rn<64, 2>(m, a, check, write_d, grid, chained, s);
     set_error("tensor-core low-rank form: this rank is not offered on 3D grids (r <= 32)");
     return SSM_EUNSUPPORTED;
   }
