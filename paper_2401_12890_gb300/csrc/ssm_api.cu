@@ -101,11 +101,13 @@ int64_t lowrank_state_floats(const ssm_plan_s* pl, int64_t grid) {
                                        : lowrank_partial_floats(pl, grid);
 }
 
-// floats of one state array (z or d): blocked for the TF32x3 form, else Q x ld
+// floats of one state array (z or d): blocked for the low-rank forms, else Q x ld (a group
+// runs low-rank FP32 plans in their buffers map-major: room for either)
 int64_t state_floats(const ssm_plan_s* pl) {
-  if (pl->p.form == SSM_FORM_LOWRANK && pl->p.precision == SSM_TF32X3)
-    return lrtc_state_floats(pl);
-  return (int64_t)pl->Q * pl->g.ld;
+  const int64_t flat = (int64_t)pl->Q * pl->g.ld;
+  if (pl->p.form != SSM_FORM_LOWRANK || pl->ndict > 0) return flat;
+  const int64_t blocked = blocked_floats(pl->g, pl->Q);
+  return pl->p.precision == SSM_TF32X3 ? blocked : std::max(flat, blocked);
 }
 
 int padded_rank(int r) {
@@ -192,7 +194,8 @@ ssm_status validate(const ssm_params* p) {
 void release(ssm_plan_s* pl) {
   if (!pl) return;
   tc_release(pl);
-  lrtc_release(pl);
+  if (pl->p.form == SSM_FORM_LOWRANK && pl->p.precision == SSM_TF32X3) lrtc_release(pl);
+  else lowrank_release(pl);
   dfree(pl->K64);
   dfree(pl->Bp64);
   dfree(pl->Kt64);
@@ -441,8 +444,8 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
       pl->lr_grid = lrtc_grid(pl);
       maxparts = (int)pl->lr_grid;
     } else {
-      pl->lr_grid = lowrank_grid(pl);
-      maxparts = lowrank_max_partials(pl);
+      SSM_TRY(lowrank_prepare(pl));
+      maxparts = (int)pl->lr_grid;
     }
     const size_t pf = (size_t)lowrank_state_floats(pl, pl->lr_grid);
     for (int i = 0; i < 2; ++i) SSM_TRY(palloc(pl, &pl->U[i], pf, s));
@@ -985,9 +988,13 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
     // (and both tensor-core operands) must hold zeros there
     const int nbuf = pl->mask ? 2 : 1;
     const size_t zbytes = sizeof(float) * (size_t)state_floats(pl);
+    // the low-rank forms read d^k only in a residual test, after the iteration before has
+    // stored it: d = 0 is needed only where the first iteration tests (or none runs, and a
+    // resumed solve's first one may)
+    const bool need_d = p.form != SSM_FORM_LOWRANK || p.max_iter <= 1 || p.check_every == 1;
     for (int i = 0; i < nbuf; ++i) {
       SSM_CUDA(cudaMemsetAsync(pl->Z[i], 0, zbytes, s));
-      SSM_CUDA(cudaMemsetAsync(pl->Dl[i], 0, zbytes, s));
+      if (need_d) SSM_CUDA(cudaMemsetAsync(pl->Dl[i], 0, zbytes, s));
     }
     if (pl->mask && pl->Whi[1]) {
       const size_t WN = (size_t)pl->g.ld * pl->Qp;
@@ -1043,8 +1050,8 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
   pl->has_state = true;
   // F = z (the feasible iterate; y for Algorithm 1)
   const float* Fsrc = p.form == SSM_FORM_ADMM ? pl->adm.y : pl->Z[cur];
-  if (pl->lrtc_state)
-    SSM_TRY(lrtc_output(pl, cur, F, ldf, s));
+  if (pl->lr_state)
+    SSM_TRY(blocked_output(pl, cur, F, ldf, s));
   else
     SSM_CUDA(cudaMemcpy2DAsync(F, sizeof(float) * ldf, Fsrc, sizeof(float) * ld,
                                sizeof(float) * pl->g.N, pl->Q, cudaMemcpyDeviceToDevice, s));

@@ -105,6 +105,19 @@ struct Grid {
   int zlink = 1;      // 0: the z axis stacks independent slices (no smoothness across it)
 };
 
+// The tiles of a grid: patches of bx x by x bz voxels (lane = lx + bx (ly + by lz)), loaded
+// with a halo of one voxel on every axis with smoothness (h = 1) as X x Y x Z rows
+struct Patch {
+  int bx, by, bz, hx, hy, hz;
+  int X, Y, Z, rows;
+  int tx, ty, tz;            // tiles per axis
+  int64_t ntiles;
+  int naxes;                 // axes with smoothness (at least 1: see patch_of)
+  int zst;                   // bytes of the z rows, rounded up to 1024
+};
+
+Patch patch_of(const Grid& g);
+
 // One element of the full-rank iteration's z-step (Eq. 31, with D^T D z = s (deg z -
 // sum_nbr z)) and dual step (step 11), given f = h + M w:
 //     z' = max(0, (xi z - lambda s (deg z - nb) + beta f + d) / (xi + beta))
@@ -200,7 +213,6 @@ struct ssm_plan_s {
   float* V2h = nullptr;
   float* V2l = nullptr;
   int lrtc_qs = 0;             // row stride of V^T: Q rounded up to 32
-  void* lrtc_state = nullptr;  // its tiles and tensor maps (ssm_lowrank_tc.cu)
   float* coefA = nullptr;      // R      1/(beta + sigma_i^2)
   float* coefW = nullptr;      // R      sigma_i^2/(beta^2 + beta sigma_i^2)
   double* alpha64 = nullptr;   // n      S_i = alpha_i c_i
@@ -214,13 +226,14 @@ struct ssm_plan_s {
   int* vexp = nullptr;               // ld
   int Qp = 0;                  // padded row stride of Q x Q operands
 
-  // per-voxel state (map-major, leading dimension g.ld; z and d of the TF32x3 form are
-  // blocked, see ssm_lowrank_tc.cu)
+  // per-voxel state (map-major, leading dimension g.ld; z and d of the low-rank forms are
+  // blocked, see ssm_blocked.cu, except in a plan with spatially varying dictionaries)
   float* Z[2] = {nullptr, nullptr};  // z ping-pong            (Q x ld)
   float* Dl[2] = {nullptr, nullptr}; // dual d ping-pong       (Q x ld)
   float* S = nullptr;                // S_i = sigma_i u_i^T m  (R x ld)
   float* U[2] = {nullptr, nullptr};  // partial u = V^T (beta z - d) per (tile, segment)
   int64_t lr_grid = 0;               // persistent grid of the low-rank kernel
+  void* lr_state = nullptr;          // its tiles, tensor maps and layout
   float* H = nullptr;                // h = M g                (Q x ld)     dense
   float* Wf = nullptr;               // w = beta z - d (FP32)  (Q x ld)     dense fp32
   float* Acc = nullptr;              // M w                    (Q x ld)     dense fp32
@@ -313,7 +326,14 @@ ssm_status exact_product(const __nv_bfloat16* slices, const int* rexp, int rows,
                          const float* M, int64_t ldm, int64_t N, float* out, int64_t ldo,
                          int* vexp, int* err, cudaStream_t s);
 
+// blocked state of the low-rank forms (ssm_blocked.cu): floats of one array; F = z of
+// ping-pong half `cur`
+int64_t blocked_floats(const Grid& g, int Q);
+ssm_status blocked_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, cudaStream_t s);
+
 // low-rank iteration (ssm_lowrank.cu)
+ssm_status lowrank_prepare(ssm_plan_s* pl);
+void lowrank_release(ssm_plan_s* pl);
 // low-rank iteration k -> k+1 with state (z, per-voxel u); `check` forms the residual
 // sums (and reads d^k), `write_d` stores d^{k+1} for the next iteration's test
 ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
@@ -326,10 +346,8 @@ int64_t lowrank_partial_floats(const ssm_plan_s* pl, int64_t grid);
 int lrtc_padded_rank(int r, bool three_d);
 int64_t lrtc_grid(const ssm_plan_s* pl);
 int64_t lrtc_partial_floats(const ssm_plan_s* pl, int64_t grid);
-int64_t lrtc_state_floats(const ssm_plan_s* pl);
 ssm_status lrtc_prepare(ssm_plan_s* pl);
 void lrtc_release(ssm_plan_s* pl);
-ssm_status lrtc_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, cudaStream_t s);
 ssm_status lrtc_split_basis(ssm_plan_s* pl, cudaStream_t s);
 ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                           int* nparts, cudaStream_t s);

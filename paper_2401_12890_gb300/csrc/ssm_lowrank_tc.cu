@@ -136,17 +136,6 @@ struct Lay {
   static_assert(T_U + 2 * RP * UB <= TMEM_COLS, "tensor memory");
 };
 
-// The tiles of a grid: patches of bx x by x bz voxels (lane = lx + bx (ly + by lz)), loaded
-// with a halo of one voxel on every axis with smoothness (h = 1) as X x Y x Z rows
-struct Patch {
-  int bx, by, bz, hx, hy, hz;
-  int X, Y, Z, rows;
-  int tx, ty, tz;            // tiles per axis
-  int64_t ntiles;
-  int naxes;                 // axes with smoothness (at least 1: see patch_of)
-  int zst;                   // bytes of the z rows, rounded up to 1024
-};
-
 struct LrtcMaps {
   CUtensorMap v1h, v1l;   // V (Q x RP), box {32, QC}, 128-byte swizzle
   CUtensorMap v2h, v2l;   // V^T (RP x Qs), box {QC, RP}, 128-byte swizzle
@@ -266,20 +255,6 @@ __device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, floa
                "f"(w)
                : "memory");
 }
-__device__ __forceinline__ void group_barrier(int id) {
-  asm volatile("bar.sync %0, 128;\n" ::"r"(id) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() {
-  asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-}
-// the thread's bulk stores have read their shared memory
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
-}
-
 // NAX: axes with smoothness (neighbour pairs per element)
 template <int RP, int NAX, bool CHECK, bool WD>
 __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ LrtcMaps maps,
@@ -743,7 +718,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           // the group's single buffer: the previous store has read it
           if (storer) bulk_wait_read();
           __syncwarp();
-          group_barrier(1 + grp);
+          named_barrier(1 + grp, 128);
         }
         // (the stages are 1024-byte-aligned: the piece index only flips bits 4-6)
         const uint32_t zb = in ? ring + sz * zst : zero;
@@ -851,7 +826,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
         // write it after the barrier
         if (nob == 2 && storer) bulk_wait_read();
         __syncwarp();
-        group_barrier(1 + grp);
+        named_barrier(1 + grp, 128);
         if (storer) {
           const unsigned char* ob_ = obuf + grp * nob * OB + (nob == 2 ? (own & 1) * OB : 0);
           tma_store_5d(&maps.zo, ob_, 0, x0, y0, z0, c0 + i);
@@ -940,39 +915,6 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   }
 }
 
-// F (Q x ldf, map-major) from the blocked z: a block transposes 128 voxels of a chunk
-// through shared memory (both sides coalesced; bound by memory)
-__global__ void __launch_bounds__(256) unblock_kernel(const float* __restrict__ Z, int64_t N,
-                                                      int Q, float* __restrict__ F,
-                                                      int64_t ldf) {
-  __shared__ float sm[QC][129];
-  const int64_t n0 = blockIdx.x * (int64_t)128;
-  const int c = blockIdx.y;
-  const float4* src = reinterpret_cast<const float4*>(Z) + ((int64_t)c * N + n0) * (QC / 4);
-  const int nv = (int)min((int64_t)128, N - n0);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int t = threadIdx.x + i * 256, n = t >> 3, j = t & 7;
-    if (n < nv) {
-      const float4 f = __ldg(src + t);
-      sm[4 * j][n] = f.x;
-      sm[4 * j + 1][n] = f.y;
-      sm[4 * j + 2][n] = f.z;
-      sm[4 * j + 3][n] = f.w;
-    }
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int r = w; r < QC; r += 8) {
-    const int q = c * QC + r;
-    if (q >= Q) break;
-    float* dst = F + (int64_t)q * ldf + n0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (lane + 32 * i < nv) dst[lane + 32 * i] = sm[r][lane + 32 * i];
-  }
-}
-
 // V (Q x RP) and V^T (RP x Qs), each split into TF32 hi/lo parts (round to nearest)
 __global__ void split_basis_kernel(const float* __restrict__ V32, int Q, int RP, int Qs,
                                    float* __restrict__ v1h, float* __restrict__ v1l,
@@ -989,36 +931,6 @@ __global__ void split_basis_kernel(const float* __restrict__ V32, int Q, int RP,
     v1h[(int64_t)q * RP + i] = h;
     v1l[(int64_t)q * RP + i] = l;
   }
-}
-
-// The patch of a grid's tiles: among all bx x by x bz <= 128 whose rows with halo fit the
-// staging area, the one with the least tiles x (a tile's fixed work + its staged rows). The
-// weight of the fixed work (300 rows) and the penalty for rows that do not start on
-// multiples of 8 (a quarter warp's 128-bit loads then meet in the same banks) only break
-// near-ties: 16 x 8 (2D) and 8 x 4 x 4 (3D) where the grid divides. An axis without
-// smoothness (one voxel, or the stacking axis of a batch) needs no halo; a single voxel
-// takes one on x (zero-filled rows), so that there is always a neighbour pair to read.
-constexpr int kMaxRows = 400;
-Patch patch_of(const Grid& g) {
-  Patch best{};
-  double cost = 1e300;
-  const int hy = g.ny > 1, hz = g.nz > 1 && g.zlink;
-  const int hx = g.nx > 1 || (!hy && !hz);
-  const int rmax = hx + hy + hz == 3 ? kMaxRows : 260;
-  for (int bz = 1; bz <= std::min(g.nz, TV); ++bz)
-    for (int by = 1; by <= std::min(g.ny, TV / bz); ++by)
-      for (int bx = 1; bx <= std::min(g.nx, TV / (bz * by)); ++bx) {
-        const int X = bx + 2 * hx, Y = by + 2 * hy, Z = bz + 2 * hz, rows = X * Y * Z;
-        if (rows > rmax) continue;
-        const int64_t tx = (g.nx + bx - 1) / bx, ty = (g.ny + by - 1) / by, tz = (g.nz + bz - 1) / bz;
-        const double c = (double)tx * ty * tz * (300 + rows + (bx % 8 ? 60 : 0));
-        if (c < cost) {
-          cost = c;
-          best = Patch{bx, by, bz, hx, hy, hz, X, Y, Z, rows, (int)tx, (int)ty, (int)tz,
-                       tx * ty * tz, hx + hy + hz, (rows * 128 + 1023) / 1024 * 1024};
-        }
-      }
-  return best;
 }
 
 // what a plan of this form keeps: the tiles, and the tensor maps of both ping-pong halves
@@ -1076,7 +988,7 @@ ssm_status launch_rn(const LrtcMaps& maps, const LrtcArgs& args, bool check, boo
 }
 
 int64_t ntiles_of(const ssm_plan_s* pl) {
-  if (pl->lrtc_state) return static_cast<const LrtcState*>(pl->lrtc_state)->p.ntiles;
+  if (pl->lr_state) return static_cast<const LrtcState*>(pl->lr_state)->p.ntiles;
   return patch_of(pl->g).ntiles;
 }
 int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
@@ -1138,9 +1050,6 @@ int lrtc_padded_rank(int r, bool three_d) {
   return 0;
 }
 
-// floats of one blocked state array
-int64_t lrtc_state_floats(const ssm_plan_s* pl) { return chunks_of(pl) * QC * pl->g.N; }
-
 int64_t lrtc_grid(const ssm_plan_s* pl) {
   int64_t grid;
   int spc, split;
@@ -1168,7 +1077,7 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
     SSM_TRY((prepare_rn<64, 2>()));
   }
   auto* st = new LrtcState();
-  pl->lrtc_state = st;
+  pl->lr_state = st;
   st->p = patch_of(pl->g);
   layout(pl, &pl->lr_grid, &st->spc, &st->split);
   const Patch& p = st->p;
@@ -1195,16 +1104,8 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
 }
 
 void lrtc_release(ssm_plan_s* pl) {
-  delete static_cast<LrtcState*>(pl->lrtc_state);
-  pl->lrtc_state = nullptr;
-}
-
-// F = z of ping-pong half `cur`
-ssm_status lrtc_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, cudaStream_t s) {
-  const dim3 grid((unsigned)((pl->g.N + 127) / 128), (unsigned)chunks_of(pl));
-  unblock_kernel<<<grid, 256, 0, s>>>(pl->Z[cur], pl->g.N, pl->Q, F, ldf);
-  SSM_LAUNCHED();
-  return SSM_OK;
+  delete static_cast<LrtcState*>(pl->lr_state);
+  pl->lr_state = nullptr;
 }
 
 // the TF32 hi/lo parts of V and V^T from the plan's FP32 basis V32 (Q x R)
@@ -1219,7 +1120,7 @@ ssm_status lrtc_split_basis(ssm_plan_s* pl, cudaStream_t s) {
 
 ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                           int* nparts, cudaStream_t s) {
-  const LrtcState& st = *static_cast<const LrtcState*>(pl->lrtc_state);
+  const LrtcState& st = *static_cast<const LrtcState*>(pl->lr_state);
   const int64_t grid = pl->lr_grid;
   LrtcArgs a;
   a.S = pl->S;
