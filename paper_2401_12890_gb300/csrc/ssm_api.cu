@@ -825,7 +825,7 @@ ssm_status one_iteration(ssm_plan_s* pl, int cur, bool check, bool check_next, i
   SSM_TRY(prof_mark(pl, true, s));
   if (pl->ndict > 0) {
     SSM_TRY(table_iteration(pl->tprob, pl->ttable, pl->tblocks, pl->R, cur, check, check_next,
-                            pl->red, s));
+                            pl->red, pl->chained, s));
     *nparts = (int)pl->tblocks;
     return prof_mark(pl, false, s);
   }

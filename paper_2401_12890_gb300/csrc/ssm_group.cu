@@ -212,17 +212,17 @@ ssm_status solve_impl(ssm_group_s* g, const float* const* M, const int64_t* ldm,
                       float* const* F, const int64_t* ldf, ssm_info* infos, cudaStream_t s) {
   const int np = (int)g->plans.size();
   std::vector<ProbRun> run(np);
+  bool clear_d = false;
+  for (ssm_plan_t pl : g->plans)
+    clear_d = clear_d || pl->p.max_iter <= 1 || pl->p.check_every == 1;
   for (int i = 0; i < np; ++i) {
     ssm_plan_s* pl = g->plans[i];
-    const size_t QN = (size_t)pl->Q * pl->g.ld;
     pl->has_state = false;   // the group's partial u is not the plan's: nothing to resume
-    // step 4: projections (FP64 accumulation); step 2: z = d = 0, u = 0
-    SSM_TRY(table_project(g->B[i], pl->P, g->R, nullptr, M[i], ldm[i], pl->g.N, g->S[i],
-                          pl->g.ld, s));
-    SSM_CUDA(cudaMemsetAsync(pl->Z[0], 0, sizeof(float) * QN, s));
-    SSM_CUDA(cudaMemsetAsync(pl->Dl[0], 0, sizeof(float) * QN, s));
-    SSM_CUDA(cudaMemsetAsync(
-        g->U0[i], 0, sizeof(float) * (size_t)table_state_floats(pl->g.N, g->nseg[i], g->R), s));
+    // step 4: projections (FP64 accumulation); step 2: z = d = 0, u = 0 (d^k is read only in
+    // a test, after the iteration before has stored it; any problem's test makes the launch
+    // read every problem's d)
+    SSM_TRY(group_start(g->probs, i, g->B[i], pl->P, pl->r, M[i], ldm[i], pl->g.N,
+                        table_state_floats(pl->g.N, g->nseg[i], g->R), g->R, clear_d, i > 0, s));
     run[i].active = pl->p.max_iter > 0;
     run[i].use_tol = pl->p.tol_primal > 0 || pl->p.tol_change > 0;
   }
@@ -250,6 +250,7 @@ ssm_status solve_impl(ssm_group_s* g, const float* const* M, const int64_t* ldm,
   };
   SSM_TRY(rebuild());
   int k = 0, cur = 0;
+  bool chained = false;            // the last launch was an iteration of the same table
   while (!act.empty()) {
     bool check = false, write_d = false;
     for (int i : act) {
@@ -257,7 +258,8 @@ ssm_status solve_impl(ssm_group_s* g, const float* const* M, const int64_t* ldm,
       write_d = write_d || is_check(g->plans[i]->p, k + 1);
     }
     SSM_TRY(table_iteration(g->probs, g->table, (int64_t)entries.size(), g->R, cur, check,
-                            write_d, g->red, s));
+                            write_d, g->red, chained, s));
+    chained = !check;
     cur ^= 1;
     ++k;
     if (!check) continue;

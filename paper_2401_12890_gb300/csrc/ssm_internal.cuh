@@ -73,10 +73,10 @@ __device__ __forceinline__ void pdl_wait() {
 // kernel must call pdl_wait before it touches anything an earlier launch reads or writes
 // since the chain began (every kernel of a chain waits, so completion is transitive).
 template <typename K, typename... A>
-ssm_status launch_chained(K kernel, unsigned grid, unsigned block, size_t shm, cudaStream_t s,
+ssm_status launch_chained(K kernel, dim3 grid, unsigned block, size_t shm, cudaStream_t s,
                           bool chained, const A&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = shm;
   cfg.stream = s;
@@ -148,7 +148,7 @@ struct TableProblem {
   float* Z[2];                      // z ping-pong (Q x ld)
   float* D[2];                      // d ping-pong (Q x ld; read/written around tests)
   float* U[2];                      // partial u per (tile, segment) [tile][seg][R][32]
-  const float* S;                   // R x ld: S_i = sigma_i u_i^T m per voxel
+  float* S;                         // R x ld: S_i = sigma_i u_i^T m per voxel
   const float* V;                   // Q x ndict x R  [q][c][i]: a compartment's rows of
                                     // every dictionary side by side
   const float* coefA;               // ndict x R: 1/(beta + sigma^2)
@@ -370,8 +370,11 @@ ssm_status table_project(const double* B, int P, int R, const int32_t* labels, c
                          int64_t ldm, int64_t N, float* S, int64_t ld, cudaStream_t s);
 // one iteration of every problem of the table (blocks = entries); z^k in Z[cur]
 ssm_status table_iteration(const TableProblem* probs, const int4* table, int64_t nblocks, int R,
-                           int cur, bool check, bool write_d, double* partial, cudaStream_t s);
-
+                           int cur, bool check, bool write_d, double* partial, bool chained,
+                           cudaStream_t s);
+ssm_status group_start(const TableProblem* probs, int i, const double* B, int P, int r,
+                       const float* M, int64_t ldm, int64_t N, int64_t ufloats, int R, bool clear_d,
+                       bool chained, cudaStream_t s);
 
 // dense iteration and shared kernels (ssm_dense.cu)
 ssm_status sgemm(int M, int N, int K, float alpha, const float* A, int64_t lda,

@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
   __shared__ float sh_a[R][VT];           // a_i of the tile's voxels
   __shared__ float sh_u[WPB][R][VT];      // the warps' partial u', summed in warp order
   __shared__ double sh_red[WPB][3];
+  pdl_launch_next();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int4 e = table[blockIdx.x];
@@ -108,10 +109,10 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
   bool hxm = false, hxp = false, hym = false, hyp = false, hzm = false, hzp = false;
   if (in) {
     c = P.labels ? P.labels[n] : 0;
-    const int x = (int)(n % nx);
-    const int64_t t = n / nx;
-    const int y = (int)(t % ny);
-    const int zc = (int)(t / ny);
+    const unsigned t = (unsigned)n / (unsigned)nx;
+    const int x = (int)((unsigned)n - t * (unsigned)nx);
+    const int y = (int)(t % (unsigned)ny);
+    const int zc = (int)(t / (unsigned)ny);
     hxm = x > 0;
     hxp = x < nx - 1;
     hym = y > 0;
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
 
   // a_i = S_i/(beta + sigma_{c,i}^2) - W_{c,i} u_i, u summed over the tile's segments of
   // the previous iteration in segment order
+  pdl_wait();       // what the previous iteration wrote is read from here on
   {
     // this warp's ranks i = warp + j WPB; slot by slot, their loads in flight together
     constexpr int RPW = R / WPB;
@@ -279,6 +281,46 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
   }
 }
 
+// A problem's start in a group: the projections (a block forms four ranks of 128 voxels, FP64
+// accumulation), z^0 = 0 (and d^0 where a first iteration tests) and u = 0. The launches of
+// a group's problems overlap (they are chained, and wait for one another only when their
+// work is done). One thread per voxel for all ranks, one launch after another and three
+// memsets each took 24 to 52 us per problem. 24 problems of six shapes, 100 iterations: 4.76 ->
+// 3.61 ms (with the iterations chained by programmatic dependent launch)
+__global__ void __launch_bounds__(MT) group_start_kernel(const TableProblem* __restrict__ probs,
+                                                         int problem, const double* __restrict__ B,
+                                                         int P, int r, const float* __restrict__ M,
+                                                         int64_t ldm, int64_t ufloats, int clear_d,
+                                                         int R) {
+  pdl_launch_next();
+  const TableProblem& pr = probs[problem];
+  const int64_t n = blockIdx.x * (int64_t)MT + threadIdx.x, ld = pr.g.ld;
+  const int i0 = blockIdx.y * 4;
+  if (n < pr.g.N) {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if (i0 < r) {
+#pragma unroll 4
+      for (int p = 0; p < P; ++p) {
+        const double m = (double)__ldg(M + (int64_t)p * ldm + n);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = fma(__ldg(B + (int64_t)p * R + i0 + j), m, acc[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) pr.S[(int64_t)(i0 + j) * ld + n] = (float)acc[j];
+  }
+  const int64_t zn = (int64_t)pr.Q * ld;
+  const int64_t t0 = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * MT + threadIdx.x;
+  const int64_t st = (int64_t)gridDim.x * gridDim.y * MT;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int64_t i = t0; i < zn / 4; i += st) {             // ld is a multiple of 128
+    reinterpret_cast<float4*>(pr.Z[0])[i] = zero;
+    if (clear_d) reinterpret_cast<float4*>(pr.D[0])[i] = zero;
+  }
+  for (int64_t i = t0; i < ufloats / 4; i += st) reinterpret_cast<float4*>(pr.U[0])[i] = zero;
+  pdl_wait();
+}
+
 // out[k] = alpha_i Bp[p][i] for i < r (sigma_i u_i), 0 for r <= i < R; k = p R + i
 __global__ void gather_b_kernel(const double* __restrict__ Bp, const double* __restrict__ alpha,
                                 int P, int n, int r, int R, double* __restrict__ out) {
@@ -374,8 +416,19 @@ ssm_status table_project(const double* B, int P, int R, const int32_t* labels, c
   return SSM_OK;
 }
 
+// the start of problem `i` of a group (B: its sigma_i u_i [P][R], r its rank, ufloats its
+// partial-u buffer's size); `chained`: right after another problem's
+ssm_status group_start(const TableProblem* probs, int i, const double* B, int P, int r,
+                       const float* M, int64_t ldm, int64_t N, int64_t ufloats, int R, bool clear_d,
+                       bool chained, cudaStream_t s) {
+  const dim3 grid((unsigned)((N + MT - 1) / MT), (unsigned)(R / 4));
+  return launch_chained(group_start_kernel, grid, MT, 0, s, chained, probs, i, B, P, r, M, ldm, ufloats,
+                        clear_d ? 1 : 0, R);
+}
+
 ssm_status table_iteration(const TableProblem* probs, const int4* table, int64_t nblocks, int R,
-                           int cur, bool check, bool write_d, double* partial, cudaStream_t s) {
+                           int cur, bool check, bool write_d, double* partial, bool chained,
+                           cudaStream_t s) {
   if (nblocks < 1 || nblocks > INT32_MAX) {
     set_error("work-table iteration: bad table size");
     return SSM_EINVAL;
@@ -385,19 +438,16 @@ ssm_status table_iteration(const TableProblem* probs, const int4* table, int64_t
   switch (R) {
 #define SSM_R(RR)                                                                           \
   case RR:                                                                                  \
-    if (check)                                                                              \
-      table_iter_kernel<RR, true><<<grid, VT * WPB, 0, s>>>(probs, table, cur, wd, partial); \
-    else                                                                                    \
-      table_iter_kernel<RR, false><<<grid, VT * WPB, 0, s>>>(probs, table, cur, wd, partial); \
-    break;
+    return check ? launch_chained(table_iter_kernel<RR, true>, grid, VT * WPB, 0, s, chained, \
+                                  probs, table, cur, wd, partial)                            \
+                 : launch_chained(table_iter_kernel<RR, false>, grid, VT * WPB, 0, s, chained, \
+                                  probs, table, cur, wd, partial);
     SSM_TABLE_RANKS(SSM_R)
 #undef SSM_R
     default:
       set_error("work-table iteration: unsupported padded rank");
       return SSM_EUNSUPPORTED;
   }
-  SSM_LAUNCHED();
-  return SSM_OK;
 }
 
 }  // namespace ssm
