@@ -226,8 +226,9 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
   if (in) {
     // UR rows' state loads issued together (memory-level parallelism of a latency-bound
     // loop; one row at a time measured 184 us, two 145, four 131, eight 136 at R = 8 on
-    // the 61-level fingerprinting stand-in)
-    constexpr int UR = R <= 16 ? 4 : 2;
+    // the 61-level fingerprinting stand-in; at R = 32 two rows took 3.60 ms for the group of
+    // 24 problems x 100 iterations, four 3.28)
+    constexpr int UR = 4;
     int q = qa;
 #pragma unroll 1
     for (; q + UR <= qb; q += UR) {
