@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
   uint64_t* eempty = efull + 4;     // epilogue stage consumed (4 warps: one half)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(eempty + 4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_launch_next();
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -319,6 +320,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
     if (lane == 0) {
       tma_prefetch_map(&maps.a_hi);
       tma_prefetch_map(&maps.b_hi);
+      pdl_wait();            // w is written by the iteration before
       int c = 0;
       for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
         const int vt = t / a.ntq, qt = t % a.ntq;
@@ -353,6 +355,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
             (unsigned)((UG * EZW + NR * UG * ENW + (C::DH ? 2 * UG * BM : 0)) * 4);
         tma_prefetch_map(&maps.ez_c);
         tma_prefetch_map(&maps.ez_n);
+        pdl_wait();
         int i = 0;
         for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
           const int vt = t / a.ntq, qt = t % a.ntq;
@@ -416,6 +419,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
     }
   } else {
     // ------------------------------------------------------------ accumulator drain
+    pdl_wait();              // z, d and w are read and written below
     const int quarter = warp & 3;                  // TMEM lanes 32*quarter .. +31
     const int row = quarter * 32 + lane;           // voxel within the tile
     const int half = NEPI == 8 ? (warp - 2) >> 2 : 0;   // which column groups this warp takes
@@ -801,9 +805,10 @@ ssm_status launch_gemm(const ssm_plan_s* pl, int cur, double* partial, cudaStrea
   a.xi = (float)pl->xi;
   a.lam_s = (float)pl->lam_s;
   a.inv_xb = (float)(1.0 / (pl->xi + pl->p.beta));
-  tc_gemm_kernel<BN, EPI, NRT><<<gemm_grid(pl, BN), NTHR, C::SMEM_BYTES, s>>>(m, a);
-  SSM_LAUNCHED();
-  return SSM_OK;
+  // the fused iterations of a block are chained (the two-kernel form's update is not)
+  const bool chained = EPI != EPI_STORE && pl->tc_fused && pl->chained;
+  return launch_chained(tc_gemm_kernel<BN, EPI, NRT>, (unsigned)gemm_grid(pl, BN), NTHR,
+                        C::SMEM_BYTES, s, chained, m, a);
 }
 
 // staged neighbour rows of the plan's grid: 4 on 3D grids, else at most 2
