@@ -311,7 +311,7 @@ def dominant_kernel(form, prec, Q, N, r, fused=0):
     if prec == "fp32":
         # (for Algorithm 1 the profiled time is the whole iteration, of which the x-step
         # product is this amount of work)
-        return ("sgemm_kernel", "ssm_dense.cu", "alu", 2.0 * Q * Q * N, "TFLOP/s", "sgemm_kernel")
+        return ("product_kernel", "ssm_dense.cu", "alu", 2.0 * Q * Q * N, "TFLOP/s", "product_kernel")
     key = {0: "tc_gemm_kernel", 1: "tc_gemm_kernel (fused, staged epilogue)",
            2: "tc_gemm_kernel (fused, register epilogue)"}[fused]
     return ("tc_gemm_kernel", "ssm_tc.cu", "tensor", 3 * 2.0 * Q * Q * N, "TFLOP/s", key)

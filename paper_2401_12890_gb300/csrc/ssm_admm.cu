@@ -9,7 +9,7 @@
 //
 // x-step: as in the full-rank LADMM form, M g is large against M (beta f - d_x) in
 // FP32, so h = M g is formed once per solve and x = h + M w with w = beta f - d_x (the
-// FP32 SIMT GEMM sgemm_kernel).
+// FP32 SIMT product of ssm_dense.cu).
 // z-step: on the free-boundary box grid D^T D = s L, L the Kronecker sum of path-graph
 // Laplacians, which the orthonormal DCT-II along each axis diagonalises: the path
 // Laplacian of n nodes has eigenvectors c_k(j) = a_k cos(pi (j + 1/2) k / n) (a_0 =
@@ -321,7 +321,7 @@ ssm_status admm_iteration(ssm_plan_s* pl, bool check, double* partial, int* npar
     admm_pre_kernel<false><<<eg, EW, 0, s>>>(st, pl->Q, pl->g, beta, partial);
   SSM_LAUNCHED();
   // x-step product: acc = M w
-  SSM_TRY(sgemm(pl->Q, (int)pl->g.N, pl->Q, 1.f, pl->Mq32, pl->Qp, st.w, pl->g.ld, 0.f, pl->Acc,
+  SSM_TRY(sgemm(pl->Q, (int)pl->g.N, pl->Q, pl->Mq32, pl->Qp, st.w, pl->g.ld, pl->Acc,
                 pl->g.ld, s));
   // z-step: forward transforms along every axis longer than 1, scaling, inverse transforms;
   // the data ping-pong between r and t and the last inverse writes z

@@ -838,10 +838,10 @@ ssm_status one_iteration(ssm_plan_s* pl, int cur, bool check, bool check_next, i
   }
   if (p.precision == SSM_FP32) {
     // acc = M w (w^0 = 0, so the first product is 0)
-    SSM_TRY(sgemm(pl->Q, (int)pl->g.N, pl->Q, 1.f, pl->Mq32, pl->Qp, pl->Wf, pl->g.ld, 0.f,
-                  pl->Acc, pl->g.ld, s));
+    SSM_TRY(sgemm(pl->Q, (int)pl->g.N, pl->Q, pl->Mq32, pl->Qp, pl->Wf, pl->g.ld, pl->Acc, pl->g.ld,
+                  s));
     SSM_TRY(prof_mark(pl, false, s));
-    return dense_update(pl, cur, pl->Acc, check, true, false, pl->red, nparts, s);
+    return dense_update(pl, cur, pl->Acc, check, pl->red, nparts, s);
   }
   if (pl->tc_fused) {
     // one kernel: the product M w with the element-wise steps in its epilogue

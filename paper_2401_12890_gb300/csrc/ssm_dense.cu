@@ -7,92 +7,13 @@
 //     f = h + M w,   h = M g (formed once per solve),   w = beta z - d,
 // and runs the Q x Q by Q x N contraction on w only. The update kernel then applies
 // the z-step (Eq. 31 with the nonnegativity projection) and the dual step, and
-// writes the next w (FP32 for this form, or the BF16 hi/lo pair for the tensor-core
-// form), so one iteration is: sgemm (M w) -> dense_update.
+// writes the next w, so one iteration is: sgemm (M w) -> dense_update.
 #include <algorithm>
 
 #include "ssm_internal.cuh"
 
 namespace ssm {
 namespace {
-
-// ---------------------------------------------------------------------------
-// C (M x N) = alpha * A (M x K) B (K x N) + beta * C, all row-major FP32.
-// 128 x 128 block tile, 8-deep k slices double-buffered in shared memory,
-// 8 x 8 outputs per thread, FP32 accumulation.
-// ---------------------------------------------------------------------------
-constexpr int BM = 128, BN = 128, BK = 8;
-
-__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, float alpha,
-                                                    const float* __restrict__ A, int64_t lda,
-                                                    const float* __restrict__ B, int64_t ldb,
-                                                    float beta, float* __restrict__ C,
-                                                    int64_t ldc) {
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
-  const int tid = threadIdx.x;
-  const int ty = tid >> 4, tx = tid & 15;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  // loader mapping: A tile 128 x 8 -> row tid/2, k (tid&1)*4..+4
-  //                 B tile 8 x 128 -> k tid/32, col (tid&31)*4..+4
-  const int ar = tid >> 1, ak = (tid & 1) * 4;
-  const int bk = tid >> 5, bc = (tid & 31) * 4;
-  float ra[4], rb[4];
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gm = m0 + ar, gk = k0 + ak + j;
-      ra[j] = (gm < M && gk < K) ? __ldg(A + (int64_t)gm * lda + gk) : 0.f;
-      const int gk2 = k0 + bk, gn = n0 + bc + j;
-      rb[j] = (gk2 < K && gn < N) ? __ldg(B + (int64_t)gk2 * ldb + gn) : 0.f;
-    }
-  };
-  auto store = [&](int buf) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) As[buf][ak + j][ar] = ra[j];
-    *reinterpret_cast<float4*>(&Bs[buf][bk][bc]) = make_float4(rb[0], rb[1], rb[2], rb[3]);
-  };
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  const int ntile = (K + BK - 1) / BK;
-  load(0);
-  store(0);
-  __syncthreads();
-  for (int kt = 0; kt < ntile; ++kt) {
-    const int buf = kt & 1;
-    if (kt + 1 < ntile) load((kt + 1) * BK);
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][64 + tx * 4]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    if (kt + 1 < ntile) store(buf ^ 1);
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int gm = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-    if (gm >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int gn = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
-      if (gn >= N) continue;
-      float* c = C + (int64_t)gm * ldc + gn;
-      *c = beta == 0.f ? alpha * acc[i][j] : fmaf(alpha, acc[i][j], beta * *c);
-    }
-  }
-}
 
 // ---------------------------------------------------------------------------
 // z-step (Eq. 31 + projection) and dual step for the full-rank form
@@ -109,9 +30,7 @@ struct UpdateArgs {
   const float* __restrict__ Din;
   float* __restrict__ Zout;
   float* __restrict__ Dout;
-  float* __restrict__ Wf;            // optional FP32 w'
-  __nv_bfloat16* __restrict__ Whi;   // optional BF16 split of w'
-  __nv_bfloat16* __restrict__ Wlo;
+  float* __restrict__ Wf;            // w'
   double* __restrict__ partial;
   const uint8_t* __restrict__ mask;  // voxels inside the object (nullptr: every voxel)
   Grid g;
@@ -160,12 +79,7 @@ __global__ void __launch_bounds__(UV) dense_update_kernel(UpdateArgs a) {
       const float w = a.beta * zn - dn;
       a.Zout[o] = zn;
       a.Dout[o] = dn;
-      if (a.Wf) a.Wf[o] = w;
-      if (a.Whi) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(w);
-        a.Whi[o] = h;
-        a.Wlo[o] = __float2bfloat16_rn(w - __bfloat162float(h));
-      }
+      a.Wf[o] = w;
       if (CHECK) {
         const float e = zn - f, c = zn - z;
         s1 = fmaf(e, e, s1);
@@ -228,14 +142,16 @@ __device__ __forceinline__ void cp_async(float* dst, const float* src, int n) {
                  : "memory");
 }
 
-struct ResidualArgs {
-  int P, N, Q;
-  const float* __restrict__ Kt;       // K^T: Q x P, row stride ldk
-  int64_t ldk;
-  const float* __restrict__ F;
-  int64_t ldf;
-  const float* __restrict__ M;
-  int64_t ldm;
+struct ProductArgs {
+  int M, N, K;
+  const float* __restrict__ At;       // A transposed: K x M, row stride lda
+  int64_t lda;
+  const float* __restrict__ B;        // K x N, row stride ldb
+  int64_t ldb;
+  float* __restrict__ C;              // A B (store)
+  int64_t ldc;
+  const float* __restrict__ D;        // residual: sum (D - A B)^2
+  int64_t ldd;
   const uint8_t* __restrict__ mask;   // voxels inside the object (nullptr: every voxel)
   double* __restrict__ partial;       // 4 doubles per CTA
 };
@@ -324,24 +240,27 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
                     partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 4);
 }
 
-// The objective's data term: sum (M - K F)^2 over the voxels inside the object, K F in FP32,
-// each product one FMA chain over the compartments in ascending order (so the residuals
-// depend on neither the tile shape nor the grid), squares and sums in FP64. K is given
-// transposed, so that both operands' compartment slices are rows.
+// A B for the full-rank FP32 forms (C = A B), or the objective's data term, sum (D - A B)^2
+// over the voxels inside the object with squares and sums in FP64. FP32, each product one
+// FMA chain over k in ascending order (so the results depend on neither the tile shape nor
+// the grid). A is given transposed (K^T, or the symmetric M), so that both operands' k
+// slices are rows.
 //
 // Bound: the FP32 pipe (128 FMA per SM and cycle), and next to it the shared-memory pipe. A
-// thread owns 16 rows x 4 voxels and a warp 16 rows x 128 voxels: the rows' K values are
+// thread owns 16 rows x 4 columns and a warp 16 rows x 128 columns: the rows' A values are
 // the same for every lane (broadcast reads), which takes 8 shared-memory wavefronts per 64
 // FMAs of a warp against the 12 of 8 x 8 outputs per thread, whose reads queued behind one
-// another. Slices of 8 compartments come by cp.async into a ring of NST stages, and the
-// fragments of slice entry k + 1 are read while those of k are multiplied. Tiles of 64
-// rows (4 warps) spread a small problem evenly over the SMs; 128 (8 warps) where that
-// gives every SM two CTAs. P = 120, Q = 2500, N = 16384 (the 128 x 128 slice): 313 -> 278 us
-// in ncu, with sgemm_kernel's 128 CTAs before.
-// VEC: the rows of K^T and F are 16-byte aligned (else scalar copies)
-template <int BM, bool VEC>
+// another. Slices of 8 k come by cp.async into a ring of NST stages, and the fragments of
+// slice entry k + 1 are read while those of k are multiplied. Tiles of 64 rows (4 warps)
+// spread a small problem evenly over the SMs; 128 (8 warps) where that gives every SM two
+// CTAs. Against 128 x 128 tiles with the next slice held in registers: M = K = 300, N =
+// 6048 (144 CTAs then) 57.5 -> 49.2 us per iteration with the update, M = K = 225, N = 1024 43.4 ->
+// 24.9 us, M = K = 2500, N = 16384 4858 -> 4700 us, M = 120, K = 2500, N = 16384 (the
+// objective's) 313 -> 278 us in ncu
+// VEC: the rows of A^T and B are 16-byte aligned (else scalar copies)
+template <int BM, bool RESIDUAL, bool VEC>
 __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
-    residual_kernel(const ResidualArgs a) {
+    product_kernel(const ProductArgs a) {
   constexpr int BN = 128;
   constexpr int T = 2 * BM;                        // 16 x 4 outputs each
   constexpr int BK = 8;
@@ -352,7 +271,7 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
   __shared__ __align__(16) float ring[NST * STAGE];
   const int tid = threadIdx.x;
   const int r16 = (tid >> 5) * 16, c4 = (tid & 31) * 4;   // this thread's rows and columns
-  const int M = a.P, N = a.N, K = a.Q;
+  const int M = a.M, N = a.N, K = a.K;
   const int mt = (M + BM - 1) / BM;
   const int m0 = ((int)blockIdx.x % mt) * BM, n0 = ((int)blockIdx.x / mt) * BN;
   const int ntile = (K + BK - 1) / BK;
@@ -372,12 +291,12 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
 #pragma unroll
     for (int i = 0; i < LA; ++i) {
       const int f = tid + i * T, kk = f / (BM / 4), c = (f % (BM / 4)) * 4;
-      copy4(st + kk * BM + c, a.Kt, a.ldk, kt * BK + kk, m0 + c, M);
+      copy4(st + kk * BM + c, a.At, a.lda, kt * BK + kk, m0 + c, M);
     }
 #pragma unroll
     for (int i = 0; i < LB; ++i) {
       const int f = tid + i * T, kk = f / (BN / 4), c = (f % (BN / 4)) * 4;
-      copy4(st + BK * BM + kk * BN + c, a.F, a.ldf, kt * BK + kk, n0 + c, N);
+      copy4(st + BK * BM + kk * BN + c, a.B, a.ldb, kt * BK + kk, n0 + c, N);
     }
   };
   auto commit = [] { asm volatile("cp.async.commit_group;\n" ::: "memory"); };
@@ -431,32 +350,49 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
       }
     }
   }
-  double r2 = 0.0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int gn = n0 + c4 + j;
-    if (gn >= N || (a.mask && !a.mask[gn])) continue;
+  if constexpr (!RESIDUAL) {
+    const bool vec = a.ldc % 4 == 0 && n0 + c4 + 3 < N;    // (C is 16-byte aligned)
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int gm = m0 + r16 + i;
-      if (gm >= M) continue;
-      const float r = __fsub_rn(__ldg(a.M + (int64_t)gm * a.ldm + gn), acc[i][j]);
-      r2 += (double)r * r;
+      if (gm >= M) break;
+      float* c = a.C + (int64_t)gm * a.ldc + n0 + c4;
+      if (vec) {
+        *reinterpret_cast<float4*>(c) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (n0 + c4 + j < N) c[j] = acc[i][j];
+      }
     }
+  } else {
+    double r2 = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int gn = n0 + c4 + j;
+      if (gn >= N || (a.mask && !a.mask[gn])) continue;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int gm = m0 + r16 + i;
+        if (gm >= M) continue;
+        const float r = __fsub_rn(__ldg(a.D + (int64_t)gm * a.ldd + gn), acc[i][j]);
+        r2 += (double)r * r;
+      }
+    }
+    block_partial<T>(r2, 0.0, 0.0, a.partial + (int64_t)blockIdx.x * 4);
   }
-  block_partial<T>(r2, 0.0, 0.0, a.partial + (int64_t)blockIdx.x * 4);
 }
 
 // rows per tile: 128 where that gives every SM two CTAs and pads no rows that 64 would not
 // (by more than a tenth), else 64
-int residual_rows(int64_t M, int64_t N) {
+int product_rows(int64_t M, int64_t N) {
   auto up = [](int64_t v, int64_t b) { return (v + b - 1) / b; };
   const int64_t big = up(M, 128) * up(N, 128), small = up(M, 64) * up(N, 128);
   return big >= 2 * (int64_t)sm_count() && 20 * big <= 11 * small ? 128 : 64;
 }
 
-int64_t residual_ctas(int64_t M, int64_t N) {
-  const int64_t b = residual_rows(M, N);
+int64_t product_ctas(int64_t M, int64_t N) {
+  const int64_t b = product_rows(M, N);
   return (M + b - 1) / b * ((N + 127) / 128);
 }
 
@@ -468,23 +404,50 @@ int rough_chunks(const ssm_plan_s* pl, int* chunk) {
   return (pl->Q + *chunk - 1) / *chunk;
 }
 
-}  // namespace
-
-ssm_status sgemm(int M, int N, int K, float alpha, const float* A, int64_t lda, const float* B,
-                 int64_t ldb, float beta, float* C, int64_t ldc, cudaStream_t s) {
-  if (M <= 0 || N <= 0) return SSM_OK;
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-  sgemm_kernel<<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+template <bool RESIDUAL>
+ssm_status launch_product(const ProductArgs& a, cudaStream_t s) {
+  if (a.M <= 0 || a.N <= 0) return SSM_OK;
+  const int64_t ctas = product_ctas(a.M, a.N);
+  if (ctas > INT32_MAX) {
+    set_error("matrix product: too many tiles");
+    return SSM_EINVAL;
+  }
+  const bool big = product_rows(a.M, a.N) == 128;
+  const bool vec = a.lda % 4 == 0 && a.ldb % 4 == 0 &&
+                   ((reinterpret_cast<uintptr_t>(a.At) | reinterpret_cast<uintptr_t>(a.B)) & 15) == 0;
+  const unsigned gr = (unsigned)ctas;
+  if (big && vec) product_kernel<128, RESIDUAL, true><<<gr, 256, 0, s>>>(a);
+  else if (big) product_kernel<128, RESIDUAL, false><<<gr, 256, 0, s>>>(a);
+  else if (vec) product_kernel<64, RESIDUAL, true><<<gr, 128, 0, s>>>(a);
+  else product_kernel<64, RESIDUAL, false><<<gr, 128, 0, s>>>(a);
   SSM_LAUNCHED();
   return SSM_OK;
+}
+
+}  // namespace
+
+// C = A B with A given transposed (K x M)
+ssm_status sgemm(int M, int N, int K, const float* At, int64_t lda, const float* B, int64_t ldb,
+                 float* C, int64_t ldc, cudaStream_t s) {
+  ProductArgs a{};
+  a.M = M;
+  a.N = N;
+  a.K = K;
+  a.At = At;
+  a.lda = lda;
+  a.B = B;
+  a.ldb = ldb;
+  a.C = C;
+  a.ldc = ldc;
+  return launch_product<false>(a, s);
 }
 
 int dense_max_partials(const ssm_plan_s* pl) {
   return (int)(((pl->g.N + UV - 1) / UV) * ((pl->Q + UQ - 1) / UQ));
 }
 
-ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check, bool write_fp32_w,
-                        bool write_bf16_w, double* partial, int* nparts, cudaStream_t s) {
+ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check, double* partial,
+                        int* nparts, cudaStream_t s) {
   UpdateArgs a;
   a.acc = acc;
   a.H = pl->H;
@@ -492,9 +455,7 @@ ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check, b
   a.Din = pl->Dl[cur];
   a.Zout = pl->Z[cur ^ 1];
   a.Dout = pl->Dl[cur ^ 1];
-  a.Wf = write_fp32_w ? pl->Wf : nullptr;
-  a.Whi = write_bf16_w ? pl->Whi[cur ^ 1] : nullptr;
-  a.Wlo = write_bf16_w ? pl->Wlo[cur ^ 1] : nullptr;
+  a.Wf = pl->Wf;
   a.partial = partial;
   a.mask = pl->mask;
   a.g = pl->g;
@@ -505,6 +466,9 @@ ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check, b
   a.inv_xb = (float)(1.0 / (pl->xi + pl->p.beta));
   dim3 grid((unsigned)((pl->g.N + UV - 1) / UV), (unsigned)((pl->Q + UQ - 1) / UQ));
   *nparts = (int)(grid.x * grid.y);
+  // (ordinary launches: chained by programmatic dependent launch, the next kernel's waiting
+  // blocks took the product's places on the SMs: 49 -> 60 us per iteration on the masked
+  // 84 x 72 workload)
   if (check)
     dense_update_kernel<true><<<grid, UV, 0, s>>>(a);
   else
@@ -523,7 +487,7 @@ ssm_status finish_partials(const double* partial, int nparts, int width, double*
 int objective_partials(const ssm_plan_s* pl) {
   int chunk;
   const int64_t rough = (pl->g.N + RT - 1) / RT * rough_chunks(pl, &chunk);
-  return (int)std::min<int64_t>(INT32_MAX, residual_ctas(pl->P, pl->g.N) + rough);
+  return (int)std::min<int64_t>(INT32_MAX, product_ctas(pl->P, pl->g.N) + rough);
 }
 
 // ||M - K F||^2 and the sum over neighbour pairs of the squared differences of F, as
@@ -531,31 +495,20 @@ int objective_partials(const ssm_plan_s* pl) {
 ssm_status objective_terms(const ssm_plan_s* pl, const float* Kt, const float* M, int64_t ldm,
                            const float* F, int64_t ldf, double* partial, int* nparts,
                            cudaStream_t s) {
-  ResidualArgs a;
-  a.P = pl->P;
+  ProductArgs a{};
+  a.M = pl->P;
   a.N = (int)pl->g.N;
-  a.Q = pl->Q;
-  a.Kt = Kt;
-  a.ldk = (pl->P + 3) / 4 * 4;
-  a.F = F;
-  a.ldf = ldf;
-  a.M = M;
-  a.ldm = ldm;
+  a.K = pl->Q;
+  a.At = Kt;
+  a.lda = (pl->P + 3) / 4 * 4;
+  a.B = F;
+  a.ldb = ldf;
+  a.D = M;
+  a.ldd = ldm;
   a.mask = pl->mask;
   a.partial = partial;
-  const int64_t ctas = residual_ctas(pl->P, pl->g.N);
-  if (ctas > INT32_MAX) {
-    set_error("objective: too many tiles");
-    return SSM_EINVAL;
-  }
-  const bool big = residual_rows(pl->P, pl->g.N) == 128;
-  const bool vec = ldf % 4 == 0 && (reinterpret_cast<uintptr_t>(F) & 15) == 0;
-  const unsigned gr = (unsigned)ctas;
-  if (big && vec) residual_kernel<128, true><<<gr, 256, 0, s>>>(a);
-  else if (big) residual_kernel<128, false><<<gr, 256, 0, s>>>(a);
-  else if (vec) residual_kernel<64, true><<<gr, 128, 0, s>>>(a);
-  else residual_kernel<64, false><<<gr, 128, 0, s>>>(a);
-  SSM_LAUNCHED();
+  SSM_TRY(launch_product<true>(a, s));
+  const int64_t ctas = product_ctas(pl->P, pl->g.N);
   int chunk;
   const int chunks = rough_chunks(pl, &chunk);
   const dim3 grid((unsigned)((pl->g.N + RT - 1) / RT), (unsigned)chunks);

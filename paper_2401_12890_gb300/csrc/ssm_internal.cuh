@@ -377,12 +377,11 @@ ssm_status group_start(const TableProblem* probs, int i, const double* B, int P,
                        bool chained, cudaStream_t s);
 
 // dense iteration and shared kernels (ssm_dense.cu)
-ssm_status sgemm(int M, int N, int K, float alpha, const float* A, int64_t lda,
-                 const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
-                 cudaStream_t s);
-ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check,
-                        bool write_fp32_w, bool write_bf16_w, double* partial, int* nparts,
-                        cudaStream_t s);
+// C = A B with A given transposed (the full-rank M is symmetric)
+ssm_status sgemm(int M, int N, int K, const float* At, int64_t lda, const float* B, int64_t ldb,
+                 float* C, int64_t ldc, cudaStream_t s);
+ssm_status dense_update(ssm_plan_s* pl, int cur, const float* acc, bool check, double* partial,
+                        int* nparts, cudaStream_t s);
 int dense_max_partials(const ssm_plan_s* pl);
 ssm_status finish_partials(const double* partial, int nparts, int width, double* out,
                            cudaStream_t s);
