@@ -284,6 +284,9 @@ struct ssm_plan_s {
   // the iteration about to be launched directly follows another of the same block in its
   // stream (set by run_block)
   bool chained = false;
+  // the iteration about to be launched starts from z = 0 (set by run_block): the low-rank
+  // forms then read no z
+  bool from_zero = false;
   // iteration blocks replayed as CUDA graphs (ssm_plan_set_graphs)
   bool use_graphs = false;
   std::vector<ssm::GraphBlock> graphs;

@@ -120,6 +120,7 @@ ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, 
   a.Pout = pl->U[cur ^ 1];
   a.nst = (pl->Q + QS - 1) / QS;
   a.nseg = st.nseg;
+  a.coff = pl->from_zero ? (pl->Q + 31) / 32 : 0;
   a.nb = a.nob = 0;                  // set per variant (the launch)
   a.coefA = pl->coefA;
   a.coefW = pl->coefW;

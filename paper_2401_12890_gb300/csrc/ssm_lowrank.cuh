@@ -72,6 +72,8 @@ struct LowrankArgs {
   const float* __restrict__ Pin;    // partial u of the previous iteration [tile][seg][R][TV]
   float* __restrict__ Pout;         // partial u of this iteration
   int nst;                          // stages per tile: ceil(Q / QS)
+  int coff;                         // added to the chunk of the z loads: past the tensor (all
+                                    // zeros, nothing read) in an iteration from z = 0
   int nseg;                         // segments per tile
   int nb, nob;                      // ring stages; z' (and d') buffers, 1 or 2
   const float* __restrict__ coefA;  // R
@@ -194,7 +196,8 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
           unsigned char* st = smem + b * stb;
           mbar_arrive_expect_tx(&full[b], bytes);
           const int q0 = (t & 1) * QS, ch = t >> 1;
-          tma_load_5d(st, &maps.zi, q0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, ch, &full[b]);
+          tma_load_5d(st, &maps.zi, q0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, ch + a.coff,
+                      &full[b]);
           unsigned char* vs = st + rb;
           if (CHECK) {
             tma_load_5d(vs, &maps.di, q0, x0, y0, z0, ch, &full[b]);

@@ -151,6 +151,8 @@ struct LrtcArgs {
   int spc;                          // segments per tile (each a contiguous run of chunks)
   int split;                        // > 0: main/tail layout, the chunk where tails start
   int kr;                           // K steps of 8 ranks holding the rank r (<= RP / 8)
+  int coff;                         // added to the chunk of the z loads: past the tensor (all
+                                    // zeros, nothing read) in an iteration from z = 0
   int nsz, nob;                     // z stages; z' (and d') buffers per group, 1 or 2
   const float* __restrict__ coefA;  // RP
   const float* __restrict__ coefW;  // RP
@@ -409,7 +411,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           unsigned char* zs = zring + sz * zst;
           uint64_t* bar = &zfull[2 * sz + (kz & 1)];
           mbar_arrive_expect_tx(bar, zbytes);
-          tma_load_5d(zs, &maps.zi, 0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, c, bar);
+          tma_load_5d(zs, &maps.zi, 0, x0 - a.p.hx, y0 - a.p.hy, z0 - a.p.hz, c + a.coff, bar);
           if (CHECK) tma_load_5d(zs + a.p.zst, &maps.di, 0, x0, y0, z0, c, bar);
         }
       }
@@ -1131,6 +1133,7 @@ ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, dou
   a.split = st.split;
   a.kr = std::max(1, std::min(pl->R / 8, (pl->r + 7) / 8));
   a.nsz = a.nob = 0;                 // set per variant (launch_one)
+  a.coff = pl->from_zero ? a.nch : 0;
   a.coefA = pl->coefA;
   a.coefW = pl->coefW;
   a.partial = partial;
