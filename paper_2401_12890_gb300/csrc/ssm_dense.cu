@@ -251,18 +251,24 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
 // the same for every lane (broadcast reads), which takes 8 shared-memory wavefronts per 64
 // FMAs of a warp against the 12 of 8 x 8 outputs per thread, whose reads queued behind one
 // another. Slices of 8 k come by cp.async into a ring of NST stages, and the fragments of
-// slice entry k + 1 are read while those of k are multiplied. Tiles of 64 rows (4 warps)
-// spread a small problem evenly over the SMs; 128 (8 warps) where that gives every SM two
-// CTAs. Against 128 x 128 tiles with the next slice held in registers: M = K = 300, N =
-// 6048 (144 CTAs then) 57.5 -> 49.2 us per iteration with the update, M = K = 225, N = 1024 43.4 ->
-// 24.9 us, M = K = 2500, N = 16384 4858 -> 4700 us, M = 120, K = 2500, N = 16384 (the
-// objective's) 313 -> 278 us in ncu
+// slice entry k + 1 are read while those of k are multiplied. Tiles of 64 rows x 128 columns
+// (4 warps, three CTAs per SM): CTAs that wait for their own slices only, and a shorter last
+// wave. Against tiles of 128 rows (8 warps, two CTAs): M = K = 2500, N = 16384 4704 -> 4605 us
+// per iteration with the update, M = K = 1600, N = 589824 71.1 -> 67.2 ms, M = K = 900,
+// N = 36864 1700 -> 1525 us, M = K = 300, N = 6048 53.7 -> 47.9 us; the objective with M = 64,
+// K = 1600, N = 589824 6851 -> 4011 us (half of a 128-row tile is padding there), with M = 1000,
+// K = 900, N = 36864 1722 -> 1579 us. Against 128 x 128 tiles with the next slice held in
+// registers: M = K = 300, N = 6048 57.5 us, M = K = 225, N = 1024 43.4 us (now 24.9), M = K =
+// 2500, N = 16384 4858 us, M = 120, K = 2500, N = 16384 (the objective's product) 313 -> 278
+// us in ncu
 // VEC: the rows of A^T and B are 16-byte aligned (else scalar copies)
-template <int BM, bool RESIDUAL, bool VEC>
-__global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
+constexpr int PM = 64;
+
+template <bool RESIDUAL, bool VEC>
+__global__ void __launch_bounds__(2 * PM, 3)
     product_kernel(const ProductArgs a) {
   constexpr int BN = 128;
-  constexpr int T = 2 * BM;                        // 16 x 4 outputs each
+  constexpr int BM = PM, T = 2 * BM;               // 16 x 4 outputs each
   constexpr int BK = 8;
   constexpr int NST = 4;                           // stages
   constexpr int STAGE = BK * (BM + BN);            // floats per stage: A slice, B slice
@@ -383,17 +389,8 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 3)
   }
 }
 
-// rows per tile: 128 where that gives every SM two CTAs and pads no rows that 64 would not
-// (by more than a tenth), else 64
-int product_rows(int64_t M, int64_t N) {
-  auto up = [](int64_t v, int64_t b) { return (v + b - 1) / b; };
-  const int64_t big = up(M, 128) * up(N, 128), small = up(M, 64) * up(N, 128);
-  return big >= 2 * (int64_t)sm_count() && 20 * big <= 11 * small ? 128 : 64;
-}
-
 int64_t product_ctas(int64_t M, int64_t N) {
-  const int64_t b = product_rows(M, N);
-  return (M + b - 1) / b * ((N + 127) / 128);
+  return (M + PM - 1) / PM * ((N + 127) / 128);
 }
 
 // Compartment chunks of the roughness sum: about 8 CTAs per SM, at least 16 maps each
@@ -412,14 +409,11 @@ ssm_status launch_product(const ProductArgs& a, cudaStream_t s) {
     set_error("matrix product: too many tiles");
     return SSM_EINVAL;
   }
-  const bool big = product_rows(a.M, a.N) == 128;
   const bool vec = a.lda % 4 == 0 && a.ldb % 4 == 0 &&
                    ((reinterpret_cast<uintptr_t>(a.At) | reinterpret_cast<uintptr_t>(a.B)) & 15) == 0;
   const unsigned gr = (unsigned)ctas;
-  if (big && vec) product_kernel<128, RESIDUAL, true><<<gr, 256, 0, s>>>(a);
-  else if (big) product_kernel<128, RESIDUAL, false><<<gr, 256, 0, s>>>(a);
-  else if (vec) product_kernel<64, RESIDUAL, true><<<gr, 128, 0, s>>>(a);
-  else product_kernel<64, RESIDUAL, false><<<gr, 128, 0, s>>>(a);
+  if (vec) product_kernel<RESIDUAL, true><<<gr, 2 * PM, 0, s>>>(a);
+  else product_kernel<RESIDUAL, false><<<gr, 2 * PM, 0, s>>>(a);
   SSM_LAUNCHED();
   return SSM_OK;
 }
