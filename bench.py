@@ -306,7 +306,7 @@ def dominant_kernel(form, prec, Q, N, r, fused=0):
         if prec == "tf32x3":
             return ("lrtc_kernel", "ssm_lowrank_tc.cu", "hbm", 8.0 * Q * N + 12.0 * r * N,
                     "GB/s", "lrtc_kernel")
-        return ("lowrank_iter_kernel", "ssm_lowrank.cu", "hbm",
+        return ("lowrank_iter_kernel", "ssm_lowrank.cuh", "hbm",
                 8.0 * Q * N + 12.0 * r * N, "GB/s", "lowrank_iter_kernel")
     if prec == "fp32":
         # (for Algorithm 1 the profiled time is the whole iteration, of which the x-step
@@ -783,11 +783,11 @@ def bench_multidict():
     rec["lowrank_fp32_multi"] = {
         "us_per_iteration": 1e3 * per_it, "value": w.N * w.Q / (per_it / 1e3), "unit": METRIC,
         "rank": r, "plan_s": plan_s, "segments_grid": launch.get("lowrank_grid"),
-        "roofline": {"bound": "hbm", "kernel": "table_iter_kernel", "achieved": achieved,
+        "roofline": {"bound": "hbm", "kernel": "lowrank_iter_kernel", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "main_kernel_ms_avg": kms / max(kl, 1),
                      "algorithmic_per_launch": amount,
-                     "traffic": traffic_record("ssm_table.cu", "table_iter_kernel",
+                     "traffic": traffic_record("ssm_lowrank.cuh", "lowrank_iter_kernel",
                                                w.name)},
         "err_vs_oracle": {"voxels": 3, "iterations": n_err, "max_rel_l2": max(errs),
                           "oracle": "FP64 oracle.multidict on each voxel's patch"}}

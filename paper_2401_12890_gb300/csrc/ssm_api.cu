@@ -96,7 +96,7 @@ double dtd_norm_closed(const int64_t* dims, int ndim, int pairs) {
 
 // floats of one partial-u buffer of the low-rank forms
 int64_t lowrank_state_floats(const ssm_plan_s* pl, int64_t grid) {
-  if (pl->ndict > 0) return table_state_floats(pl->g.N, pl->mseg, pl->R);
+  if (pl->ndict > 0 && !pl->multi_patches) return table_state_floats(pl->g.N, pl->mseg, pl->R);
   return pl->p.precision == SSM_TF32X3 ? lrtc_partial_floats(pl, grid)
                                        : lowrank_partial_floats(pl, grid);
 }
@@ -105,9 +105,9 @@ int64_t lowrank_state_floats(const ssm_plan_s* pl, int64_t grid) {
 // runs low-rank FP32 plans in their buffers map-major: room for either)
 int64_t state_floats(const ssm_plan_s* pl) {
   const int64_t flat = (int64_t)pl->Q * pl->g.ld;
-  if (pl->p.form != SSM_FORM_LOWRANK || pl->ndict > 0) return flat;
+  if (pl->p.form != SSM_FORM_LOWRANK || (pl->ndict > 0 && !pl->multi_patches)) return flat;
   const int64_t blocked = blocked_floats(pl->g, pl->Q);
-  return pl->p.precision == SSM_TF32X3 ? blocked : std::max(flat, blocked);
+  return pl->p.precision == SSM_TF32X3 || pl->ndict > 0 ? blocked : std::max(flat, blocked);
 }
 
 int padded_rank(int r) {
@@ -559,11 +559,15 @@ ssm_status multi_plan_impl(ssm_plan_s* pl, int ndict, const double* K_host,
   }
   pl->r = rmax;
   pl->R = table_padded_rank(rmax);
+  pl->multi_patches = lowrank_multi_patches(pl);
   // the common padded rank: repack the staged factors at stride R
   ssm_status st = SSM_OK;
   auto repack = [&]() -> ssm_status {
     const int R = pl->R;
-    SSM_TRY(palloc(pl, &pl->V32, (size_t)ndict * Q * R, s));
+    // (rows of zeros past Q: whole stages, and the rows the kernel reads ahead)
+    const size_t rows = (size_t)(Q + 15) / 16 * 16 + 8;
+    SSM_TRY(palloc(pl, &pl->V32, (size_t)ndict * rows * R, s));
+    SSM_CUDA(cudaMemsetAsync(pl->V32, 0, sizeof(float) * ndict * rows * R, s));
     SSM_TRY(palloc(pl, &pl->coefA, (size_t)ndict * R, s));
     SSM_TRY(palloc(pl, &pl->coefW, (size_t)ndict * R, s));
     SSM_TRY(palloc(pl, &pl->B_multi, (size_t)ndict * P * R, s));
@@ -587,47 +591,54 @@ ssm_status multi_plan_impl(ssm_plan_s* pl, int ndict, const double* K_host,
                            cudaMemcpyHostToDevice, s));
   SSM_TRY(palloc(pl, &pl->dev_err, 1, s));
   SSM_CUDA(cudaMemsetAsync(pl->dev_err, 0, sizeof(int), s));
-  const size_t QN = (size_t)Q * pl->g.ld;
+  const size_t zn = (size_t)state_floats(pl);
   for (int i = 0; i < 2; ++i) {
-    SSM_TRY(palloc(pl, &pl->Z[i], QN, s));
-    SSM_TRY(palloc(pl, &pl->Dl[i], QN, s));
+    SSM_TRY(palloc(pl, &pl->Z[i], zn, s));
+    SSM_TRY(palloc(pl, &pl->Dl[i], zn, s));
   }
   SSM_TRY(palloc(pl, &pl->S, (size_t)pl->R * pl->g.ld, s));
-  const int64_t ntiles = (pl->g.N + kTableTile - 1) / kTableTile;
-  pl->mseg = table_segments(ntiles, Q, pl->R);
-  const size_t pf = (size_t)table_state_floats(pl->g.N, pl->mseg, pl->R);
-  for (int i = 0; i < 2; ++i) SSM_TRY(palloc(pl, &pl->U[i], pf, s));
-  // the iteration's problem descriptor and (tile, segment) table
-  std::vector<int4> entries;
-  table_entries(0, ntiles, pl->mseg, &entries);
-  pl->tblocks = (int64_t)entries.size();
-  pl->lr_grid = pl->tblocks;
-  TableProblem tp{};
-  for (int i = 0; i < 2; ++i) {
-    tp.Z[i] = pl->Z[i];
-    tp.D[i] = pl->Dl[i];
-    tp.U[i] = pl->U[i];
+  if (pl->multi_patches) {
+    SSM_TRY(lowrank_prepare(pl));
+    const size_t pf = (size_t)lowrank_state_floats(pl, pl->lr_grid);
+    for (int i = 0; i < 2; ++i) SSM_TRY(palloc(pl, &pl->U[i], pf, s));
+  } else {
+    const int64_t ntiles = (pl->g.N + kTableTile - 1) / kTableTile;
+    pl->mseg = table_segments(ntiles, Q, pl->R);
+    const size_t pf = (size_t)lowrank_state_floats(pl, pl->lr_grid);
+    for (int i = 0; i < 2; ++i) SSM_TRY(palloc(pl, &pl->U[i], pf, s));
+    // the iteration's problem descriptor and (tile, segment) table
+    std::vector<int4> entries;
+    table_entries(0, ntiles, pl->mseg, &entries);
+    pl->tblocks = (int64_t)entries.size();
+    pl->lr_grid = pl->tblocks;
+    TableProblem tp{};
+    for (int i = 0; i < 2; ++i) {
+      tp.Z[i] = pl->Z[i];
+      tp.D[i] = pl->Dl[i];
+      tp.U[i] = pl->U[i];
+    }
+    tp.S = pl->S;
+    tp.V = pl->V32;
+    tp.coefA = pl->coefA;
+    tp.coefW = pl->coefW;
+    tp.labels = pl->labels;
+    tp.g = pl->g;
+    tp.Q = Q;
+    tp.nseg = pl->mseg;
+    tp.ndict = ndict;
+    tp.beta = (float)p.beta;
+    tp.inv_beta = (float)(1.0 / p.beta);
+    tp.xi = (float)pl->xi;
+    tp.lam_s = (float)pl->lam_s;
+    tp.inv_xb = (float)(1.0 / (pl->xi + p.beta));
+    SSM_TRY(palloc(pl, &pl->tprob, 1, s));
+    SSM_TRY(palloc(pl, &pl->ttable, entries.size(), s));
+    SSM_CUDA(cudaMemcpyAsync(pl->tprob, &tp, sizeof(tp), cudaMemcpyHostToDevice, s));
+    SSM_CUDA(cudaMemcpyAsync(pl->ttable, entries.data(), sizeof(int4) * entries.size(),
+                             cudaMemcpyHostToDevice, s));
+    SSM_CUDA(cudaStreamSynchronize(s));   // the table's host copies are temporaries
   }
-  tp.S = pl->S;
-  tp.V = pl->V32;
-  tp.coefA = pl->coefA;
-  tp.coefW = pl->coefW;
-  tp.labels = pl->labels;
-  tp.g = pl->g;
-  tp.Q = Q;
-  tp.nseg = pl->mseg;
-  tp.ndict = ndict;
-  tp.beta = (float)p.beta;
-  tp.inv_beta = (float)(1.0 / p.beta);
-  tp.xi = (float)pl->xi;
-  tp.lam_s = (float)pl->lam_s;
-  tp.inv_xb = (float)(1.0 / (pl->xi + p.beta));
-  SSM_TRY(palloc(pl, &pl->tprob, 1, s));
-  SSM_TRY(palloc(pl, &pl->ttable, entries.size(), s));
-  SSM_CUDA(cudaMemcpyAsync(pl->tprob, &tp, sizeof(tp), cudaMemcpyHostToDevice, s));
-  SSM_CUDA(cudaMemcpyAsync(pl->ttable, entries.data(), sizeof(int4) * entries.size(),
-                           cudaMemcpyHostToDevice, s));
-  SSM_CUDA(cudaStreamSynchronize(s));   // the host copies are temporaries
+  SSM_CUDA(cudaStreamSynchronize(s));     // so are the caller's labels
   const int maxparts = (int)std::max<int64_t>(pl->lr_grid, (pl->g.N + 255) / 256);
   pl->red_cap = maxparts;
   SSM_TRY(palloc(pl, &pl->red, (size_t)maxparts * 4, s));
@@ -823,7 +834,7 @@ ssm_status one_iteration(ssm_plan_s* pl, int cur, bool check, bool check_next, i
     return prof_mark(pl, false, s);
   }
   SSM_TRY(prof_mark(pl, true, s));
-  if (pl->ndict > 0) {
+  if (pl->ndict > 0 && !pl->multi_patches) {
     SSM_TRY(table_iteration(pl->tprob, pl->ttable, pl->tblocks, pl->R, cur, check, check_next,
                             pl->red, pl->chained, s));
     *nparts = (int)pl->tblocks;

@@ -276,9 +276,11 @@ struct ssm_plan_s {
   int ndict = 0;
   int32_t* labels = nullptr;         // N dictionary labels
   double* B_multi = nullptr;         // ndict x P x R: sigma_{c,i} u_{c,i} (S = B^T m per voxel)
-  int mseg = 1;                      // compartment segments per voxel tile
   std::vector<int> ranks;            // r_c per dictionary
-  ssm::TableProblem* tprob = nullptr;  // the iteration's problem descriptor (device)
+  bool multi_patches = false;        // iterated by lowrank_iter_kernel (blocked state); else
+                                     // by table_iter_kernel, with
+  int mseg = 1;                      // its compartment segments per voxel tile
+  ssm::TableProblem* tprob = nullptr;  // its problem descriptor (device)
   int4* ttable = nullptr;            // its (problem, tile, segment) table (device)
   int64_t tblocks = 0;               // entries of the table
   // the iteration about to be launched directly follows another of the same block in its
@@ -336,6 +338,8 @@ ssm_status blocked_output(const ssm_plan_s* pl, int cur, float* F, int64_t ldf, 
 
 // low-rank iteration (ssm_lowrank.cu)
 ssm_status lowrank_prepare(ssm_plan_s* pl);
+// whether a plan with a dictionary per voxel label runs lowrank_iter_kernel
+bool lowrank_multi_patches(const ssm_plan_s* pl);
 void lowrank_release(ssm_plan_s* pl);
 // low-rank iteration k -> k+1 with state (z, per-voxel u); `check` forms the residual
 // sums (and reads d^k), `write_d` stores d^{k+1} for the next iteration's test

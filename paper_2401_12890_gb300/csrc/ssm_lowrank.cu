@@ -11,10 +11,13 @@ namespace {
 constexpr int TV = 128, QS = 16;
 
 // a unit's start (the a-vector from the segment slots, the partial u' at its end) costs
-// about as much as this many compartment rows
+// about as much as this many compartment rows (8, 24 and 64 give the same times within 1 % on
+// 32x32 .. 192x192)
 constexpr int kUnitRows = 24;
 
-LowrankKernel kernel_for(int R, int naxes) {
+LowrankKernel kernel_for(const ssm_plan_s* pl, int naxes) {
+  const int R = pl->R;
+  if (pl->ndict > 0) return lowrank_kernel_multi(R, naxes);
   if (R <= 16) return lowrank_kernel_small(R, naxes);
   if (R <= 32) return lowrank_kernel_mid(R, naxes);
   return lowrank_kernel_large(R, naxes);
@@ -24,7 +27,7 @@ LowrankKernel kernel_for(int R, int naxes) {
 // per tile, the units (segment, tile) dealt round-robin. nseg minimises rounds x (rows
 // per unit + a unit's start), rounds = ceil(ntiles nseg / G).
 void layout(const ssm_plan_s* pl, const Patch& p, int64_t* grid, int* nseg) {
-  const LowrankKernel k = kernel_for(pl->R, p.naxes);
+  const LowrankKernel k = kernel_for(pl, p.naxes);
   int64_t g0 = (int64_t)sm_count() * (k.blocks_per_sm ? k.blocks_per_sm(p) : 1) *
                std::max(1, pl->waves);
   if (const char* env = getenv("SSM_LOWRANK_GRID")) {   // launch-shape override for sweeps
@@ -55,6 +58,15 @@ struct LowrankState {
 };
 
 }  // namespace
+
+// A dictionary per voxel label: patch tiles up to rank 16 from 1600 voxels on, else the work
+// table. Per iteration, table kernel -> this one: 156x156, Q = 900, 61 dictionaries,
+// r = 4 88.1 -> 53.9 us, r = 8 105.8 -> 68.8 (random labels 134.7 -> 117.7), r = 16
+// 159.4 -> 144.5, but r = 24 198.8 -> 212.2 and r = 32 355.8 -> 408.3 (the basis rows of
+// the resident CTAs no longer fit L1, and fewer threads wait for them); 40x40, Q = 300, r = 8
+// 8.1 -> 8.0, but 1000 voxels 6.6 -> 6.8 and 16x16 6.2 -> 6.4 (two to eight tiles of 128
+// voxels, in at most 10 segments each, leave most SMs idle; the table's tiles are 32).
+bool lowrank_multi_patches(const ssm_plan_s* pl) { return pl->R <= 16 && pl->g.N >= 1600; }
 
 int64_t lowrank_grid(const ssm_plan_s* pl) {
   int64_t grid;
@@ -94,6 +106,7 @@ ssm_status lowrank_prepare(ssm_plan_s* pl) {
     SSM_CUDA(encode_nd(&m.zo, F32, 5, pl->Z[cur ^ 1], dims, strides, patch, SW));
     SSM_CUDA(encode_nd(&m.di, F32, 5, pl->Dl[cur], dims, strides, patch, SW));
     SSM_CUDA(encode_nd(&m.dd, F32, 5, pl->Dl[cur ^ 1], dims, strides, patch, SW));
+    if (pl->ndict > 0) continue;     // their rows are not staged
     SSM_CUDA(encode_2d(&m.v, F32, 4, pl->V32, (uint64_t)pl->R, (uint64_t)pl->Q, (uint64_t)pl->R,
                        (unsigned)pl->R, QS));
   }
@@ -108,7 +121,7 @@ void lowrank_release(ssm_plan_s* pl) {
 ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                              int* nparts, cudaStream_t s) {
   const LowrankState& st = *static_cast<const LowrankState*>(pl->lr_state);
-  const LowrankKernel k = kernel_for(pl->R, st.p.naxes);
+  const LowrankKernel k = kernel_for(pl, st.p.naxes);
   if (!k.launch) {
     set_error("low-rank kernel: unsupported padded rank");
     return SSM_EUNSUPPORTED;
@@ -124,6 +137,9 @@ ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, 
   a.nb = a.nob = 0;                  // set per variant (the launch)
   a.coefA = pl->coefA;
   a.coefW = pl->coefW;
+  a.V = pl->V32;
+  a.labels = pl->labels;
+  a.ndict = pl->ndict;
   a.partial = partial;
   a.mask = pl->mask;
   a.err = pl->dev_err;
@@ -136,7 +152,9 @@ ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, 
   a.lam_s = (float)pl->lam_s;
   a.inv_xb = (float)(1.0 / (pl->xi + pl->p.beta));
   *nparts = (int)grid;
-  // (few units per CTA, as for the tensor-core form)
+  // Chained where the launch gap weighs: 32x32 12.3 -> 9.2 us per iteration, 192x192 at
+  // Q = 900 65.7 -> 62.4, 128x128 at Q = 2500 129.7 -> 126.1; with more units per CTA it gives
+  // nothing (256x256 510.7 -> 508.1, 96x96x64 3893 -> 3893)
   const bool chained = pl->chained && st.p.ntiles * st.nseg <= 8 * grid;
   return k.launch(st.maps[cur], a, check, grid, chained, s);
 }

@@ -49,6 +49,12 @@
 //   96x96x64, Q = 1600, r = 30            4543 -> 3871 us
 //   84x72, Q = 300, r = 13               12.3 -> 8.2 us
 //   32x32, Q = 225, r = 20               12.4 -> 9.5 us
+// A dictionary per voxel label (MULTI; ssm_plan_multi): a thread reads its voxel's own rows of
+// V through L1, some pairs ahead of their use, instead of staged ones (V [q][dictionary][R]:
+// the labels of a patch are mostly neighbours, and so are their rows). Two 128-bit loads per
+// element at r = 8 whose lanes differ take 4 passes of L1 each, which is what bounds it.
+// 156x156, Q = 900, r = 8, 61 dictionaries: 105.8 us per iteration with the table kernel
+// (ssm_table.cu), now 68.8.
 // HBM traffic per state element and iteration: read z, write z' (8 B); d is read/written
 // only around residual tests. Every mbarrier wait is bounded and reports SSM_ETIMEOUT
 // through the plan's device error word.
@@ -76,8 +82,11 @@ struct LowrankArgs {
                                     // zeros, nothing read) in an iteration from z = 0
   int nseg;                         // segments per tile
   int nb, nob;                      // ring stages; z' (and d') buffers, 1 or 2
-  const float* __restrict__ coefA;  // R
-  const float* __restrict__ coefW;  // R
+  const float* __restrict__ coefA;  // R (one row per dictionary)
+  const float* __restrict__ coefW;  // R (one row per dictionary)
+  const float* __restrict__ V;      // spatially varying dictionaries: V [q][dictionary][R],
+  const int32_t* __restrict__ labels;   // each voxel's dictionary, and their number
+  int ndict;
   double* __restrict__ partial;     // 4 doubles per block (check iterations)
   const uint8_t* __restrict__ mask; // voxels inside the object (nullptr: every voxel)
   int* __restrict__ err;            // device error word (SSM_ETIMEOUT on a failed wait)
@@ -96,6 +105,8 @@ struct LowrankKernel {
 LowrankKernel lowrank_kernel_small(int R, int naxes);   // R <= 16
 LowrankKernel lowrank_kernel_mid(int R, int naxes);     // 20 .. 32
 LowrankKernel lowrank_kernel_large(int R, int naxes);   // 40 .. 64
+// a dictionary per voxel label, R <= 16
+LowrankKernel lowrank_kernel_multi(int R, int naxes);
 
 #ifdef SSM_LOWRANK_KERNEL   // the translation units that instantiate the kernel
 namespace {
@@ -108,7 +119,14 @@ constexpr int kMaxNB = 6;          // ring stages at most
 constexpr int OUT_BYTES = TV * 64; // one stage of a tile's z' (or d')
 
 // registers are capped for this many resident CTAs per SM
-template <int R> constexpr int min_blocks() { return R <= 24 ? 3 : (R <= 40 ? 2 : 1); }
+template <int R, bool MULTI> constexpr int min_blocks() {
+  return R <= (MULTI ? 12 : 24) ? 3 : (R <= 40 ? 2 : 1);
+}
+// MULTI: pairs of basis rows a thread has in flight ahead of the one it works on (156x156,
+// Q = 900, 61 dictionaries: R = 4 with 2 pairs 67.0 us, 4 pairs 53.9; R = 8 68.8, 71.9;
+// R = 16 with 1 pair 176, 2 pairs 144.5; a fourth CTA per SM instead: R = 8 86.8)
+template <int R> constexpr int rows_ahead() { return R <= 4 ? 4 : 2; }
+constexpr int kMultiNB = 3;        // MULTI: ring stages (the rest of shared memory is L1)
 
 // bytes of one stage: the staged rows and a row of zeros (swizzle atoms of 512 B), V rows, d
 __host__ __device__ __forceinline__ int rows_bytes(const Patch& p) {
@@ -133,15 +151,15 @@ __device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, floa
 
 // NAX: neighbour pairs read per element (2 on 1D and 2D grids: an axis that is not there
 // reads the row of zeros; 3 on 3D grids)
-template <int R, int NAX, bool CHECK>
-__global__ void __launch_bounds__(NT, min_blocks<R>())
+template <int R, int NAX, bool CHECK, bool MULTI>
+__global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
     lowrank_iter_kernel(const __grid_constant__ LowrankMaps maps, const LowrankArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   pdl_launch_next();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nb = a.nb, nob = a.nob;
-  const int rb = rows_bytes(a.p), stb = stage_bytes(a.p, R, CHECK);
+  const int rb = rows_bytes(a.p), stb = stage_bytes(a.p, MULTI ? 0 : R, CHECK);
   const int OB = OUT_BYTES * (a.write_d ? 2 : 1);
   unsigned char* obuf = smem + nb * stb;
   uint64_t* full = reinterpret_cast<uint64_t*>(obuf + nob * OB);
@@ -181,8 +199,8 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
     // ------------------------------- producer warp: one elected lane issues TMA
     if (lane == 0) {
       tma_prefetch_map(&maps.zi);
-      tma_prefetch_map(&maps.v);
-      const unsigned bytes = (unsigned)(a.p.rows * 64 + QS * R * 4 +
+      if (!MULTI) tma_prefetch_map(&maps.v);
+      const unsigned bytes = (unsigned)(a.p.rows * 64 + (MULTI ? 0 : QS * R * 4) +
                                         (CHECK ? a.p.bx * a.p.by * a.p.bz * 64 : 0));
       pdl_wait();
       int c = 0;   // running stage counter over all units
@@ -203,7 +221,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
             tma_load_5d(vs, &maps.di, q0, x0, y0, z0, ch, &full[b]);
             vs += OUT_BYTES;
           }
-          tma_load_2d(vs, &maps.v, 0, t * QS, &full[b]);
+          if (!MULTI) tma_load_2d(vs, &maps.v, 0, t * QS, &full[b]);
         }
       // no copy may be in flight when the CTA exits
       for (int b = 0; b < nb && b < c; ++b) mbar_wait_sleep(&full[b], ((c - 1 - b) / nb) & 1);
@@ -262,6 +280,8 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
       for (int i = 0; i < 1 + 2 * NAX; ++i) rr[i] = in ? ro[i] : zrow;
       // a_i = S_i/(beta + sigma_i^2) - W_i u_i, u_i summed over the tile's segment
       // slots of the previous iteration in segment order (R loads of a slot in flight)
+      const int lab = MULTI && valid ? __ldg(a.labels + n) : 0;
+      const float *cA = a.coefA + lab * R, *cW = a.coefW + lab * R;
       float2 av[R / 2];
       {
         float us[R];
@@ -279,10 +299,9 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
         for (int i = 0; i < R / 2; ++i) {
           float a0 = 0.f, a1 = 0.f;
           if (in) {
-            a0 = __ldg(a.S + (2 * i) * ld + n) * __ldg(a.coefA + 2 * i) -
-                 __ldg(a.coefW + 2 * i) * us[2 * i];
-            a1 = __ldg(a.S + (2 * i + 1) * ld + n) * __ldg(a.coefA + 2 * i + 1) -
-                 __ldg(a.coefW + 2 * i + 1) * us[2 * i + 1];
+            a0 = __ldg(a.S + (2 * i) * ld + n) * __ldg(cA + 2 * i) - __ldg(cW + 2 * i) * us[2 * i];
+            a1 = __ldg(a.S + (2 * i + 1) * ld + n) * __ldg(cA + 2 * i + 1) -
+                 __ldg(cW + 2 * i + 1) * us[2 * i + 1];
           }
           av[i] = make_float2(a0, a1);
         }
@@ -290,6 +309,22 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
       float2 uacc[R / 2];
 #pragma unroll
       for (int i = 0; i < R / 2; ++i) uacc[i] = make_float2(0.f, 0.f);
+      // MULTI: the voxel's own basis rows, read through L1 a few pairs ahead (rows past Q are
+      // zero; V has room for the last pairs ahead)
+      constexpr int D = MULTI ? rows_ahead<R>() : 1;
+      const float4* vg = reinterpret_cast<const float4*>(a.V) + lab * (R / 4);
+      const int64_t vq1 = MULTI ? (int64_t)a.ndict * (R / 4) : 0;
+      if (MULTI) vg += (int64_t)t0 * QS * vq1;
+      float4 ahead[D][2][R / 4];
+#pragma unroll
+      for (int p = 0; MULTI && p < D; ++p) {
+#pragma unroll
+        for (int i = 0; i < R / 4; ++i) {
+          ahead[p][0][i] = __ldg(vg + i);
+          ahead[p][1][i] = __ldg(vg + vq1 + i);
+        }
+        vg += 2 * vq1;
+      }
 #pragma unroll 1
       for (int t = t0; t < t1; ++t, ++c) {
         const int b = c % nb;
@@ -308,6 +343,13 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
         uint32_t za[1 + 2 * NAX];
 #pragma unroll
         for (int q = 0; q < 1 + 2 * NAX; ++q) za[q] = sb + rr[q];
+        // MULTI: u' of the stage by itself, then added to the running sum (the shorter chains
+        // round less, as the table kernel's quarters of a segment do)
+        float2 ust[R / 2];
+        if (MULTI) {
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) ust[i] = make_float2(0.f, 0.f);
+        }
 #pragma unroll
         for (int j = 0; j < QS / 4; ++j) {
           const uint32_t jx = (uint32_t)j << 4;
@@ -331,13 +373,24 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
             // two compartments: their products with a, then the z-step and dual step packed
             float va[2];
             float4 vr[2][R / 4];
+            if constexpr (MULTI) {
+              const int p = (2 * j + h) % D;
+#pragma unroll
+              for (int i = 0; i < R / 4; ++i) {
+                vr[0][i] = ahead[p][0][i];
+                vr[1][i] = ahead[p][1][i];
+                ahead[p][0][i] = __ldg(vg + i);
+                ahead[p][1][i] = __ldg(vg + vq1 + i);
+              }
+              vg += 2 * vq1;
+            }
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               float2 p0 = make_float2(0.f, 0.f), p1 = make_float2(0.f, 0.f);
               const float4* vq = v4 + (4 * j + 2 * h + e) * (R / 4);
 #pragma unroll
               for (int i = 0; i < R / 4; ++i) {
-                vr[e][i] = vq[i];
+                if (!MULTI) vr[e][i] = vq[i];
                 p0 = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), av[2 * i], p0);
                 p1 = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), av[2 * i + 1], p1);
               }
@@ -357,9 +410,9 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
               const float2 ww = make_float2(w, w);
 #pragma unroll
               for (int i = 0; i < R / 4; ++i) {
-                uacc[2 * i] = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), ww, uacc[2 * i]);
-                uacc[2 * i + 1] =
-                    __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), ww, uacc[2 * i + 1]);
+                float2* us = MULTI ? ust : uacc;
+                us[2 * i] = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), ww, us[2 * i]);
+                us[2 * i + 1] = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), ww, us[2 * i + 1]);
               }
             }
             zn[2 * h] = n2.x;
@@ -379,6 +432,10 @@ __global__ void __launch_bounds__(NT, min_blocks<R>())
           }
           sts4(ob ^ jx, zn[0], zn[1], zn[2], zn[3]);
           if (a.write_d) sts4((ob + OUT_BYTES) ^ jx, dn[0], dn[1], dn[2], dn[3]);
+        }
+        if (MULTI) {
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) uacc[i] = __fadd2_rn(uacc[i], ust[i]);
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         // the other buffer: its store (of the previous stage) has read it
@@ -437,13 +494,13 @@ constexpr int smem_budget(int blocks) {
 constexpr int kFixed = 1024 + 128;   // alignment slack, barriers
 
 // ring stages and z' buffers: two buffers where three stages fit beside them
-template <int R>
+template <int R, bool MULTI>
 bool ring(const Patch& p, bool check, bool write_d, int* nb, int* nob, int* bytes) {
-  const int st = stage_bytes(p, R, check), ob = OUT_BYTES * (write_d ? 2 : 1);
-  for (int blocks = min_blocks<R>(); blocks >= 1; --blocks) {
+  const int st = stage_bytes(p, MULTI ? 0 : R, check), ob = OUT_BYTES * (write_d ? 2 : 1);
+  for (int blocks = min_blocks<R, MULTI>(); blocks >= 1; --blocks) {
     const int room = smem_budget(blocks) - kFixed;
     *nob = (room - 2 * ob) / st >= 3 ? 2 : 1;
-    *nb = std::min(kMaxNB, (room - *nob * ob) / st);
+    *nb = std::min(MULTI ? kMultiNB : kMaxNB, (room - *nob * ob) / st);
     if (*nb >= 2) {
       *bytes = kFixed + *nb * st + *nob * ob;
       return true;
@@ -452,44 +509,45 @@ bool ring(const Patch& p, bool check, bool write_d, int* nb, int* nob, int* byte
   return false;
 }
 
-template <int R, int NAX, bool CHECK>
+template <int R, int NAX, bool CHECK, bool MULTI>
 cudaError_t allow_smem() {
-  return cudaFuncSetAttribute(lowrank_iter_kernel<R, NAX, CHECK>,
+  return cudaFuncSetAttribute(lowrank_iter_kernel<R, NAX, CHECK, MULTI>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
 }
 
-template <int R, int NAX>
+template <int R, int NAX, bool MULTI>
 ssm_status launch_r(const LowrankMaps& maps, LowrankArgs args, bool check, int64_t grid,
                     bool chained, cudaStream_t s) {
   int bytes;
-  if (!ring<R>(args.p, check, args.write_d != 0, &args.nb, &args.nob, &bytes)) {
+  if (!ring<R, MULTI>(args.p, check, args.write_d != 0, &args.nb, &args.nob, &bytes)) {
     set_error("low-rank form: two ring stages do not fit");
     return SSM_EUNSUPPORTED;
   }
-  return check ? launch_chained(lowrank_iter_kernel<R, NAX, true>, (unsigned)grid, NT, bytes, s,
+  return check ? launch_chained(lowrank_iter_kernel<R, NAX, true, MULTI>, (unsigned)grid, NT, bytes, s,
                                 chained, maps, args)
-               : launch_chained(lowrank_iter_kernel<R, NAX, false>, (unsigned)grid, NT, bytes, s,
+               : launch_chained(lowrank_iter_kernel<R, NAX, false, MULTI>, (unsigned)grid, NT, bytes, s,
                                 chained, maps, args);
 }
 
 // resident CTAs per SM of a plain iteration (also sets the kernels' shared-memory limits)
-template <int R, int NAX>
+template <int R, int NAX, bool MULTI>
 int blocks_per_sm(const Patch& p) {
   std::lock_guard<std::mutex> lock(attr_mutex());
-  if (allow_smem<R, NAX, true>() != cudaSuccess || allow_smem<R, NAX, false>() != cudaSuccess) {
+  if (allow_smem<R, NAX, true, MULTI>() != cudaSuccess ||
+      allow_smem<R, NAX, false, MULTI>() != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
   int nb, nob, bytes, b = 0;
-  if (!ring<R>(p, false, false, &nb, &nob, &bytes)) return 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lowrank_iter_kernel<R, NAX, false>, NT, bytes);
+  if (!ring<R, MULTI>(p, false, false, &nb, &nob, &bytes)) return 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lowrank_iter_kernel<R, NAX, false, MULTI>, NT, bytes);
   return std::max(1, b);
 }
 
-template <int R>
+template <int R, bool MULTI = false>
 LowrankKernel kernel_of(int naxes) {
-  if (naxes == 3) return LowrankKernel{launch_r<R, 3>, blocks_per_sm<R, 3>};
-  return LowrankKernel{launch_r<R, 2>, blocks_per_sm<R, 2>};
+  if (naxes == 3) return LowrankKernel{launch_r<R, 3, MULTI>, blocks_per_sm<R, 3, MULTI>};
+  return LowrankKernel{launch_r<R, 2, MULTI>, blocks_per_sm<R, 2, MULTI>};
 }
 
 }  // namespace

@@ -7,7 +7,8 @@
 //    voxel's f-step taking its own dictionary's factors (Eq. 27, Eq. 28, each
 //    dictionary's rank by the rule of Sec. III-E). With a label c(n) per voxel Eq. 7
 //    becomes sum_n 1/2 ||m_n - K_{c(n)} f_n||^2 + lambda/2 ||D F||^2; the z-step and the
-//    dual step do not involve K.
+//    dual step do not involve K. (Ranks up to 16 on 1600 voxels or more run
+//    lowrank_iter_kernel instead: lowrank_multi_patches has the figures.)
 //  - groups of independent small problems of differing N, P and Q (ssm_group_*; serving's
 //    small requests, no counterpart in the paper): one dictionary per problem.
 //
