@@ -1002,7 +1002,10 @@ int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 //    tile would leave G0 - ntiles SMs idle, two would give some CTAs two whole-Q-halves
 //    of work; instead CTA j < ntiles takes chunks [0, split) of tile j and the spare
 //    CTAs take the tails, `split` chosen so that both kinds finish together, a unit's start
-//    counting as kStart chunks.
+//    counting as kStart chunks. Where the few spare CTAs would take longer over their tails
+//    than a whole tile takes (many tails each, few chunks), every tile is one unit instead
+//    (13 slices of 36x29, Q = 225, 130 tiles, 46 iterations: 1466 us with tails, 693
+//    without; 177x74, 38 iterations 849, 571).
 //  - Fewer tiles: each tile is split into spc equal segments so that all CTAs have work.
 // chunks a unit's start (a-vector, filling the pipeline) takes as long as. On 128x128, Q = 2500
 // (79 chunks) 6 gives split = 72: 75 us per iteration; split 70 78, 74 75, 76 77
@@ -1036,6 +1039,11 @@ void layout(const ssm_plan_s* pl, int64_t* grid, int* spc, int* split) {
       }
     }
     if (force_split > 0) best = force_split;
+    if (force_split < 0 && cost >= nch + kStart) {
+      *spc = 1;
+      *grid = ntiles;
+      return;
+    }
     *split = (int)best;
     *spc = 2;
     *grid = ntiles + (ntiles + per - 1) / per;
