@@ -75,7 +75,8 @@ struct LowrankMaps {
 
 struct LowrankArgs {
   const float* __restrict__ S;      // R x ld
-  const float* __restrict__ Pin;    // partial u of the previous iteration [tile][seg][R][TV]
+  const float* Pin;                 // partial u of the previous iteration [tile][seg][R][TV]
+                                    // (which may still run: read after pdl_wait)
   float* __restrict__ Pout;         // partial u of this iteration
   int nst;                          // stages per tile: ceil(Q / QS)
   int coff;                         // added to the chunk of the z loads: past the tensor (all

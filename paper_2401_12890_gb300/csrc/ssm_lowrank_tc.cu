@@ -145,7 +145,8 @@ struct LrtcMaps {
 
 struct LrtcArgs {
   const float* __restrict__ S;      // RP x ld
-  const float* __restrict__ Pin;    // partial u of the previous iteration [tile][slot][RP][TV]
+  const float* Pin;                 // partial u of the previous iteration [tile][slot][RP][TV]
+                                    // (which may still run: read after pdl_wait)
   float* __restrict__ Pout;         // partial u of this iteration
   int nch;                          // compartment chunks per tile
   int spc;                          // segments per tile (each a contiguous run of chunks)

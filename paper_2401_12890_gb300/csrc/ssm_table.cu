@@ -98,11 +98,13 @@ __global__ void __launch_bounds__(VT * WPB, min_blocks<R>())
   const bool zl = nz > 1 && g.zlink;
   const int64_t plane = (int64_t)nx * ny;
   const float beta = P.beta, inv_beta = P.inv_beta;
-  const float* __restrict__ Zin = P.Z[cur];
+  // (Zin, Din, Uin: written by the previous iteration, which may still run: read after
+  // pdl_wait, by ordinary loads)
+  const float* Zin = P.Z[cur];
   float* __restrict__ Zo = P.Z[cur ^ 1];
-  const float* __restrict__ Din = P.D[cur];
+  const float* Din = P.D[cur];
   float* __restrict__ Do = write_d ? P.D[cur ^ 1] : nullptr;
-  const float* __restrict__ Uin = P.U[cur];
+  const float* Uin = P.U[cur];
   float* __restrict__ Uo = P.U[cur ^ 1];
   const int64_t n = tile * VT + lane;
   const bool in = n < N;

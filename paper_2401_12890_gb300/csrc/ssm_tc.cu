@@ -98,9 +98,12 @@ struct TcArgs {
   int* __restrict__ err;
   Grid g;
   int Q, ntv, ntq;
-  // fused update epilogue
-  const float* __restrict__ Zin;     // z^k, d^k, h (Q x ld)
-  const float* __restrict__ Din;
+  // fused update epilogue. z^k and d^k (Q x ld) are written by the iteration before, which a
+  // chained launch overlaps until its pdl_wait: they are read by ordinary loads (or TMA)
+  // after it, never through the read-only path (ld.global.nc is for data that no running
+  // kernel writes). h is the solve's
+  const float* Zin;
+  const float* Din;
   const float* __restrict__ H;
   float* __restrict__ Zout;          // z^{k+1}, d^{k+1}
   float* __restrict__ Dout;
@@ -455,7 +458,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
 #pragma unroll
         for (int j = 0; j < UG; ++j) {
           const int64_t o = (int64_t)min(q0n + j, a.Q - 1) * ld + nn;
-          dnext[j] = __ldg(a.Din + o);
+          dnext[j] = a.Din[o];
           hnext[j] = __ldg(a.H + o);
         }
       }
@@ -613,21 +616,21 @@ __global__ void __launch_bounds__(NTHR, 1) tc_gemm_kernel(const __grid_constant_
               // a padding column reads the last compartment's row (in bounds), unused;
               // absent neighbours read the voxel's own value and are dropped
               const int64_t o = (int64_t)min(q0 + j, a.Q - 1) * ld + n;
-              b.z[j] = __ldg(a.Zin + o);
-              b.d[j] = __ldg(a.Din + o);
+              b.z[j] = a.Zin[o];
+              b.d[j] = a.Din[o];
               b.h[j] = __ldg(a.H + o);
   #pragma unroll
-              for (int k = 0; k < NRT; ++k) b.zk[k][j] = __ldg(a.Zin + o + dk[k]);
+              for (int k = 0; k < NRT; ++k) b.zk[k][j] = a.Zin[o + dk[k]];
               if constexpr (!XSHFL) {
-                b.xm[j] = __ldg(a.Zin + o + dxm);
-                b.xp[j] = __ldg(a.Zin + o + dxp);
+                b.xm[j] = a.Zin[o + dxm];
+                b.xp[j] = a.Zin[o + dxp];
               }
             }
             if constexpr (XSHFL) {
               const int je = lane % UG, side = lane / UG;
               const int64_t ne = side == 0 ? (n0w > 0 ? n0w - 1 : n0w)
                                            : side == 1 ? min(n0w + 32, ld - 1) : n0w;
-              b.edge = __ldg(a.Zin + (int64_t)min(q0 + je, a.Q - 1) * ld + ne);
+              b.edge = a.Zin[(int64_t)min(q0 + je, a.Q - 1) * ld + ne];
             }
           };
           auto process = [&](int cg, Buf& b) {
