@@ -42,28 +42,30 @@ __global__ void __launch_bounds__(256) unblock_kernel(const float* __restrict__ 
   }
 }
 
-constexpr int kMaxRows = 400;        // staged rows of a 3D patch at most (ring stages)
-
 }  // namespace
 
-// The patch of a grid's tiles: among all bx x by x bz <= 128 whose rows with halo fit the
-// staging area, the one with the least tiles x (a tile's fixed work + its staged rows). The
+// axes with smoothness (at least 1: see patch_of)
+int grid_axes(const Grid& g) {
+  return std::max(1, (g.nx > 1) + (g.ny > 1) + (g.nz > 1 && g.zlink));
+}
+
+// The patch of a grid's tiles: among all bx x by x bz <= 128 with at most max_rows staged
+// rows (halo included; what the kernel's ring has room for), the one with the least tiles x (a tile's fixed work + its staged rows). The
 // weight of the fixed work (300 rows) and the penalty for rows that do not start on
 // multiples of 8 (a quarter warp's 128-bit loads then meet in the same banks) only break
 // near-ties: 16 x 8 (2D) and 8 x 4 x 4 (3D) where the grid divides. An axis without
 // smoothness (one voxel, or the stacking axis of a batch) needs no halo; a single voxel
 // takes one on x (zero-filled rows), so that there is always a neighbour pair to read.
-Patch patch_of(const Grid& g) {
+Patch patch_of(const Grid& g, int max_rows) {
   Patch best{};
   double cost = 1e300;
   const int hy = g.ny > 1, hz = g.nz > 1 && g.zlink;
   const int hx = g.nx > 1 || (!hy && !hz);
-  const int rmax = hx + hy + hz == 3 ? kMaxRows : 260;
   for (int bz = 1; bz <= std::min(g.nz, TV); ++bz)
     for (int by = 1; by <= std::min(g.ny, TV / bz); ++by)
       for (int bx = 1; bx <= std::min(g.nx, TV / (bz * by)); ++bx) {
         const int X = bx + 2 * hx, Y = by + 2 * hy, Z = bz + 2 * hz, rows = X * Y * Z;
-        if (rows > rmax) continue;
+        if (rows > max_rows) continue;
         const int64_t tx = (g.nx + bx - 1) / bx, ty = (g.ny + by - 1) / by, tz = (g.nz + bz - 1) / bz;
         const double c = (double)tx * ty * tz * (300 + rows + (bx % 8 ? 60 : 0));
         if (c < cost) {

@@ -116,7 +116,8 @@ struct Patch {
   int zst;                   // bytes of the z rows, rounded up to 1024
 };
 
-Patch patch_of(const Grid& g);
+int grid_axes(const Grid& g);
+Patch patch_of(const Grid& g, int max_rows);
 
 // One element of the full-rank iteration's z-step (Eq. 31, with D^T D z = s (deg z -
 // sum_nbr z)) and dual step (step 11), given f = h + M w:

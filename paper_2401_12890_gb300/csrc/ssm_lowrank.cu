@@ -10,6 +10,12 @@ namespace {
 
 constexpr int TV = 128, QS = 16;
 
+// the plan's tiles: at most 400 staged rows on 3D grids, else 260 (the ring of every rank has
+// room for two such stages: ring())
+Patch tiles_of(const ssm_plan_s* pl) {
+  return patch_of(pl->g, grid_axes(pl->g) == 3 ? 400 : 260);
+}
+
 // a unit's start (the a-vector from the segment slots, the partial u' at its end) costs
 // about as much as this many compartment rows (8, 24 and 64 give the same times within 1 % on
 // 32x32 .. 192x192)
@@ -71,7 +77,7 @@ bool lowrank_multi_patches(const ssm_plan_s* pl) { return pl->R <= 16 && pl->g.N
 int64_t lowrank_grid(const ssm_plan_s* pl) {
   int64_t grid;
   int nseg;
-  layout(pl, patch_of(pl->g), &grid, &nseg);
+  layout(pl, tiles_of(pl), &grid, &nseg);
   return grid;
 }
 
@@ -79,7 +85,7 @@ int64_t lowrank_partial_floats(const ssm_plan_s* pl, int64_t grid) {
   (void)grid;
   int64_t g;
   int nseg;
-  const Patch p = patch_of(pl->g);
+  const Patch p = tiles_of(pl);
   layout(pl, p, &g, &nseg);
   return p.ntiles * nseg * (int64_t)pl->R * TV;
 }
@@ -90,7 +96,7 @@ int lowrank_max_partials(const ssm_plan_s* pl) { return (int)lowrank_grid(pl); }
 ssm_status lowrank_prepare(ssm_plan_s* pl) {
   auto* st = new LowrankState();
   pl->lr_state = st;
-  st->p = patch_of(pl->g);
+  st->p = tiles_of(pl);
   layout(pl, st->p, &pl->lr_grid, &st->nseg);
   const Patch& p = st->p;
   const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;

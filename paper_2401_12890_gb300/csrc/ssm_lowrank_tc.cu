@@ -961,22 +961,51 @@ ssm_status prepare_rn() {
   return SSM_OK;
 }
 
+// shared memory of one variant for patches of `z_bytes` bytes of staged rows: ring stages, z'
+// (and d') buffers per group, dynamic bytes
+struct Ring {
+  int nsz, nob;
+  size_t shm;
+};
+template <int RP, int NAX, bool CHECK, bool WD>
+constexpr Ring ring_of(int z_bytes) {
+  const int zst = z_bytes + (CHECK ? OUT_BYTES : 0);
+  const int ob = OUT_BYTES * (WD && !CHECK ? 2 : 1);
+  const int vbytes = 2 * Lay<RP, NAX>::NSV * Lay<RP, NAX>::VST;
+  const int room = kSmemLimit - kReserve - vbytes;
+  // two z' buffers per group spare a barrier per chunk, where three z stages still fit
+  const int nob = (room - NG * 2 * ob) / zst >= 3 ? 2 : 1;
+  const int fit = (room - NG * nob * ob) / zst, nsz = fit < kMaxNSZ ? fit : kMaxNSZ;
+  return Ring{nsz, nob, (size_t)(kReserve - 1024) + vbytes + (size_t)(NG * nob * ob) +
+                            (size_t)nsz * zst};
+}
+
+// staged rows at most: every variant has two ring stages, and 400 (3D grids) or 260 rows pack
+// 128 voxels well enough. At RP = 64 the V rings leave room for 248 (2D: 260 otherwise, taken
+// by patches two voxels wide and by stacks of very small slices)
+template <int RP, int NAX>
+constexpr int max_rows() {
+  int rows = NAX == 3 ? 400 : 260;
+  for (; rows > 0; --rows) {
+    const int z = (rows * 128 + 1023) / 1024 * 1024;
+    if (ring_of<RP, NAX, false, false>(z).nsz >= 2 && ring_of<RP, NAX, false, true>(z).nsz >= 2 &&
+        ring_of<RP, NAX, true, false>(z).nsz >= 2 && ring_of<RP, NAX, true, true>(z).nsz >= 2)
+      break;
+  }
+  return rows;
+}
+// (a patch of one voxel has 3, 9 or 27 rows)
+static_assert(max_rows<32, 1>() == 260 && max_rows<32, 2>() == 260 && max_rows<32, 3>() == 400 &&
+                  max_rows<64, 1>() == 248 && max_rows<64, 2>() == 248,
+              "rows of a patch");
+
 template <int RP, int NAX, bool CHECK, bool WD>
 ssm_status launch_one(const LrtcMaps& maps, LrtcArgs args, int64_t grid, bool chained,
                       cudaStream_t s) {
-  const int zst = args.p.zst + (CHECK ? OUT_BYTES : 0);
-  const int ob = OUT_BYTES * (WD && !CHECK ? 2 : 1);
-  constexpr int vbytes = 2 * Lay<RP, NAX>::NSV * Lay<RP, NAX>::VST;
-  const int room = kSmemLimit - kReserve - vbytes;
-  // two z' buffers per group spare a barrier per chunk, where three z stages still fit
-  args.nob = (room - NG * 2 * ob) / zst >= 3 ? 2 : 1;
-  args.nsz = std::min(kMaxNSZ, (room - NG * args.nob * ob) / zst);
-  if (args.nsz < 2) {
-    set_error("tensor-core low-rank form: two ring stages do not fit");
-    return SSM_EUNSUPPORTED;
-  }
-  const size_t shm = (size_t)(kReserve - 1024) + vbytes + NG * args.nob * ob +
-                     (size_t)args.nsz * zst;
+  const Ring ring = ring_of<RP, NAX, CHECK, WD>(args.p.zst);
+  args.nob = ring.nob;
+  args.nsz = ring.nsz;
+  const size_t shm = ring.shm;
   return launch_chained(lrtc_kernel<RP, NAX, CHECK, WD>, (unsigned)grid, NT, shm, s, chained, maps,
                         args);
 }
@@ -990,9 +1019,14 @@ ssm_status launch_rn(const LrtcMaps& maps, const LrtcArgs& args, bool check, boo
   return launch_one<RP, NAX, false, false>(maps, args, grid, chained, s);
 }
 
+Patch tiles_of(const ssm_plan_s* pl) {
+  const int axes = grid_axes(pl->g);
+  if (pl->R == 64) return patch_of(pl->g, max_rows<64, 2>());
+  return patch_of(pl->g, axes == 3 ? max_rows<32, 3>() : max_rows<32, 2>());
+}
 int64_t ntiles_of(const ssm_plan_s* pl) {
   if (pl->lr_state) return static_cast<const LrtcState*>(pl->lr_state)->p.ntiles;
-  return patch_of(pl->g).ntiles;
+  return tiles_of(pl).ntiles;
 }
 int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 
@@ -1091,7 +1125,7 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
   }
   auto* st = new LrtcState();
   pl->lr_state = st;
-  st->p = patch_of(pl->g);
+  st->p = tiles_of(pl);
   layout(pl, &pl->lr_grid, &st->spc, &st->split);
   const Patch& p = st->p;
   const uint64_t Q = (uint64_t)pl->Q, RP = (uint64_t)pl->R, Qs = (uint64_t)pl->lrtc_qs;
