@@ -963,7 +963,25 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
     set_error("nothing to resume: the plan has no iteration state (solve first)");
     return SSM_EINVAL;
   }
+  const bool use_tol = p.tol_primal > 0 || p.tol_change > 0;
+  // iteration j forms the residual sums when it ends on a test boundary or is the last;
+  // "iteration max_iter" counts as a test, so the last iteration also stores d (the
+  // low-rank forms keep d only around tests), which a resumed solve's first test reads
+  auto is_check = [&](int j) {
+    if (j >= p.max_iter) return j == p.max_iter;
+    const bool at = p.check_every > 0 && ((j + 1) % p.check_every == 0);
+    return (use_tol && at) || j + 1 == p.max_iter;
+  };
   pl->has_state = false;   // set again when this solve completes
+  if (resume && p.form == SSM_FORM_LOWRANK && !pl->has_d && is_check(0)) {
+    // The last solve stopped on its tolerance, so its last iteration k-1 -> k stored no d, and
+    // the first test here reads d^k: that iteration once more, from the z and u it started
+    // from (the other ping-pong halves) and its S, stores it (and the same z^k and u)
+    int np = 0;
+    pl->chained = pl->from_zero = false;
+    SSM_TRY(one_iteration(pl, pl->cur_state ^ 1, false, true, &np, s));
+    pl->has_d = true;
+  }
   // step 4: projections of the data on the singular vectors (accurate to an FP64 accumulation)
   if (pl->ndict > 0) {
     // each voxel's projections on its own dictionary's factors (zero past its rank)
@@ -1020,19 +1038,10 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
     }
   }
 
-  const bool use_tol = p.tol_primal > 0 || p.tol_change > 0;
   int cur = resume ? pl->cur_state : 0, k = 0;
   double rp = -1, rc = -1;
   ssm_status result = SSM_OK;
   bool converged = false;
-  // iteration j forms the residual sums when it ends on a test boundary or is the last;
-  // "iteration max_iter" counts as a test, so the last iteration also stores d (the
-  // low-rank forms keep d only around tests), which a resumed solve's first test reads
-  auto is_check = [&](int j) {
-    if (j >= p.max_iter) return j == p.max_iter;
-    const bool at = p.check_every > 0 && ((j + 1) % p.check_every == 0);
-    return (use_tol && at) || j + 1 == p.max_iter;
-  };
   const bool graphs = pl->use_graphs && !pl->prof_enabled && capturable(s);
   // blocks of iterations end at each residual test (the host reads the sums there) or
   // after kBlockMax iterations; a block runs as direct launches or as one graph replay
@@ -1064,6 +1073,7 @@ ssm_status solve_impl(ssm_plan_s* pl, const float* M, int64_t ldm, float* F, int
   }
   if (use_tol && !converged) result = SSM_ENOTCONVERGED;
   pl->cur_state = cur;
+  pl->has_d = k == 0 || is_check(k);
   pl->has_state = true;
   // F = z (the feasible iterate; y for Algorithm 1)
   const float* Fsrc = p.form == SSM_FORM_ADMM ? pl->adm.y : pl->Z[cur];

@@ -272,6 +272,7 @@ struct ssm_plan_s {
   // the iteration state left by the last completed solve (ssm_solve_resume continues it)
   bool has_state = false;
   int cur_state = 0;           // ping-pong half holding z^k (and w^k, partial u)
+  bool has_d = false;          // ... and d^k (the low-rank forms store it only for tests)
   // spatially varying dictionaries (ssm_plan_multi): ndict > 0. V32, coefA and coefW
   // then hold every dictionary's factors ([q][c][i], [c][i]), padded to the common R
   int ndict = 0;
