@@ -186,10 +186,12 @@ __device__ __forceinline__ void block_partial(double d1, double d2, double d3, d
   }
 }
 
-// sum over a chunk of maps and RT voxels of (F_n - F_m)^2, m the forward neighbours: a
-// float-float sum per thread (its error, 2^-48 relative, is far below that of the FP32
-// squares; an FP64 add per element would take 77 us of the 41 M elements of the 128 x 128
-// slice at this chip's FP64 rate)
+// sum over a chunk of maps and RT voxels of (F_n - F_m)^2, m the forward neighbours: FP32
+// squares (a map's three added in FP32), their sum over the maps in FP64. Eight maps at a time
+// are added as a float-float number (its error, seven roundings of the low part, is at most
+// 2^-43 of the eight's sum) and that to the FP64 sum: at this chip's FP64 rate an FP64 add per
+// element would take 77 us of the 41 M elements of the 128 x 128 slice. Where the FP32 part
+// overflows (or is not a number), the eight go to the FP64 sum one by one.
 constexpr int RT = 256;
 __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__ F, int64_t ldf,
                                                        int Q, int chunk, Grid g,
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
                                                        double* __restrict__ partial) {
   const int64_t n = blockIdx.x * (int64_t)RT + threadIdx.x;
   const int q0 = (int)blockIdx.y * chunk, q1 = min(Q, q0 + chunk);
-  float s = 0.f, c = 0.f;
+  double e2 = 0.0;
   if (n < g.N && (!mk || mk[n])) {
     const int x = (int)(n % g.nx);
     const int64_t t = n / g.nx;
@@ -206,10 +208,15 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
     const bool hx = x + 1 < g.nx && (!mk || mk[n + 1]);
     const bool hy = y + 1 < g.ny && (!mk || mk[n + sy]);
     const bool hz = g.zlink && z + 1 < g.nz && (!mk || mk[n + sz]);
-    // an absent neighbour is the voxel itself
+    // an absent neighbour reads the voxel itself, and its difference is dropped
     const int64_t ox = hx ? 1 : 0, oy = hy ? sy : 0, oz = hz ? sz : 0;
     const float* p = F + (int64_t)q0 * ldf + n;
     const bool z3 = g.zlink && g.nz > 1;
+    auto square = [&](float v, float vx, float vy, float vz) {
+      const float dx = hx ? __fsub_rn(v, vx) : 0.f, dy = hy ? __fsub_rn(v, vy) : 0.f;
+      const float dz = hz ? __fsub_rn(v, vz) : 0.f;
+      return fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
+    };
     // RU maps' loads in flight per thread
     constexpr int RU = 8;
     int q = q0;
@@ -222,22 +229,23 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
         vy[u] = __ldg(p + u * ldf + oy);
         vz[u] = z3 ? __ldg(p + u * ldf + oz) : v[u];
       }
+      float s = 0.f, c = 0.f;
 #pragma unroll
       for (int u = 0; u < RU; ++u) {
-        const float dx = __fsub_rn(v[u], vx[u]), dy = __fsub_rn(v[u], vy[u]);
-        const float dz = __fsub_rn(v[u], vz[u]);
-        two_sum(s, c, fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, 0.f))));
+        v[u] = square(v[u], vx[u], vy[u], vz[u]);
+        two_sum(s, c, v[u]);
+      }
+      if (s <= 3.402823466e38f) {
+        e2 += (double)s + (double)c;
+      } else {
+#pragma unroll
+        for (int u = 0; u < RU; ++u) e2 += (double)v[u];
       }
     }
-    for (; q < q1; ++q, p += ldf) {
-      const float v = __ldg(p);
-      const float dx = __fsub_rn(v, __ldg(p + ox)), dy = __fsub_rn(v, __ldg(p + oy));
-      const float dz = z3 ? __fsub_rn(v, __ldg(p + oz)) : 0.f;
-      two_sum(s, c, fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, 0.f))));
-    }
+    for (; q < q1; ++q, p += ldf)
+      e2 += (double)square(__ldg(p), __ldg(p + ox), __ldg(p + oy), z3 ? __ldg(p + oz) : 0.f);
   }
-  block_partial<RT>(0.0, (double)s + (double)c, 0.0,
-                    partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 4);
+  block_partial<RT>(0.0, e2, 0.0, partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 4);
 }
 
 // A B for the full-rank FP32 forms (C = A B), or the objective's data term, sum (D - A B)^2
