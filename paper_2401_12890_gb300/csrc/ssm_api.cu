@@ -42,7 +42,9 @@ std::mutex& attr_mutex() {
 cudaError_t encode_nd(CUtensorMap* map, CUtensorMapDataType dtype, unsigned rank, const void* base,
                       const uint64_t* dims, const uint64_t* strides, const unsigned* box,
                       CUtensorMapSwizzle swizzle) {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  // (solves of different threads come here at once; every one stores the same pointer)
+  static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> entry{nullptr};
+  PFN_cuTensorMapEncodeTiled_v12000 fn = entry.load(std::memory_order_acquire);
   if (!fn) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -53,6 +55,7 @@ cudaError_t encode_nd(CUtensorMap* map, CUtensorMapDataType dtype, unsigned rank
       return e != cudaSuccess ? e : cudaErrorNotSupported;
     }
     fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    entry.store(fn, std::memory_order_release);
   }
   cuuint64_t d[5], st[4];
   cuuint32_t bx[5], estr[5];
