@@ -248,8 +248,11 @@ ssm_status ssm_group_destroy(ssm_group_t group);
  *   F_dev : Q x N floats on the device, leading dimension ldf >= N; written.
  *   info  : host struct, may be NULL; filled after the solve (synchronises `stream`).
  * z, f and d start at 0 (Algorithm 2, step 2). The projections of M on the singular
- * vectors (g_n of step 4) are formed once, to the accuracy of an FP64 accumulation (for
- * a sum that does not cancel below 2^-14 of its terms). The returned F is
+ * vectors (g_n of step 4) are formed once. Low-rank form: sigma_i u_i^T m_n to the accuracy
+ * of an FP64 accumulation, rounded to FP32. Dense form and Algorithm 1: h = (K^T K +
+ * beta I)^{-1} K^T m to P * 6 * 2^-40 of the product of the power-of-two scales of the
+ * matrix's row and of the voxel's data (each at most twice its largest entry), rounded to
+ * FP32. The returned F is
  * the feasible iterate z (F >= 0 elementwise). With a tolerance set, residuals are
  * tested every check_every iterations (a host read of three FP64 sums); the status
  * is SSM_ENOTCONVERGED when the budget ran out first (F is still written).

@@ -398,11 +398,10 @@ ssm_status plan_impl(ssm_plan_s* pl, const double* K_host, cudaStream_t s) {
     }
   }
   {
-    const int xr = p.form == SSM_FORM_LOWRANK ? pl->r : Q;
-    int xrp, xpp;
-    exact_shape(xr, P, &xrp, &xpp);
-    SSM_TRY(palloc(pl, &pl->Xs, (size_t)exact_elems(xr, P), s));
-    SSM_TRY(palloc(pl, &pl->xexp, (size_t)xrp, s));
+    const bool lowrank = p.form == SSM_FORM_LOWRANK;
+    const ExactShape x = exact_shape(lowrank ? pl->r : Q, P, lowrank);
+    SSM_TRY(palloc(pl, &pl->Xs, (size_t)x.elems(), s));
+    SSM_TRY(palloc(pl, &pl->xexp, (size_t)x.rows, s));
     SSM_TRY(palloc(pl, &pl->vexp, (size_t)pl->g.ld, s));
   }
   st = factors_fp64(pl, E, s);
@@ -710,11 +709,10 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
     if (p.precision == SSM_BF16X3) add(2, 2 * Q * t.Qp);  // Mhi, Mlo
   }
   {
-    const int xr = p.form == SSM_FORM_LOWRANK ? t.r : p.Q;
-    int xrp, xpp;
-    exact_shape(xr, p.P, &xrp, &xpp);
-    add(2, exact_elems(xr, p.P));             // Xs
-    add(4, xrp);                              // xexp
+    const bool lowrank = p.form == SSM_FORM_LOWRANK;
+    const ExactShape x = exact_shape(lowrank ? t.r : p.Q, p.P, lowrank);
+    add(2, x.elems());                        // Xs
+    add(4, x.rows);                           // xexp
     add(4, ld);                               // vexp
   }
   const int64_t QN = Q * ld;

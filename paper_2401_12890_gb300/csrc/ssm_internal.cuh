@@ -322,14 +322,21 @@ ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, cudaS
 ssm_status split_bf16(const float* X, int rows, int cols, int64_t ldx,
                       __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t ldo, cudaStream_t s);
 
-// out = A m to FP64 grade on the tensor cores (ssm_exact.cu): the rows of A are cut into
-// slices once (exact_slice; the operand holds exact_elems BF16 values and the padded row
-// count of exponents)
-void exact_shape(int rows, int P, int* rows_pad, int* P_pad);
-int64_t exact_elems(int rows, int P);
+// out (rows x ldo) = A m on the tensor cores for the data M (P x N, row stride ldm), A given in
+// FP64 as A[i][p] = scale_i src[i sr + p sp] (scale nullptr: 1) and cut into slices once
+// (ssm_exact.cu). `checked`: as accurate as an FP64 accumulation (at most 64 rows, with a
+// scale; src is read again where the slices fall short); else to 6 P 2^-40 of the rows' and
+// columns' scales. vexp: N ints of scratch
+struct ExactShape {
+  int slices, rows, cols;          // the sliced operand is slices x rows x cols BF16 values,
+                                   // with an exponent per row
+  int64_t elems() const { return (int64_t)slices * rows * cols; }
+};
+ExactShape exact_shape(int rows, int P, bool checked);
 ssm_status exact_slice(const double* src, int64_t sr, int64_t sp, const double* scale, int rows,
-                       int P, __nv_bfloat16* slices, int* rexp, cudaStream_t s);
-ssm_status exact_product(const __nv_bfloat16* slices, const int* rexp, int rows, int P,
+                       int P, bool checked, __nv_bfloat16* slices, int* rexp, cudaStream_t s);
+ssm_status exact_product(const double* src, int64_t sr, int64_t sp, const double* scale,
+                         const __nv_bfloat16* slices, const int* rexp, int rows, int P, bool checked,
                          const float* M, int64_t ldm, int64_t N, float* out, int64_t ldo,
                          int* vexp, int* err, cudaStream_t s);
 

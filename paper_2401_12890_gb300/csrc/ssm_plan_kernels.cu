@@ -402,7 +402,7 @@ ssm_status beta_weights(ssm_plan_s* pl, cudaStream_t s) {
         pl->coefW, floor);
     SSM_LAUNCHED();
     if (pl->V1h) SSM_TRY(lrtc_split_basis(pl, s));
-    SSM_TRY(exact_slice(pl->Bp64, 1, n, pl->alpha64, pl->r, pl->P, pl->Xs, pl->xexp, s));
+    SSM_TRY(exact_slice(pl->Bp64, 1, n, pl->alpha64, pl->r, pl->P, true, pl->Xs, pl->xexp, s));
   } else {
     // A = (K^T K + beta I)^{-1} K^T = sum_i k_i b_i^T / (sigma_i^2 + beta), b_i the left
     // factors (rows of Bp^T), in FP64
@@ -412,7 +412,7 @@ ssm_status beta_weights(ssm_plan_s* pl, cudaStream_t s) {
     inv_weights<<<nblk(n, 256), 256, 0, s>>>(pl->sig64, n, 1, pl->p.beta, w);
     SSM_LAUNCHED();
     SSM_TRY(dgemm(Q, pl->P, n, pl->Kt64, n, false, pl->Bp64, n, true, A, pl->P, s, w));
-    SSM_TRY(exact_slice(A, pl->P, 1, nullptr, Q, pl->P, pl->Xs, pl->xexp, s));
+    SSM_TRY(exact_slice(A, pl->P, 1, nullptr, Q, pl->P, false, pl->Xs, pl->xexp, s));
     SSM_CUDA(cudaFreeAsync(A, s));
     SSM_CUDA(cudaFreeAsync(w, s));
   }
@@ -449,9 +449,11 @@ ssm_status split_bf16(const float* X, int rows, int cols, int64_t ldx, __nv_bflo
 // The projections of step 4: S_i = sigma_i u_i^T m (low-rank forms) or h = M g with
 // M g = (K^T K + beta I)^{-1} K^T m (full-rank forms and Algorithm 1)
 ssm_status project_data(const ssm_plan_s* pl, const float* M, int64_t ldm, cudaStream_t s) {
-  const bool lowrank = pl->p.form == SSM_FORM_LOWRANK;
-  return exact_product(pl->Xs, pl->xexp, lowrank ? pl->r : pl->Q, pl->P, M, ldm, pl->g.N,
-                       lowrank ? pl->S : pl->H, pl->g.ld, pl->vexp, pl->dev_err, s);
+  if (pl->p.form == SSM_FORM_LOWRANK)
+    return exact_product(pl->Bp64, 1, pl->n, pl->alpha64, pl->Xs, pl->xexp, pl->r, pl->P, true,
+                         M, ldm, pl->g.N, pl->S, pl->g.ld, pl->vexp, pl->dev_err, s);
+  return exact_product(nullptr, 0, 0, nullptr, pl->Xs, pl->xexp, pl->Q, pl->P, false, M, ldm,
+                       pl->g.N, pl->H, pl->g.ld, pl->vexp, pl->dev_err, s);
 }
 
 }  // namespace ssm
