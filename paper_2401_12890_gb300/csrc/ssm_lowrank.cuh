@@ -121,12 +121,16 @@ constexpr int OUT_BYTES = TV * 64; // one stage of a tile's z' (or d')
 
 // registers are capped for this many resident CTAs per SM
 template <int R, bool MULTI> constexpr int min_blocks() {
-  return R <= (MULTI ? 12 : 24) ? 3 : (R <= 40 ? 2 : 1);
+  return R <= (MULTI ? 12 : 20) ? 3 : (R <= 32 ? 2 : 1);
 }
 // MULTI: pairs of basis rows a thread has in flight ahead of the one it works on (156x156,
 // Q = 900, 61 dictionaries: R = 4 with 2 pairs 67.0 us, 4 pairs 53.9; R = 8 68.8, 71.9;
 // R = 16 with 1 pair 176, 2 pairs 144.5; a fourth CTA per SM instead: R = 8 86.8)
 template <int R> constexpr int rows_ahead() { return R <= 4 ? 4 : 2; }
+// Two compartments are worked on at once where their V rows fit the registers between the
+// product with a and the part of u' (2 R, next to 2 R for a and u'), else one (R = 64 with two
+// spilled 1 KB per thread: 128x100, Q = 400 125 us per iteration, now 62.7)
+template <int R> constexpr bool two_at_once() { return R <= 40; }
 constexpr int kMultiNB = 3;        // MULTI: ring stages (the rest of shared memory is L1)
 
 // bytes of one stage: the staged rows and a row of zeros (swizzle atoms of 512 B), V rows, d
@@ -313,6 +317,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
       // MULTI: the voxel's own basis rows, read through L1 a few pairs ahead (rows past Q are
       // zero; V has room for the last pairs ahead)
       constexpr int D = MULTI ? rows_ahead<R>() : 1;
+      constexpr bool TWO = MULTI || two_at_once<R>();
       const float4* vg = reinterpret_cast<const float4*>(a.V) + lab * (R / 4);
       const int64_t vq1 = MULTI ? (int64_t)a.ndict * (R / 4) : 0;
       if (MULTI) vg += (int64_t)t0 * QS * vq1;
@@ -369,66 +374,102 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
           float zn[4], dn[4];
           float4 dk = make_float4(0.f, 0.f, 0.f, 0.f);
           if (CHECK) dk = lds4(db ^ jx);
+          if constexpr (!TWO) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            // two compartments: their products with a, then the z-step and dual step packed
-            float va[2];
-            float4 vr[2][R / 4];
-            if constexpr (MULTI) {
-              const int p = (2 * j + h) % D;
-#pragma unroll
-              for (int i = 0; i < R / 4; ++i) {
-                vr[0][i] = ahead[p][0][i];
-                vr[1][i] = ahead[p][1][i];
-                ahead[p][0][i] = __ldg(vg + i);
-                ahead[p][1][i] = __ldg(vg + vq1 + i);
-              }
-              vg += 2 * vq1;
-            }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
+            for (int e = 0; e < 4; ++e) {
+              // one compartment: its product with a, the z-step and dual step, its part of u'
+              const float4* vq = v4 + (4 * j + e) * (R / 4);
+              float4 vr[R / 4];
               float2 p0 = make_float2(0.f, 0.f), p1 = make_float2(0.f, 0.f);
-              const float4* vq = v4 + (4 * j + 2 * h + e) * (R / 4);
 #pragma unroll
               for (int i = 0; i < R / 4; ++i) {
-                if (!MULTI) vr[e][i] = vq[i];
-                p0 = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), av[2 * i], p0);
-                p1 = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), av[2 * i + 1], p1);
+                vr[i] = vq[i];
+                p0 = __ffma2_rn(make_float2(vr[i].x, vr[i].y), av[2 * i], p0);
+                p1 = __ffma2_rn(make_float2(vr[i].z, vr[i].w), av[2 * i + 1], p1);
               }
-              va[e] = (p0.x + p0.y) + (p1.x + p1.y);     // (V a)_q
-            }
-            const float2 va2 = make_float2(va[0], va[1]);
-            const float2 z2 = h ? make_float2(z4.z, z4.w) : make_float2(z4.x, z4.y);
-            const float2 yv = __ffma2_rn(
-                e1_2, z2, __ffma2_rn(c2_2, h ? s23 : s01, __fmul2_rn(c3_2, va2)));
-            const float2 n2 = make_float2(fmaxf(0.f, yv.x), fmaxf(0.f, yv.y));
-            const float2 t2 = __fadd2_rn(z2, va2);
-            const float2 w2 =                                  // beta z' - d'
-                __fmul2_rn(beta2, __ffma2_rn(two2, n2, __fmul2_rn(m1, t2)));
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float w = e ? w2.y : w2.x;
+              auto pick = [&](const float4& f) { return e == 0 ? f.x : e == 1 ? f.y : e == 2 ? f.z : f.w; };
+              const float va = (p0.x + p0.y) + (p1.x + p1.y), z = pick(z4);     // (V a)_q
+              const float s = e == 0 ? s01.x : e == 1 ? s01.y : e == 2 ? s23.x : s23.y;
+              const float n = fmaxf(0.f, fmaf(e1, z, fmaf(c2, s, __fmul_rn(c3, va))));
+              const float t = __fadd_rn(z, va);
+              const float w = __fmul_rn(a.beta, fmaf(2.f, n, -t));              // beta z' - d'
               const float2 ww = make_float2(w, w);
 #pragma unroll
               for (int i = 0; i < R / 4; ++i) {
-                float2* us = MULTI ? ust : uacc;
-                us[2 * i] = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), ww, us[2 * i]);
-                us[2 * i + 1] = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), ww, us[2 * i + 1]);
+                uacc[2 * i] = __ffma2_rn(make_float2(vr[i].x, vr[i].y), ww, uacc[2 * i]);
+                uacc[2 * i + 1] = __ffma2_rn(make_float2(vr[i].z, vr[i].w), ww, uacc[2 * i + 1]);
+              }
+              zn[e] = n;
+              dn[e] = a.beta * (t - n);
+              if (CHECK && in) {
+                const float er = n - (t - pick(dk) * a.inv_beta), ch = n - z;
+                s1 = fmaf(er, er, s1);
+                s2 = fmaf(ch, ch, s2);
+                s3 = fmaf(n, n, s3);
               }
             }
-            zn[2 * h] = n2.x;
-            zn[2 * h + 1] = n2.y;
-            dn[2 * h] = a.beta * (t2.x - n2.x);
-            dn[2 * h + 1] = a.beta * (t2.y - n2.y);
-            if (CHECK && in) {
-              // f^{k+1} = t - d^k / beta
-              const float f0 = t2.x - (h ? dk.z : dk.x) * a.inv_beta;
-              const float f1 = t2.y - (h ? dk.w : dk.y) * a.inv_beta;
-              const float ea = n2.x - f0, eb = n2.y - f1;
-              const float ca = n2.x - z2.x, cb = n2.y - z2.y;
-              s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
-              s2 = fmaf(cb, cb, fmaf(ca, ca, s2));
-              s3 = fmaf(n2.y, n2.y, fmaf(n2.x, n2.x, s3));
+          } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              // two compartments: their products with a, then the z-step and dual step packed
+              float va[2];
+              float4 vr[2][R / 4];
+              if constexpr (MULTI) {
+                const int p = (2 * j + h) % D;
+#pragma unroll
+                for (int i = 0; i < R / 4; ++i) {
+                  vr[0][i] = ahead[p][0][i];
+                  vr[1][i] = ahead[p][1][i];
+                  ahead[p][0][i] = __ldg(vg + i);
+                  ahead[p][1][i] = __ldg(vg + vq1 + i);
+                }
+                vg += 2 * vq1;
+              }
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                float2 p0 = make_float2(0.f, 0.f), p1 = make_float2(0.f, 0.f);
+                const float4* vq = v4 + (4 * j + 2 * h + e) * (R / 4);
+#pragma unroll
+                for (int i = 0; i < R / 4; ++i) {
+                  if (!MULTI) vr[e][i] = vq[i];
+                  p0 = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), av[2 * i], p0);
+                  p1 = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), av[2 * i + 1], p1);
+                }
+                va[e] = (p0.x + p0.y) + (p1.x + p1.y);     // (V a)_q
+              }
+              const float2 va2 = make_float2(va[0], va[1]);
+              const float2 z2 = h ? make_float2(z4.z, z4.w) : make_float2(z4.x, z4.y);
+              const float2 yv = __ffma2_rn(
+                  e1_2, z2, __ffma2_rn(c2_2, h ? s23 : s01, __fmul2_rn(c3_2, va2)));
+              const float2 n2 = make_float2(fmaxf(0.f, yv.x), fmaxf(0.f, yv.y));
+              const float2 t2 = __fadd2_rn(z2, va2);
+              const float2 w2 =                                  // beta z' - d'
+                  __fmul2_rn(beta2, __ffma2_rn(two2, n2, __fmul2_rn(m1, t2)));
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const float w = e ? w2.y : w2.x;
+                const float2 ww = make_float2(w, w);
+#pragma unroll
+                for (int i = 0; i < R / 4; ++i) {
+                  float2* us = MULTI ? ust : uacc;
+                  us[2 * i] = __ffma2_rn(make_float2(vr[e][i].x, vr[e][i].y), ww, us[2 * i]);
+                  us[2 * i + 1] = __ffma2_rn(make_float2(vr[e][i].z, vr[e][i].w), ww, us[2 * i + 1]);
+                }
+              }
+              zn[2 * h] = n2.x;
+              zn[2 * h + 1] = n2.y;
+              dn[2 * h] = a.beta * (t2.x - n2.x);
+              dn[2 * h + 1] = a.beta * (t2.y - n2.y);
+              if (CHECK && in) {
+                // f^{k+1} = t - d^k / beta
+                const float f0 = t2.x - (h ? dk.z : dk.x) * a.inv_beta;
+                const float f1 = t2.y - (h ? dk.w : dk.y) * a.inv_beta;
+                const float ea = n2.x - f0, eb = n2.y - f1;
+                const float ca = n2.x - z2.x, cb = n2.y - z2.y;
+                s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
+                s2 = fmaf(cb, cb, fmaf(ca, ca, s2));
+                s3 = fmaf(n2.y, n2.y, fmaf(n2.x, n2.x, s3));
+              }
             }
           }
           sts4(ob ^ jx, zn[0], zn[1], zn[2], zn[3]);
