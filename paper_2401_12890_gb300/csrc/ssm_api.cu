@@ -734,7 +734,7 @@ ssm_status footprint_impl(const ssm_params& p, bool staging, int waves, int64_t*
       maxparts = t.lr_grid;
     } else {
       t.lr_grid = lowrank_grid(&t);
-      maxparts = lowrank_max_partials(&t);
+      maxparts = t.lr_grid;
     }
     add(4, 2 * lowrank_state_floats(&t, t.lr_grid));  // U[2]
   } else {

@@ -1,5 +1,6 @@
 // The blocked state of the low-rank forms, [chunk][voxel][32 compartments], and its tiles.
 #include <algorithm>
+#include <map>
 
 #include "ssm_internal.cuh"
 
@@ -49,31 +50,83 @@ int grid_axes(const Grid& g) {
   return std::max(1, (g.nx > 1) + (g.ny > 1) + (g.nz > 1 && g.zlink));
 }
 
-// The patch of a grid's tiles: among all bx x by x bz <= 128 with at most max_rows staged
-// rows (halo included; what the kernel's ring has room for), the one with the least tiles x (a tile's fixed work + its staged rows). The
-// weight of the fixed work (300 rows) and the penalty for rows that do not start on
-// multiples of 8 (a quarter warp's 128-bit loads then meet in the same banks) only break
-// near-ties: 16 x 8 (2D) and 8 x 4 x 4 (3D) where the grid divides. An axis without
-// smoothness (one voxel, or the stacking axis of a batch) needs no halo; a single voxel
-// takes one on x (zero-filled rows), so that there is always a neighbour pair to read.
-Patch patch_of(const Grid& g, int max_rows) {
-  Patch best{};
-  double cost = 1e300;
+namespace {
+
+// Extra shared-memory passes of a read of every lane's own row, 16 bytes each: the lanes of a
+// quarter warp whose rows are equal mod 8 meet in the same banks (rows of 64 or 128 bytes in
+// their swizzles)
+int conflicts(int bx, int by, int bz, int hx, int hy, int hz) {
+  const int X = bx + 2 * hx, Y = by + 2 * hy;
+  int extra = 0;
+  for (int q = 0; q < TV; q += 8) {
+    int n[8] = {0}, most = 1;
+    for (int v = q; v < q + 8 && v < bx * by * bz; ++v) {
+      const int lx = v % bx, ly = v / bx % by, lz = v / (bx * by);
+      most = std::max(most, ++n[(((lz + hz) * Y + ly + hy) * X + lx + hx) % 8]);
+    }
+    extra += most - 1;
+  }
+  return extra;
+}
+
+}  // namespace
+
+// The patch of a grid's tiles, among all bx x by x bz <= 128 with at most max_rows staged rows
+// (halo included; what the kernel's ring has room for). First choice: the least tiles x (300 +
+// staged rows + 60 for rows that do not start on multiples of 8): 16 x 8 (2D) and 8 x 4 x 4 (3D)
+// where the grid divides. It knows nothing of the rounds that its tiles take: 56 slices of 39x26
+// would be 560 patches of 8x13, four rounds of 152 CTAs, instead of 504 of 13x9. So another one is
+// taken if it is 3 % better (about the model's error) by
+//     rounds(tiles) (1 + row x staged rows + line x runs of them along x + conflict x extra passes)
+// and few tiles, rounds() the time of the launch layout that so many tiles get, the weights
+// fitted to the times of 370 (grid, patch) pairs (see PatchRule's users). An axis without
+// smoothness (one voxel, or the stacking axis of a batch) needs no halo; a single voxel takes
+// one on x (zero-filled rows), so that there is always a neighbour pair to read.
+Patch patch_of(const Grid& g, const PatchRule& rule) {
   const int hy = g.ny > 1, hz = g.nz > 1 && g.zlink;
   const int hx = g.nx > 1 || (!hy && !hz);
-  for (int bz = 1; bz <= std::min(g.nz, TV); ++bz)
-    for (int by = 1; by <= std::min(g.ny, TV / bz); ++by)
-      for (int bx = 1; bx <= std::min(g.nx, TV / (bz * by)); ++bx) {
-        const int X = bx + 2 * hx, Y = by + 2 * hy, Z = bz + 2 * hz, rows = X * Y * Z;
-        if (rows > max_rows) continue;
-        const int64_t tx = (g.nx + bx - 1) / bx, ty = (g.ny + by - 1) / by, tz = (g.nz + bz - 1) / bz;
-        const double c = (double)tx * ty * tz * (300 + rows + (bx % 8 ? 60 : 0));
-        if (c < cost) {
-          cost = c;
-          best = Patch{bx, by, bz, hx, hy, hz, X, Y, Z, rows, (int)tx, (int)ty, (int)tz,
-                       tx * ty * tz, hx + hy + hz, (rows * 128 + 1023) / 1024 * 1024};
+  auto candidates = [&](auto&& f) {
+    for (int bz = 1; bz <= std::min(g.nz, TV); ++bz)
+      for (int by = 1; by <= std::min(g.ny, TV / bz); ++by)
+        for (int bx = 1; bx <= std::min(g.nx, TV / (bz * by)); ++bx) {
+          const int X = bx + 2 * hx, Y = by + 2 * hy, Z = bz + 2 * hz;
+          if (X * Y * Z > rule.max_rows) continue;
+          const int64_t tx = (g.nx + bx - 1) / bx, ty = (g.ny + by - 1) / by, tz = (g.nz + bz - 1) / bz;
+          f(Patch{bx, by, bz, hx, hy, hz, X, Y, Z, X * Y * Z, (int)tx, (int)ty, (int)tz, tx * ty * tz,
+                  hx + hy + hz, (X * Y * Z * 128 + 1023) / 1024 * 1024});
         }
-      }
+  };
+  int64_t least = INT64_MAX;
+  Patch best{};
+  double cost = 1e300;
+  candidates([&](const Patch& p) {
+    least = std::min(least, p.ntiles);
+    const double c = (double)p.ntiles * (300 + p.rows + (p.bx % 8 ? 60 : 0));
+    if (c < cost) {
+      cost = c;
+      best = p;
+    }
+  });
+  if (!rule.rounds) return best;
+  // (a small grid's segments could take any number of tiles in one round, but every tile costs
+  // a unit's whole work)
+  std::map<int64_t, int64_t> rounds;          // (the candidates share few tile counts)
+  auto time = [&](const Patch& p) {
+    auto r = rounds.find(p.ntiles);
+    if (r == rounds.end()) r = rounds.emplace(p.ntiles, rule.rounds(p.ntiles)).first;
+    return (double)r->second * (1 + 0.3 * ((double)p.ntiles / least - 1)) *
+           (1 + rule.row * p.rows + rule.line * p.Y * p.Z +
+            rule.conflict * conflicts(p.bx, p.by, p.bz, hx, hy, hz));
+  };
+  cost = 0.97 * time(best);
+  candidates([&](const Patch& p) {
+    if (4 * p.ntiles > 5 * least) return;
+    const double c = time(p);
+    if (c < cost) {
+      cost = c;
+      best = p;
+    }
+  });
   return best;
 }
 

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <functional>
 #include <mutex>
 #include <utility>
 #include <string>
@@ -116,8 +117,17 @@ struct Patch {
   int zst;                   // bytes of the z rows, rounded up to 1024
 };
 
+// how a form chooses its patches (patch_of): the staged rows that its ring has room for, the
+// time of its launch layout for a number of tiles, and what a staged row, a run of them along x
+// and an extra pass of a shared-memory read add to a tile's time (no `rounds`: the first choice)
+struct PatchRule {
+  int max_rows;
+  double row, line, conflict;
+  std::function<int64_t(int64_t)> rounds;
+};
+
 int grid_axes(const Grid& g);
-Patch patch_of(const Grid& g, int max_rows);
+Patch patch_of(const Grid& g, const PatchRule& rule);
 
 // One element of the full-rank iteration's z-step (Eq. 31, with D^T D z = s (deg z -
 // sum_nbr z)) and dual step (step 11), given f = h + M w:
@@ -354,7 +364,6 @@ void lowrank_release(ssm_plan_s* pl);
 // sums (and reads d^k), `write_d` stores d^{k+1} for the next iteration's test
 ssm_status lowrank_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, double* partial,
                              int* nparts, cudaStream_t s);
-int lowrank_max_partials(const ssm_plan_s* pl);
 int64_t lowrank_grid(const ssm_plan_s* pl);
 int64_t lowrank_partial_floats(const ssm_plan_s* pl, int64_t grid);
 

@@ -30,9 +30,9 @@
 // leaves as a TMA store.
 //
 // Mapping (persistent). The work units are (segment, tile) pairs, a segment being one of
-// nseg ranges of a tile's stages; they are dealt round-robin in segment-major order to a
-// grid sized to the resident capacity, so the CTAs of one round stream the same compartments
-// of neighbouring tiles and the halos are L2 hits; nseg is chosen by layout(). One producer
+// the ranges that layout() cuts a tile's stages into; they are dealt round-robin in
+// segment-major order to a grid sized to the resident capacity, so the CTAs of one round
+// stream the same compartments of neighbouring tiles and the halos are L2 hits. One producer
 // warp fills a ring of stages. Four consumer warps own one voxel per lane: four
 // compartments at a time they read z and its neighbours with one 128-bit load each, form
 // V a and u' from V rows that every lane reads (broadcasts), and keep u' in registers. At
@@ -81,7 +81,8 @@ struct LowrankArgs {
   int nst;                          // stages per tile: ceil(Q / QS)
   int coff;                         // added to the chunk of the z loads: past the tensor (all
                                     // zeros, nothing read) in an iteration from z = 0
-  int nseg;                         // segments per tile
+  int na, nb_seg;                   // segments (and partial-u slots) of tiles [0, fa), of the rest
+  int fa;
   int nb, nob;                      // ring stages; z' (and d') buffers, 1 or 2
   const float* __restrict__ coefA;  // R (one row per dictionary)
   const float* __restrict__ coefW;  // R (one row per dictionary)
@@ -97,11 +98,11 @@ struct LowrankArgs {
   float beta, inv_beta, xi, lam_s, inv_xb;
 };
 
-// the launch of rank R with `naxes` axes of smoothness; bpsm: resident CTAs per SM wanted
+// the launch of rank R with `naxes` axes of smoothness
 struct LowrankKernel {
   ssm_status (*launch)(const LowrankMaps&, LowrankArgs, bool check, int64_t grid, bool chained,
                        cudaStream_t);
-  int (*blocks_per_sm)(const Patch&);
+  int (*blocks_per_sm)(int rows);
 };
 LowrankKernel lowrank_kernel_small(int R, int naxes);   // R <= 16
 LowrankKernel lowrank_kernel_mid(int R, int naxes);     // 20 .. 32
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
   uint64_t* full = reinterpret_cast<uint64_t*>(obuf + nob * OB);
   uint64_t* empty = full + kMaxNB;
   const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
-  const int nst = a.nst, nseg = a.nseg;
+  const int nst = a.nst;
   if (tid == 0) {
     for (int b = 0; b < nb; ++b) {
       mbar_init(&full[b], 1);
@@ -184,20 +185,44 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
   __syncthreads();
   bool failed = false;
   float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-  // unit k of this CTA: (segment, tile), segment-major, dealt round-robin
+  // (plans with a dictionary per voxel label have one segment count. At R = 8 on 2D grids the
+  // compiler keeps the basis rows' loads ahead of their use only with this 64-bit arithmetic:
+  // 156x156, Q = 900 68 us, else 86. Other ranks are faster with the general one: r = 4 54 -> 46)
+  constexpr bool ONE = MULTI && R == 8 && NAX == 2;
+  // unit k of this CTA: (segment, tile), dealt round-robin: the first tiles' units, then the
+  // others', each segment-major
   auto unit_at = [&](int k, int& tile, int& sg, int& t0, int& t1, int& x0, int& y0,
                      int& z0) -> bool {
-    const int64_t u = blockIdx.x + (int64_t)k * gridDim.x;
-    if (u >= a.p.ntiles * nseg) return false;
-    sg = nseg > 1 ? (int)(u / a.p.ntiles) : 0;
-    tile = (int)(u - sg * a.p.ntiles);
-    t0 = (int)((int64_t)sg * nst / nseg);
-    t1 = (int)((int64_t)(sg + 1) * nst / nseg);
+    if constexpr (ONE) {
+      const int nseg = a.na;
+      const int64_t u = blockIdx.x + (int64_t)k * gridDim.x;
+      if (u >= a.p.ntiles * nseg) return false;
+      sg = nseg > 1 ? (int)(u / a.p.ntiles) : 0;
+      tile = (int)(u - sg * a.p.ntiles);
+      t0 = (int)((int64_t)sg * nst / nseg);
+      t1 = (int)((int64_t)(sg + 1) * nst / nseg);
+    } else {
+      // (32-bit arithmetic: layout() keeps the units below 2^31)
+      const unsigned nf = (unsigned)a.fa * (unsigned)a.na, i = blockIdx.x + (unsigned)k * gridDim.x;
+      const bool f = i < nf;
+      const unsigned u = f ? i : i - nf, ns = f ? a.na : a.nb_seg;
+      const unsigned nt = f ? a.fa : (unsigned)a.p.ntiles - a.fa;
+      if (u >= nt * ns) return false;
+      sg = ns > 1 ? (int)(u / nt) : 0;
+      tile = (int)((f ? 0u : (unsigned)a.fa) + u - (unsigned)sg * nt);
+      t0 = (int)((unsigned)(sg * nst) / ns);
+      t1 = (int)((unsigned)((sg + 1) * nst) / ns);
+    }
     const unsigned t = (unsigned)tile, tx = (unsigned)a.p.tx, ty = (unsigned)a.p.ty;
     x0 = (int)(t % tx) * a.p.bx;
     y0 = (int)(t / tx % ty) * a.p.by;
     z0 = (int)(t / tx / ty) * a.p.bz;
     return true;
+  };
+  // a tile's first slot of partial u
+  auto slot_of = [&](int t) {
+    if constexpr (ONE) return (int64_t)t * a.na;
+    else return (int64_t)(t < a.fa ? t * a.na : a.fa * a.na + (t - a.fa) * a.nb_seg);
   };
   int tile, sg, t0, t1, x0, y0, z0;
   if (warp == NCW) {
@@ -294,8 +319,10 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
 #pragma unroll
         for (int i = 0; i < R; ++i) us[i] = 0.f;
         if (in) {
-          const float* pt = a.Pin + (int64_t)tile * nseg * (R * TV) + v;
-          for (int s = 0; s < nseg; ++s) {
+          const float* pt = a.Pin + slot_of(tile) * (R * TV) + v;
+          int ns = a.na;
+          if constexpr (!ONE) ns = tile < a.fa ? a.na : a.nb_seg;
+          for (int s = 0; s < ns; ++s) {
 #pragma unroll
             for (int i = 0; i < R; ++i) us[i] += pt[(s * R + i) * TV];
           }
@@ -495,7 +522,7 @@ __global__ void __launch_bounds__(NT, min_blocks<R, MULTI>())
         __syncwarp();
       }
       // this segment's partial u' (zero for lanes outside the grid or the object)
-      float* po = a.Pout + ((int64_t)tile * nseg + sg) * (R * TV) + v;
+      float* po = a.Pout + (slot_of(tile) + sg) * (R * TV) + v;
 #pragma unroll
       for (int i = 0; i < R / 2; ++i) {
         po[(2 * i) * TV] = in ? uacc[i].x : 0.f;
@@ -571,15 +598,18 @@ ssm_status launch_r(const LowrankMaps& maps, LowrankArgs args, bool check, int64
                                 chained, maps, args);
 }
 
-// resident CTAs per SM of a plain iteration (also sets the kernels' shared-memory limits)
+// resident CTAs per SM of a plain iteration with patches of `rows` staged rows (also sets the
+// kernels' shared-memory limits)
 template <int R, int NAX, bool MULTI>
-int blocks_per_sm(const Patch& p) {
+int blocks_per_sm(int rows) {
   std::lock_guard<std::mutex> lock(attr_mutex());
   if (allow_smem<R, NAX, true, MULTI>() != cudaSuccess ||
       allow_smem<R, NAX, false, MULTI>() != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
+  Patch p{};
+  p.rows = rows;
   int nb, nob, bytes, b = 0;
   if (!ring<R, MULTI>(p, false, false, &nb, &nob, &bytes)) return 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lowrank_iter_kernel<R, NAX, false, MULTI>, NT, bytes);

@@ -149,7 +149,8 @@ struct LrtcArgs {
                                     // (which may still run: read after pdl_wait)
   float* __restrict__ Pout;         // partial u of this iteration
   int nch;                          // compartment chunks per tile
-  int spc;                          // segments per tile (each a contiguous run of chunks)
+  int full;                         // tiles [0, full) are one unit and one slot each, the others
+  int spc;                          // are spc segments (contiguous runs of chunks) and slots
   int split;                        // > 0: main/tail layout, the chunk where tails start
   int kr;                           // K steps of 8 ranks holding the rank r (<= RP / 8)
   int coff;                         // added to the chunk of the z loads: past the tensor (all
@@ -349,10 +350,10 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   // the k-th unit of this CTA. Main/tail layout (a.split > 0, fewer tiles than CTAs but
   // more than half as many): CTA j < ntiles owns chunks [0, split) of tile j; the other
   // CTAs take the tails [split, nch) of tiles j - ntiles, j - ntiles + (G - ntiles), ...
-  // (concurrent tails are of consecutive tiles too). Otherwise units are dealt
-  // round-robin in segment-major order, so that the CTAs running together hold the same
-  // chunks of consecutive tiles.
-  // (32-bit arithmetic: with several segments per tile there are fewer tiles than CTAs)
+  // (concurrent tails are of consecutive tiles too). Otherwise units are dealt round-robin,
+  // the whole tiles first, then the segments of the others in segment-major order, so that the
+  // CTAs running together hold the same chunks of consecutive tiles.
+  // (32-bit division: only fewer tiles than CTAs are split into segments)
   auto unit_at = [&](int k, int& tile, int& c0, int& c1, int& sg) -> bool {
     const unsigned nt = (unsigned)a.p.ntiles, G = gridDim.x, j = blockIdx.x;
     if (a.split > 0) {
@@ -373,13 +374,23 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
       return true;
     }
     const int64_t u = j + (int64_t)k * G;
-    if (u >= a.p.ntiles * spc) return false;
-    sg = spc > 1 ? (int)((unsigned)u / nt) : 0;
-    tile = (int)((unsigned)u - (unsigned)sg * nt);
-    c0 = spc > 1 ? sg * nch / spc : 0;
-    c1 = spc > 1 ? (sg + 1) * nch / spc : nch;
+    if (u < a.full) {
+      tile = (int)u;
+      sg = 0;
+      c0 = 0;
+      c1 = nch;
+      return true;
+    }
+    const unsigned rest = nt - (unsigned)a.full, v = (unsigned)(u - a.full);
+    if (u - a.full >= (int64_t)rest * spc) return false;
+    sg = (int)(v / rest);
+    tile = a.full + (int)(v - (unsigned)sg * rest);
+    c0 = sg * nch / spc;
+    c1 = (sg + 1) * nch / spc;
     return true;
   };
+  // a tile's first slot of partial u
+  auto slot_of = [&](int t) { return t < a.full ? (int64_t)t : a.full + (int64_t)(t - a.full) * spc; };
   // first voxel of a tile
   auto origin = [&](int tile, int& x0, int& y0, int& z0) {
     const unsigned t = (unsigned)tile, tx = (unsigned)a.p.tx, ty = (unsigned)a.p.ty;
@@ -605,7 +616,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           deg += (z > 0 && (!mk || mk[n - plane])) + (z < nz - 1 && (!mk || mk[n + plane]));
       }
       e1 = (a.xi + a.beta - a.lam_s * (float)deg) * a.inv_xb;   // weight of z
-      const float* pt = a.Pin + (int64_t)tile * spc * (RP * TV) + grp * RQ * TV + v;
+      const float* pt = a.Pin + slot_of(tile) * (RP * TV) + grp * RQ * TV + v;
       const float* sp = a.S + (int64_t)(grp * RQ) * ld + n;
 #pragma unroll
       for (int i = 0; i < RQ; ++i) sv[i] = in ? __ldg(sp + i * ld) : 0.f;
@@ -619,7 +630,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
           origin(t1, x1, y1, z1);
           const int64_t n1 = min(x1 + lx, nx - 1) +
                              (int64_t)nx * (min(y1 + ly, ny - 1) + (int64_t)ny * min(z1 + lz, nz - 1));
-          const float* p1 = a.Pin + ((int64_t)t1 * spc * RP + grp * RQ) * TV + v;
+          const float* p1 = a.Pin + (slot_of(t1) * RP + grp * RQ) * TV + v;
           const float* s1p = a.S + (int64_t)(grp * RQ) * ld + n1;
 #pragma unroll 4
           for (int i = 0; i < RQ; ++i) {
@@ -631,7 +642,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
       // (SB slots' loads in flight together; a slot past the last reads the last with weight 0)
       constexpr int SB = RQ <= 16 ? 3 : 1;
 #pragma unroll 1
-      for (int s = 1; s < spc; s += SB) {
+      for (int s = 1; tile >= a.full && s < spc; s += SB) {
         float u1[SB][RQ];
 #pragma unroll
         for (int t = 0; t < SB; ++t)
@@ -846,7 +857,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
         ++own;
       }
       // the next unit's loads go out before this one's last sums are waited for
-      float* po = a.Pout + ((int64_t)tile * spc + sg) * (RP * TV) + v;
+      float* po = a.Pout + (slot_of(tile) + sg) * (RP * TV) + v;
       const bool in0 = in;
       const int gl = g + nchk - 1;                   // the unit's last chunk
       more = begin(k + 1);
@@ -936,13 +947,6 @@ __global__ void split_basis_kernel(const float* __restrict__ V32, int Q, int RP,
   }
 }
 
-// what a plan of this form keeps: the tiles, and the tensor maps of both ping-pong halves
-struct LrtcState {
-  Patch p;
-  LrtcMaps maps[2];
-  int spc = 1, split = 0;   // launch layout (the grid is the plan's lr_grid)
-};
-
 template <int RP, int NAX, bool CHECK, bool WD>
 ssm_status set_attr() {
   return cudaFuncSetAttribute(lrtc_kernel<RP, NAX, CHECK, WD>,
@@ -1019,20 +1023,12 @@ ssm_status launch_rn(const LrtcMaps& maps, const LrtcArgs& args, bool check, boo
   return launch_one<RP, NAX, false, false>(maps, args, grid, chained, s);
 }
 
-Patch tiles_of(const ssm_plan_s* pl) {
-  const int axes = grid_axes(pl->g);
-  if (pl->R == 64) return patch_of(pl->g, max_rows<64, 2>());
-  return patch_of(pl->g, axes == 3 ? max_rows<32, 3>() : max_rows<32, 2>());
-}
-int64_t ntiles_of(const ssm_plan_s* pl) {
-  if (pl->lr_state) return static_cast<const LrtcState*>(pl->lr_state)->p.ntiles;
-  return tiles_of(pl).ntiles;
-}
 int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 
 // Launch layout: the CTAs' budget G0 (one per SM per launch wave).
-//  - At least G0 tiles: every tile is one unit (its whole Q range) and the grid is the
-//    fewest CTAs that keep the rounds of G tiles equal.
+//  - At least G0 tiles: whole tiles (one unit each, its whole Q range), the grid the fewest CTAs
+//    that keep the rounds of G tiles equal. Where the last round has few tiles, these are split
+//    into spc segments each instead, which all G0 CTAs take.
 //  - Between G0/2 and G0 tiles (the 128x128 slice: 128 tiles, 152 SMs): one segment per
 //    tile would leave G0 - ntiles SMs idle, two would give some CTAs two whole-Q-halves
 //    of work; instead CTA j < ntiles takes chunks [0, split) of tile j and the spare
@@ -1043,26 +1039,32 @@ int64_t chunks_of(const ssm_plan_s* pl) { return (pl->Q + QC - 1) / QC; }
 //    without; 177x74, 38 iterations 849, 571).
 //  - Fewer tiles: each tile is split into spc equal segments so that all CTAs have work.
 // chunks a unit's start (a-vector, filling the pipeline) takes as long as. On 128x128, Q = 2500
-// (79 chunks) 6 gives split = 72: 75 us per iteration; split 70 78, 74 75, 76 77
-constexpr int kStart = 6;
-void layout(const ssm_plan_s* pl, int64_t* grid, int* spc, int* split) {
-  const int64_t ntiles = ntiles_of(pl), nch = chunks_of(pl);
-  int64_t g0 = (int64_t)sm_count() * std::max(1, pl->waves);
-  if (const char* env = getenv("SSM_LRTC_GRID")) {   // launch-shape override for sweeps
-    const long v = atol(env);
-    if (v >= 1 && v <= 65536) g0 = v;
-  }
-  int64_t force_split = -1;
-  if (const char* env = getenv("SSM_LRTC_SPLIT")) {  // 0: no main/tail layout (sweeps)
-    const long v = atol(env);
-    if (v >= 0 && v < nch) force_split = v;
-  }
-  *split = 0;
+// (79 chunks) 6 gives split = 72: 75 us per iteration; split 70 78, 74 75, 76 77. Twice the
+// ranks take twice as long (128x100, Q = 400, r = 64: 26.1 us with 6, 24.9 with 12)
+constexpr int start_chunks(int R) { return R == 64 ? 12 : 6; }
+struct Layout {
+  int64_t cost, grid;        // (cost: chunks, starts included, one after another)
+  int full, spc, split;
+};
+// `wanted`: the chunk where tails start (sweeps), 0 no tails, -1 by the rule
+Layout layout(int64_t ntiles, int64_t nch, int64_t g0, int kStart, int64_t wanted) {
+  const int64_t whole = nch + kStart;
   if (ntiles >= g0) {
-    const int64_t rounds = (ntiles + g0 - 1) / g0;
-    *spc = 1;
-    *grid = (ntiles + rounds - 1) / rounds;
-  } else if (2 * ntiles > g0 && nch >= 4 && force_split != 0) {
+    const int64_t base = ntiles / g0, rest = ntiles % g0;
+    int64_t best = 1, cost = rest > 0 ? whole : 0;    // of the last round
+    for (int64_t c = 2; rest > 0 && c <= nch; ++c) {
+      const int64_t t = (rest * c + g0 - 1) / g0 * ((nch + c - 1) / c + kStart);
+      if (t < cost) {
+        cost = t;
+        best = c;
+      }
+    }
+    cost += base * whole;
+    if (best > 1) return Layout{cost, g0, (int)(base * g0), (int)best, 0};
+    const int64_t rounds = base + (rest > 0);
+    return Layout{cost, (ntiles + rounds - 1) / rounds, (int)ntiles, 1, 0};
+  }
+  if (2 * ntiles > g0 && nch >= 4 && wanted != 0) {
     const int64_t spare = g0 - ntiles;
     const int64_t per = (ntiles + spare - 1) / spare;   // tails per spare CTA
     int64_t best = 1, cost = INT64_MAX;
@@ -1073,19 +1075,54 @@ void layout(const ssm_plan_s* pl, int64_t* grid, int* spc, int* split) {
         best = c;
       }
     }
-    if (force_split > 0) best = force_split;
-    if (force_split < 0 && cost >= nch + kStart) {
-      *spc = 1;
-      *grid = ntiles;
-      return;
-    }
-    *split = (int)best;
-    *spc = 2;
-    *grid = ntiles + (ntiles + per - 1) / per;
-  } else {
-    *spc = (int)std::max<int64_t>(1, std::min(nch, g0 / ntiles));
-    *grid = ntiles * *spc;
+    if (wanted > 0) best = wanted;
+    if (wanted < 0 && cost >= whole) return Layout{whole, ntiles, (int)ntiles, 1, 0};
+    return Layout{cost, ntiles + (ntiles + per - 1) / per, 0, 2, (int)best};
   }
+  const int64_t spc = std::max<int64_t>(1, std::min(nch, g0 / ntiles));
+  return Layout{(nch + spc - 1) / spc + kStart, ntiles * spc, 0, (int)spc, 0};
+}
+Layout layout(const ssm_plan_s* pl, int64_t ntiles) {
+  const int64_t nch = chunks_of(pl);
+  int64_t g0 = (int64_t)sm_count() * std::max(1, pl->waves), wanted = -1;
+  if (const char* env = getenv("SSM_LRTC_GRID")) {   // launch-shape override for sweeps
+    const long v = atol(env);
+    if (v >= 1 && v <= 65536) g0 = v;
+  }
+  if (const char* env = getenv("SSM_LRTC_SPLIT")) {
+    const long v = atol(env);
+    if (v >= 0 && v < nch) wanted = v;
+  }
+  return layout(ntiles, nch, g0, start_chunks(pl->R), wanted);
+}
+
+// The plan's tiles. A staged row adds 0.1 % to a tile's time, a run of them along x 0.5 % and an
+// extra pass of the quarter warps' reads 1.1 %; on 3D grids 0.3, 0 and 2.7 %. (Fitted over 13
+// grids and stacks, to 4 %; the patches so chosen are within 1.2 % of the best on average)
+Patch tiles_of(const ssm_plan_s* pl) {
+  const bool cube = grid_axes(pl->g) == 3;
+  const int rows = pl->R == 64 ? max_rows<64, 2>() : cube ? max_rows<32, 3>() : max_rows<32, 2>();
+  return patch_of(pl->g, PatchRule{rows, cube ? 3e-3 : 1.1e-3, cube ? 0.0 : 5e-3,
+                                   cube ? 2.7e-2 : 1.06e-2,
+                                   [=](int64_t nt) { return layout(pl, nt).cost; }});
+}
+
+// what a plan of this form keeps: its tiles and launch layout, and the tensor maps of both
+// ping-pong halves
+struct LrtcState {
+  Patch p;
+  Layout l;
+  LrtcMaps maps[2];
+  // units, and slots of partial u: one per unit
+  int64_t units() const { return l.full + (p.ntiles - l.full) * l.spc; }
+};
+
+LrtcState shape_of(const ssm_plan_s* pl) {
+  if (pl->lr_state) return *static_cast<const LrtcState*>(pl->lr_state);
+  LrtcState st{};
+  st.p = tiles_of(pl);
+  st.l = layout(pl, st.p.ntiles);
+  return st;
 }
 
 }  // namespace
@@ -1097,19 +1134,11 @@ int lrtc_padded_rank(int r, bool three_d) {
   return 0;
 }
 
-int64_t lrtc_grid(const ssm_plan_s* pl) {
-  int64_t grid;
-  int spc, split;
-  layout(pl, &grid, &spc, &split);
-  return grid;
-}
+int64_t lrtc_grid(const ssm_plan_s* pl) { return shape_of(pl).l.grid; }
 
 int64_t lrtc_partial_floats(const ssm_plan_s* pl, int64_t grid) {
   (void)grid;
-  int64_t g;
-  int spc, split;
-  layout(pl, &g, &spc, &split);
-  return ntiles_of(pl) * spc * (int64_t)pl->R * TV;
+  return shape_of(pl).units() * (int64_t)pl->R * TV;
 }
 
 // the kernels' shared-memory limits, and the plan's tiles and tensor maps (the state
@@ -1123,10 +1152,9 @@ ssm_status lrtc_prepare(ssm_plan_s* pl) {
     SSM_TRY((prepare_rn<64, 1>()));
     SSM_TRY((prepare_rn<64, 2>()));
   }
-  auto* st = new LrtcState();
+  auto* st = new LrtcState(shape_of(pl));
   pl->lr_state = st;
-  st->p = tiles_of(pl);
-  layout(pl, &pl->lr_grid, &st->spc, &st->split);
+  pl->lr_grid = st->l.grid;
   const Patch& p = st->p;
   const uint64_t Q = (uint64_t)pl->Q, RP = (uint64_t)pl->R, Qs = (uint64_t)pl->lrtc_qs;
   const auto SW = CU_TENSOR_MAP_SWIZZLE_128B;
@@ -1174,8 +1202,9 @@ ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, dou
   a.Pin = pl->U[cur];
   a.Pout = pl->U[cur ^ 1];
   a.nch = (int)chunks_of(pl);
-  a.spc = st.spc;
-  a.split = st.split;
+  a.full = st.l.full;
+  a.spc = st.l.spc;
+  a.split = st.l.split;
   a.kr = std::max(1, std::min(pl->R / 8, (pl->r + 7) / 8));
   a.nsz = a.nob = 0;                 // set per variant (launch_one)
   a.coff = pl->from_zero ? a.nch : 0;
@@ -1198,7 +1227,7 @@ ssm_status lrtc_iteration(ssm_plan_s* pl, int cur, bool check, bool write_d, dou
   // iteration start as the last one's leave, out of step with the tiles next to them, whose
   // halo rows they then find in L2 less often: with 31 units per CTA (96x96x64) 1877 ->
   // 1979 us. With few units per CTA the gap weighs more (256x256, 3.4 units: 273 -> 269)
-  const bool chained = pl->chained && st.p.ntiles * st.spc <= 8 * grid;
+  const bool chained = pl->chained && st.units() <= 8 * grid;
   if (pl->R == 32) {
     if (st.p.naxes == 1) return launch_rn<32, 1>(m, a, check, write_d, grid, chained, s);
     if (st.p.naxes == 2) return launch_rn<32, 2>(m, a, check, write_d, grid, chained, s);
