@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
   using L = Lay<RP, NAX>;
   constexpr int UB = L::UB, NSV = L::NSV;
   constexpr int RQ = RP / NG;         // ranks of a per epilogue group
+  constexpr int UC = RP == 64 ? 8 : 16;   // columns of u' read at once (registers)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // aligned by an offset from the shared array itself (not through an integer), so that
   // the compiler keeps the shared address space of every pointer derived from it
@@ -695,16 +696,16 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
         fence_after();
         const uint32_t ub = tmem + lane_base + L::T_U + 2 * RP * (gg % UB);
 #pragma unroll
-        for (int j0 = 0; j0 < RP; j0 += 16) {
-          uint32_t um[32];
-          tld<16>(ub + j0, um);
-          tld<16>(ub + RP + j0, um + 16);
-          tld_wait<32>(um);
+        for (int j0 = 0; j0 < RP; j0 += UC) {
+          uint32_t um[2 * UC];
+          tld<UC>(ub + j0, um);
+          tld<UC>(ub + RP + j0, um + UC);
+          tld_wait<2 * UC>(um);
 #pragma unroll
-          for (int j = 0; j < 16; j += 2) {
+          for (int j = 0; j < UC; j += 2) {
             const float2 t2 = __fadd2_rn(
                 make_float2(__uint_as_float(um[j]), __uint_as_float(um[j + 1])),
-                make_float2(__uint_as_float(um[16 + j]), __uint_as_float(um[17 + j])));
+                make_float2(__uint_as_float(um[UC + j]), __uint_as_float(um[UC + 1 + j])));
             const float2 s2 = __fadd2_rn(make_float2(uacc[j0 + j], uacc[j0 + j + 1]), t2);
             uacc[j0 + j] = s2.x;
             uacc[j0 + j + 1] = s2.y;
@@ -757,63 +758,67 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
             tld<8>(tb + 8 * (sb + 1), vr);
             tld<8>(tb + 32 + 8 * (sb + 1), vr + 8);
           }
-          float4 zz[2], nb[2 * NAX][2];
+          // (with 64 ranks 4 at a time, which leaves registers for the running u')
+          constexpr int HB = RP == 64 ? 1 : 2;
+          float4 zz[2], nb[2 * NAX][2], dk[2];
+          float zn[8], w[8], dn[8];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
-            zz[h] = lds4(za[0] ^ jx);
+          for (int h0 = 0; h0 < 2; h0 += HB) {
 #pragma unroll
-            for (int q = 0; q < 2 * NAX; ++q) nb[q][h] = lds4(za[1 + q] ^ jx);
-          }
-          float zn[8], w[8];
-          float4 dk[2];
-          if constexpr (CHECK) {
+            for (int h = h0; h < h0 + HB; ++h) {
+              const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
+              zz[h] = lds4(za[0] ^ jx);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) dk[h] = lds4((db + dro) ^ ((uint32_t)(2 * sb + h) << 4));
-          }
-          float dn[8];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int h = j >> 1;
-            auto pr = [&](const float4& f) {
-              return (j & 1) ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
-            };
-            const float2 z2 = pr(zz[h]);
-            float2 s = __fadd2_rn(pr(nb[0][h]), pr(nb[1][h]));
-#pragma unroll
-            for (int q = 2; q < 2 * NAX; ++q) s = __fadd2_rn(s, pr(nb[q][h]));
-            const float2 y = __ffma2_rn(e1_2, z2, __ffma2_rn(c2_2, s, __fmul2_rn(c3_2, va2[j])));
-            const float2 n2 = make_float2(fmaxf(0.f, y.x), fmaxf(0.f, y.y));
-            const float2 mt = __ffma2_rn(m1, z2, va2[j]);                       // -t
-            const float2 w2 = __fmul2_rn(beta2, __ffma2_rn(two2, n2, mt));
-            zn[2 * j] = n2.x;
-            zn[2 * j + 1] = n2.y;
-            w[2 * j] = w2.x;
-            w[2 * j + 1] = w2.y;
-            if constexpr (WD) {
-              dn[2 * j] = -beta * (mt.x + n2.x);
-              dn[2 * j + 1] = -beta * (mt.y + n2.y);
+              for (int q = 0; q < 2 * NAX; ++q) nb[q][h] = lds4(za[1 + q] ^ jx);
             }
             if constexpr (CHECK) {
-              // f^{k+1} = t - d^k / beta
-              const float2 d2 = pr(dk[h]);
-              const float f0 = -(mt.x + d2.x * a.inv_beta), f1 = -(mt.y + d2.y * a.inv_beta);
-              const float ea = n2.x - f0, eb = n2.y - f1;
-              const float ca = n2.x - z2.x, cb = n2.y - z2.y;
-              s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
-              s2 = fmaf(cb, cb, fmaf(ca, ca, s2));
-              s3 = fmaf(n2.y, n2.y, fmaf(n2.x, n2.x, s3));
-            }
-          }
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
-            sts4(ob ^ jx, zn[4 * h], zn[4 * h + 1], zn[4 * h + 2], zn[4 * h + 3]);
-            if constexpr (OWN_D)
-              sts4((ob + OUT_BYTES) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2], dn[4 * h + 3]);
-            else if constexpr (WD)
-              sts4((ring + sz * zst + a.p.zst + vrow) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2],
-                   dn[4 * h + 3]);
+              for (int h = h0; h < h0 + HB; ++h)
+                dk[h] = lds4((db + dro) ^ ((uint32_t)(2 * sb + h) << 4));
+            }
+#pragma unroll
+            for (int j = 2 * h0; j < 2 * (h0 + HB); ++j) {
+              const int h = j >> 1;
+              auto pr = [&](const float4& f) {
+                return (j & 1) ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
+              };
+              const float2 z2 = pr(zz[h]);
+              float2 s = __fadd2_rn(pr(nb[0][h]), pr(nb[1][h]));
+#pragma unroll
+              for (int q = 2; q < 2 * NAX; ++q) s = __fadd2_rn(s, pr(nb[q][h]));
+              const float2 y = __ffma2_rn(e1_2, z2, __ffma2_rn(c2_2, s, __fmul2_rn(c3_2, va2[j])));
+              const float2 n2 = make_float2(fmaxf(0.f, y.x), fmaxf(0.f, y.y));
+              const float2 mt = __ffma2_rn(m1, z2, va2[j]);                       // -t
+              const float2 w2 = __fmul2_rn(beta2, __ffma2_rn(two2, n2, mt));
+              zn[2 * j] = n2.x;
+              zn[2 * j + 1] = n2.y;
+              w[2 * j] = w2.x;
+              w[2 * j + 1] = w2.y;
+              if constexpr (WD) {
+                dn[2 * j] = -beta * (mt.x + n2.x);
+                dn[2 * j + 1] = -beta * (mt.y + n2.y);
+              }
+              if constexpr (CHECK) {
+                // f^{k+1} = t - d^k / beta
+                const float2 d2 = pr(dk[h]);
+                const float f0 = -(mt.x + d2.x * a.inv_beta), f1 = -(mt.y + d2.y * a.inv_beta);
+                const float ea = n2.x - f0, eb = n2.y - f1;
+                const float ca = n2.x - z2.x, cb = n2.y - z2.y;
+                s1 = fmaf(eb, eb, fmaf(ea, ea, s1));
+                s2 = fmaf(cb, cb, fmaf(ca, ca, s2));
+                s3 = fmaf(n2.y, n2.y, fmaf(n2.x, n2.x, s3));
+              }
+            }
+#pragma unroll
+            for (int h = h0; h < h0 + HB; ++h) {
+              const uint32_t jx = (uint32_t)(2 * sb + h) << 4;
+              sts4(ob ^ jx, zn[4 * h], zn[4 * h + 1], zn[4 * h + 2], zn[4 * h + 3]);
+              if constexpr (OWN_D)
+                sts4((ob + OUT_BYTES) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2], dn[4 * h + 3]);
+              else if constexpr (WD)
+                sts4((ring + sz * zst + a.p.zst + vrow) ^ jx, dn[4 * h], dn[4 * h + 1], dn[4 * h + 2],
+                     dn[4 * h + 3]);
+            }
           }
           float wh[8], wl[8];
 #pragma unroll
@@ -856,11 +861,12 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
         __syncwarp();
         ++own;
       }
-      // the next unit's loads go out before this one's last sums are waited for
+      // the next unit's loads go out before this one's last sums are waited for (64 ranks: after
+      // the sums are stored, as their registers hold both only by spilling 450 bytes per thread)
       float* po = a.Pout + (slot_of(tile) + sg) * (RP * TV) + v;
       const bool in0 = in;
       const int gl = g + nchk - 1;                   // the unit's last chunk
-      more = begin(k + 1);
+      if (RP == 32) more = begin(k + 1);
       if (pend >= 0) consume_u(pend);
       // the unit's partial u': the second group hands its sums over in the TMEM slot of its
       // last chunk (read by product 2, and not written by product 1 before both groups have
@@ -893,6 +899,7 @@ __global__ void __launch_bounds__(NT, 1) lrtc_kernel(const __grid_constant__ Lrt
 #pragma unroll
         for (int i = 0; i < RP; ++i) po[i * TV] = in0 ? uacc[i] : 0.f;
       }
+      if (RP == 64) more = begin(k + 1);
       g += nchk;
       ++si;
     }
