@@ -14,6 +14,9 @@ per dictionary before the timed region; its time is reported as plan_ms.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
+prints one JSON line on stdout (the headline) and the whole record, with every form, workload
+and serving class, as one line on stderr.
+
 Under torchrun each rank solves its own independent problem (a different seed) with
 no collective on the data path: weak scaling, value = all ranks' work / max time.
 """
@@ -317,6 +320,24 @@ def dominant_kernel(form, prec, Q, N, r, fused=0):
     return ("tc_gemm_kernel", "ssm_tc.cu", "tensor", 3 * 2.0 * Q * Q * N, "TFLOP/s", key)
 
 
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "clocks",
+             "e2e", "gpu_launches", "roofline", "cpu_baseline")
+
+
+def result_line(out):
+    """The result line: the headline's keys of the record `out`, and in a few numbers what its
+    larger sections say. Short (below 2 KB), so that a reader that keeps the end of the output
+    has all of it."""
+    line = {k: out[k] for k in LINE_KEYS}
+    if out["cpu_baseline"]:
+        line["cpu_baseline"] = {k: v for k, v in out["cpu_baseline"].items() if k != "sample"}
+    rule = out["time_to_tol_ms"]["residual_rule"]
+    line["time_to_tol_ms"] = {k: rule[k] for k in ("tol", "p50", "p99", "iterations") if k in rule}
+    line["err_vs_oracle"] = {k: v["rel_fro"] for k, v in (out["err_vs_oracle"] or {}).items()}
+    return line
+
+
 # --------------------------------------------------------------------------------------
 # our arm
 # --------------------------------------------------------------------------------------
@@ -573,7 +594,10 @@ def bench_ours(args):
             "serving": serving,
             "batching": batching,
         }
-        print(json.dumps(out), flush=True)
+        # the whole record (every form, workload and serving class: about 22 KB) on stderr, the
+        # result line on stdout
+        print("bench record: " + json.dumps(out), file=sys.stderr, flush=True)
+        print(json.dumps(result_line(out)), flush=True)
     dist.close()
 
 

@@ -52,13 +52,12 @@ __global__ void __launch_bounds__(UV) dense_update_kernel(UpdateArgs a) {
     y = (int)(t % ny);
     zc = (int)(t / ny);
   }
-  const int64_t sy_ = nx, sz_ = (int64_t)nx * ny;
   const bool hxm = valid && x > 0 && (!mk || mk[n - 1]);
   const bool hxp = valid && x < nx - 1 && (!mk || mk[n + 1]);
-  const bool hym = valid && y > 0 && (!mk || mk[n - sy_]);
-  const bool hyp = valid && y < ny - 1 && (!mk || mk[n + sy_]);
-  const bool hzm = a.g.zlink && valid && zc > 0 && (!mk || mk[n - sz_]);
-  const bool hzp = a.g.zlink && valid && zc < nz - 1 && (!mk || mk[n + sz_]);
+  const bool hym = valid && y > 0 && (!mk || mk[n - sy]);
+  const bool hyp = valid && y < ny - 1 && (!mk || mk[n + sy]);
+  const bool hzm = a.g.zlink && valid && zc > 0 && (!mk || mk[n - sz]);
+  const bool hzp = a.g.zlink && valid && zc < nz - 1 && (!mk || mk[n + sz]);
   const float deg = (float)(hxm + hxp + hym + hyp + hzm + hzp);
   float s1 = 0.f, s2 = 0.f, s3 = 0.f;
   const int q0 = blockIdx.y * UQ, q1 = min(a.Q, q0 + UQ);
@@ -260,15 +259,10 @@ __global__ void __launch_bounds__(RT) roughness_kernel(const float* __restrict__
 // FMAs of a warp against the 12 of 8 x 8 outputs per thread, whose reads queued behind one
 // another. Slices of 8 k come by cp.async into a ring of NST stages, and the fragments of
 // slice entry k + 1 are read while those of k are multiplied. Tiles of 64 rows x 128 columns
-// (4 warps, three CTAs per SM): CTAs that wait for their own slices only, and a shorter last
-// wave. Against tiles of 128 rows (8 warps, two CTAs): M = K = 2500, N = 16384 4704 -> 4605 us
-// per iteration with the update, M = K = 1600, N = 589824 71.1 -> 67.2 ms, M = K = 900,
-// N = 36864 1700 -> 1525 us, M = K = 300, N = 6048 53.7 -> 47.9 us; the objective with M = 64,
-// K = 1600, N = 589824 6851 -> 4011 us (half of a 128-row tile is padding there), with M = 1000,
-// K = 900, N = 36864 1722 -> 1579 us. Against 128 x 128 tiles with the next slice held in
-// registers: M = K = 300, N = 6048 57.5 us, M = K = 225, N = 1024 43.4 us (now 24.9), M = K =
-// 2500, N = 16384 4858 us, M = 120, K = 2500, N = 16384 (the objective's product) 313 -> 278
-// us in ncu
+// (4 warps, three CTAs per SM): CTAs that wait for their own slices only, and a short last
+// wave. Per iteration with the update: M = K = 2500, N = 16384 4605 us (tiles of 128 rows and
+// two CTAs: 4704), M = K = 300, N = 6048 47.9 us (53.7). The objective with M = 64, K = 1600,
+// N = 589824 4011 us (6851: half of a 128-row tile is padding there).
 // VEC: the rows of A^T and B are 16-byte aligned (else scalar copies)
 constexpr int PM = 64;
 

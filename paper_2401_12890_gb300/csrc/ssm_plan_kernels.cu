@@ -3,8 +3,8 @@
 // the full-rank inverse of Eq. 26, and the operand of the data projections (step 4,
 // ssm_exact.cu).
 //
-// All of this runs once per plan and is FP64 where the paper's conditioning needs it. GB300's FP64 rate is low, so the
-// kernels spread FP64 work over every SM rather than one CTA.
+// All of this runs once per plan and is FP64 where the paper's conditioning needs it. GB300's
+// FP64 rate is low, so the kernels spread FP64 work over every SM rather than one CTA.
 #include <algorithm>
 #include <cmath>
 #include <numeric>
